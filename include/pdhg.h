@@ -302,7 +302,10 @@ pdhg_status pdhg_get_kernel_timing_parts(pdhg_ctx* ctx, double* ms, int64_t* sam
  * and writes the attempt's x beside it, the dual also forms A~ times the
  * move and applies the acceptance test, followed by the kernel that undoes a
  * rejected attempt (timed with the dual).  Launches are back to back as in a solve
- * (programmatic dependent launch), with no event between them.  The solver
+ * (programmatic dependent launch), with no event between them.  A context
+ * whose LP is solved on chip (constant step, tile_nnz = 0, spmv_layout = 0,
+ * kernel_timing = 0, vectors that fit in a cluster's shared memory) has no
+ * half-step kernels of its own: the tile kernels are timed.  The solver
  * state is saved to a temporary device buffer first and restored after, so
  * a solve continues as if the call had not happened.  Single-LP contexts.  */
 pdhg_status pdhg_time_kernels(pdhg_ctx* ctx, int32_t reps, double* ms);

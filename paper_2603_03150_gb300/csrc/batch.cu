@@ -226,7 +226,7 @@ __device__ __forceinline__ void beval_body(const BatchBuffers<T>& B, int chunk, 
     for (int t = B.lp_a_tiles[l]; t < B.lp_a_tiles[l + 1]; ++t)
 #pragma unroll
       for (int k = 0; k < kEvalQ; ++k) tot[k] += __ldcg(B.rec_a + (size_t)t * kEvalQ + k);
-    apply_eval_rule(sc, tot, chunk, nullptr, nullptr, nullptr);
+    apply_eval_rule(sc, tot, chunk, eval_roots(sc, tot), nullptr, nullptr, nullptr);
     if (!sc.done) ++mine;
   }
   atomicAdd(&active, mine);
@@ -1109,7 +1109,7 @@ static pdhg_status tune_batch_schedules(pdhg_ctx* ctx) {
     const int nrows = on_a ? ctx->m : ctx->n;
     const int64_t* off = on_a ? ctx->h_m_off.data() : ctx->h_n_off.data();
     std::vector<int> cands = {kFixedE};
-    if (ctx->opt.autotune) cands = {8, 16, 32};  // vector variants: never faster (measured)
+    if (ctx->opt.autotune && !ctx->resident) cands = {8, 16, 32};  // vector variants: never faster (measured)
     DevSched best = on_a ? ctx->sa8 : ctx->st8;
     int32_t* best_lp = on_a ? ctx->lp_a8_tiles : ctx->lp_t8_tiles;
     float best_ms = 1e30f;
@@ -1317,8 +1317,12 @@ static pdhg_status batch_create_impl(pdhg_ctx* ctx, const int32_t* m, const int3
 
   // per-LP scalar state
   CKS(batch_fresh_scalars(ctx));
+  CKS(resident_build(ctx));
+  stage("on-chip layout");
   // a3 per LP: power iteration
-  {
+  if (ctx->resident) {
+    CKS(resident_power(ctx));
+  } else {
     double *v = ctx->xs64, *u = ctx->ys64, *w = ctx->out_n2;
     int32_t* ticket = ctx->active + 2;
     k_bpow_init<<<(count + 255) / 256, 256, 0, ctx->stream>>>(ctx->ps, count,
@@ -1526,7 +1530,20 @@ extern "C" pdhg_status pdhg_batch_solve(pdhg_ctx* ctx, double eps_rel, int64_t m
     }
     k = max_iter;  // the kernel ran to the end (or until every LP finished)
   }
-  if (!ctx->opt.persistent && ctx->opt.use_graphs) CKS(build_batch_graphs(ctx));
+  if (ctx->resident && k < max_iter) {
+    const pdhg_status rs = ctx->mixed ? resident_solve<float>(ctx, batch_buffers<float>(ctx).it)
+                                      : resident_solve<double>(ctx, batch_buffers<double>(ctx).it);
+    CKS(rs);
+    if (rs == PDHG_TIMEOUT) {
+      ctx->last_status = rs;
+      ctx->report_valid = false;
+      if (lp_status)
+        for (int l = 0; l < count; ++l) lp_status[l] = rs;
+      return rs;
+    }
+    k = max_iter;  // every LP has ended
+  }
+  if (!ctx->opt.persistent && ctx->opt.use_graphs && !ctx->resident) CKS(build_batch_graphs(ctx));
   const long long F = ctx->opt.eval_freq;
   // pinned status words (the context's pinned status buffers are large enough)
   int32_t* h_ctl[2] = {reinterpret_cast<int32_t*>(ctx->h_sc[0]),

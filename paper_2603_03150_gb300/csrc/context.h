@@ -150,6 +150,7 @@ struct pdhg_ctx {
   void* gsync = nullptr;                      // grid-barrier state of the persistent batched solve
   double* breport = nullptr;                  // [count][8] per-LP report
   void* adjoint = nullptr;                    // active-set polish / adjoint buffers
+  void* resident = nullptr;                   // layout of LPs solved on chip (NULL: tile kernels)
   // schedules and launch shapes
   DevSched sa, st;      // iteration schedules (autotuned nonzeros per thread)
   DevSched sa8, st8;    // float64 report / Algorithm 1 / power iteration
@@ -232,5 +233,14 @@ pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out);
 // batched solve from iteration k0 to max_iter in one cooperative launch
 // (PDHG_TIMEOUT if a grid barrier's bounded wait ran out)
 pdhg_status batch_persistent_solve(pdhg_ctx* ctx, long long k0, long long max_iter);
+
+// LPs solved on chip (resident.cu).  resident_build sets ctx->resident where
+// every LP fits (needs A~ and its transpose scaled); then resident_power fills
+// ctx->ps and resident_solve runs every LP from its stored state to its end.
+pdhg_status resident_build(pdhg_ctx* ctx);
+void resident_free(pdhg_ctx* ctx);
+pdhg_status resident_power(pdhg_ctx* ctx);
+template <typename T>
+pdhg_status resident_solve(pdhg_ctx* ctx, const IterBuffers<T>& B);
 
 }  // namespace pdhg

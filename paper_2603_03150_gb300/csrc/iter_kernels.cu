@@ -149,9 +149,11 @@ __global__ void __launch_bounds__(BLOCK, sizeof(T) == 4 ? 4 : 1) k_eval(IterBuff
   if (!is_last) return;
   __threadfence();
   parts_sum<BLOCK, kEvalQ>(B.partials, (int)gridDim.x, B.split_q, B.t_sched.ngroups, tot, red);
+  if (threadIdx.x >= 32) return;
+  const EvalRoots R = eval_roots_warp(*B.sc, tot);
   if (threadIdx.x == 0) {
     B.sc->ticket = 0;
-    apply_eval_rule(*B.sc, tot, chunk, B.log_k, B.log_flags, B.log_kkt);
+    apply_eval_rule(*B.sc, tot, chunk, R, B.log_k, B.log_flags, B.log_kkt);
   }
 }
 

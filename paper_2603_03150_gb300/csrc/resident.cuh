@@ -1,0 +1,416 @@
+// On-chip LPs: one thread-block cluster holds an LP's iterate in shared memory
+// for a whole solve (the layout, its build and the device helpers shared by
+// the solve, the power iteration and the conjugate gradients).
+//
+// Layout.  Each matrix of an LP (A~ and A~^T) is stored in slices of one warp:
+// the rows are sorted by length (longest first, stable, so the order is
+// fixed), rows of up to kResShort nonzeros go 32 to a slice (a lane each),
+// rows of up to kResMid 4 to a slice (8 lanes each), longer ones one to a
+// slice.  Step k of a slice is 32 consecutive values and 16-bit columns, so
+// the loads coalesce and a row costs one fused multiply-add per nonzero and,
+// for the longer classes, the shuffle sum: GB300 runs 2 float64 operations per
+// clock and SM, so the segmented scan of the CSR tiles (5 float64 additions
+// for 8 nonzeros) is what this layout leaves out.  Columns are positions in
+// the sorted order of the other matrix, in which the vectors are kept too.
+// Entries past a row's end have value 0 and the column of a slot that holds 0.
+//
+// Slice s belongs to CTA s mod C of the cluster and warp (s / C) mod kResWarps
+// of it: always the same lane works on a row, so the row's own operands need
+// no barrier.  Every CTA holds the whole gathered vectors; a new entry is
+// written to all C copies through distributed shared memory, and one cluster
+// barrier separates the half-steps.
+#pragma once
+#include "common.cuh"
+#include "kernels.h"
+
+namespace pdhg {
+
+constexpr int kResThreads = 512, kResWarps = kResThreads / 32;
+constexpr int kResShort = 24;   // a lane per row up to this many nonzeros
+constexpr int kResMid = 256;    // 8 lanes per row up to this many, a warp above
+constexpr int kResMaxC = 16;    // CTAs of a cluster (16 needs the non-portable size)
+// What is solved on chip, and by how many CTAs (us per iteration, one LP, GB300;
+// tile kernels: 10 at 200 x 500, 11.4 at 2000 x 5000):
+//   float64, clusters of 1 / 4 / 16: 60 x 150 2.4 / 2.6 / 2.7, 200 x 500 3.4 /
+//   2.5 / 2.7, 2000 x 5000 23.7 / 7.1 / 3.7; float32: 1.1 / 1.3 / 1.5, 1.4 / 1.4
+//   / 1.5, 9.8 / 3.1 / 2.3.
+// So a CTA gets at least kResMinOps operations of an iteration (an exchange
+// between CTAs costs about 250 clocks).  Above kResMaxNnz nonzeros 16 CTAs do
+// not outrun the whole chip's tile kernels, and a row longer than kResMaxRow
+// would be a chain of more than 128 steps in one warp.
+constexpr int64_t kResMaxNnz = 320000;
+constexpr int kResMaxRow = 4096;
+constexpr double kResMinOps64 = 3000.0, kResMinOps32 = 6000.0;
+
+struct ResSlice {
+  int32_t off;  // first element of the slice, relative to the LP's matrix
+  int32_t p0;   // position of its first row
+  int32_t loc;  // slot of its first row among its CTA's own rows
+  int32_t wgr;  // steps | log2(lanes per row) << 16 | rows << 20
+};
+__host__ __device__ constexpr int res_steps(int wgr) { return wgr & 0xffff; }
+__host__ __device__ constexpr int res_lg(int wgr) { return (wgr >> 16) & 15; }
+__host__ __device__ constexpr int res_rows(int wgr) { return wgr >> 20; }
+
+struct ResLp {
+  int32_t m, n;
+  int64_t m_off, n_off;  // its first row / column in the stacked arrays (and first slice)
+  int64_t a_el, t_el;    // first element of its slices of A~ / A~^T
+  int32_t C;             // CTAs of its cluster
+  int32_t a_slices, t_slices;
+  int32_t own_m, own_n;  // slots of a CTA's own rows and columns (bounds)
+};
+
+// Slots of one CTA's own rows of a matrix of `rows` rows: a class of slices
+// dealt to C CTAs gives a CTA at most one slice above the mean.
+__host__ __device__ inline int res_own(int rows, int C) { return rows / C + 73; }
+
+// Dynamic shared memory of a cluster's CTA.  own_n / own_m: T vectors of the
+// CTA's own columns / rows (nvn, nvm of them); X and Y the gathered copies.
+struct ResSmem {
+  uint32_t sc, rec, red, tab, bar, X, Y, own_n, own_m, total;
+};
+__host__ __device__ inline ResSmem res_smem(int m, int n, int own_m, int own_n, int nvm, int nvn,
+                                            int es) {
+  ResSmem r;
+  uint32_t o = 0;
+  auto take = [&](uint32_t bytes) {
+    const uint32_t at = o;
+    o = (o + bytes + 15u) & ~15u;
+    return at;
+  };
+  r.sc = take(sizeof(Scalars));
+  r.rec = take(kResMaxC * 18 * 8);   // one record per CTA: 16 sums, 1 flag
+  r.red = take(16 * kResWarps * 8);
+  r.tab = take(64 * 8);              // averaging weights of 64 iterations
+  r.bar = take(16);                  // transaction barriers of X and Y
+  r.X = take((uint32_t)(((m > n ? m : n) + 1) * es));
+  r.Y = take((uint32_t)((m + 1) * es));
+  r.own_n = take((uint32_t)(own_n * nvn * es));
+  r.own_m = take((uint32_t)(own_m * nvm * es));
+  r.total = o;
+  return r;
+}
+
+// max(0, v) and min(0, v) of doubles with integer tests (fmax / fmin would
+// take the float64 pipe); NaN gives 0 as fmax(0, NaN) does.
+__device__ __forceinline__ double max0(double v) {
+  return (unsigned long long)__double_as_longlong(v) > 0x7ff0000000000000ull ? 0.0 : v;
+}
+__device__ __forceinline__ float max0(float v) { return fmaxf(0.f, v); }
+__device__ __forceinline__ double min0(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull ? v : 0.0;
+}
+
+// A cluster of C CTAs, one of its CTAs (rank) with its shared memory window.
+template <int C>
+struct ResCluster {
+  uint32_t base;  // this CTA's dynamic shared memory
+  int rank;
+  __device__ __forceinline__ ResCluster(void* smem) {
+    base = (uint32_t)__cvta_generic_to_shared(smem);
+    rank = 0;
+    if constexpr (C > 1) {
+      uint32_t r;
+      asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+      rank = (int)r;
+    }
+  }
+  // offset `off` of rank q's dynamic shared memory
+  __device__ __forceinline__ uint32_t at(int q, uint32_t off) const {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(base + off), "r"(q));
+    return a;
+  }
+  // all threads of all CTAs; what was pushed before is visible after
+  __device__ __forceinline__ void sync() const {
+    if constexpr (C == 1) {
+      __syncthreads();
+    } else {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+  }
+  // v to offset off on every CTA, visible after the next sync()
+  __device__ __forceinline__ void push(uint32_t off, double v) const {
+    if constexpr (C == 1)
+      asm volatile("st.shared.f64 [%0], %1;" ::"r"(base + off), "d"(v) : "memory");
+    else
+#pragma unroll 2
+      for (int q = 0; q < C; ++q)
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at(q, off)), "d"(v) : "memory");
+  }
+  __device__ __forceinline__ void push(uint32_t off, float v) const {
+    if constexpr (C == 1)
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + off), "f"(v) : "memory");
+    else
+#pragma unroll 2
+      for (int q = 0; q < C; ++q)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(at(q, off)), "f"(v) : "memory");
+  }
+  // v to offset off on every CTA, counted by the transaction barrier at offset
+  // bar of each: a CTA that has seen a whole vector arrive knows that every
+  // row of the half-step has been computed, so no other barrier is needed
+  // (C = 1: plain stores, the caller meets sync())
+  __device__ __forceinline__ void send(uint32_t off, uint32_t bar, double v) const {
+    if constexpr (C == 1) {
+      push(off, v);
+    } else {
+#pragma unroll 4
+      for (int q = 0; q < C; ++q)
+        asm volatile(
+            "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(at(q, off)),
+            "l"(__double_as_longlong(v)), "r"(at(q, bar))
+            : "memory");
+    }
+  }
+  __device__ __forceinline__ void send(uint32_t off, uint32_t bar, float v) const {
+    if constexpr (C == 1) {
+      push(off, v);
+    } else {
+#pragma unroll 4
+      for (int q = 0; q < C; ++q)
+        asm volatile(
+            "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(at(q, off)),
+            "r"(__float_as_int(v)), "r"(at(q, bar))
+            : "memory");
+    }
+  }
+  // waits until the vector counted by barrier `bar` has arrived (phase parity)
+  // and lets thread 0 expect the next one; false (for the whole warp) once a
+  // lane's wait ran past limit_ns
+  __device__ __forceinline__ bool arrived(uint32_t bar, uint32_t parity, uint32_t bytes,
+                                          unsigned long long limit_ns) const {
+    const uint32_t mb = base + bar;
+    unsigned long long t0 = 0;
+    uint32_t done = 0;
+    for (uint32_t n = 0; !done; ++n) {
+      asm volatile(
+          "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; "
+          "selp.u32 %0, 1, 0, p; }"
+          : "=r"(done)
+          : "r"(mb), "r"(parity)
+          : "memory");
+      if ((n & 255u) == 255u) {
+        if (t0 == 0) t0 = global_ns();
+        else if (global_ns() - t0 > limit_ns) break;
+      }
+    }
+    const bool ok = __all_sync(0xffffffffu, done != 0);
+    if (threadIdx.x == 0 && ok) mbar_arrive_expect(mb, bytes);
+    return ok;
+  }
+};
+
+// acc += (or -=) sum of val * buf[col] over one slice: lane l gets the sums of
+// the row l >> lg (every lane of the row the same).  Steps go by fours, the
+// next four's loads in flight while four are gathered and added; the last
+// w mod 4 are loaded first and added last, in a loop of their own: a float64
+// operation whose predicate is off still takes its slot of the float64 pipe
+// (16 clocks of an SM), so no operation here is predicated.  Slices of
+// kResWide steps and more use two accumulators: the chain of dependent float64
+// operations (68 clocks each) is what a lone warp waits for, and the extra
+// addition is a small part of so long a row.
+constexpr int kResWide = 12;
+template <bool kNegate, typename TV>
+__device__ __forceinline__ TV res_fma(TV a, TV x, TV acc) {
+  return kNegate ? fmadd(-a, x, acc) : fmadd(a, x, acc);
+}
+template <int NB, bool kNegate, typename TV, typename TX>
+__device__ __forceinline__ void res_dot(const ResSlice& s, const TV* __restrict__ val,
+                                        const uint16_t* __restrict__ col, const TX* const (&buf)[NB],
+                                        TV (&acc)[NB]) {
+  const int lane = threadIdx.x & 31, w = res_steps(s.wgr), lg = res_lg(s.wgr);
+  const TV* v = val + s.off + lane;
+  const uint16_t* c = col + s.off + lane;
+  const int full = w & ~3;
+  TV a[4], ta[3];
+  int j[4], tj[3];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    a[e] = TV(0);
+    j[e] = 0;
+    if (full) {
+      a[e] = __ldg(v + e * 32);
+      j[e] = __ldg(c + e * 32);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    ta[e] = TV(0);
+    tj[e] = 0;
+    if (full + e < w) {
+      ta[e] = __ldg(v + (full + e) * 32);
+      tj[e] = __ldg(c + (full + e) * 32);
+    }
+  }
+  // four steps: the values and columns in a, j; f adds value * entry to step e's sum
+  auto four = [&](int k, auto&& f) {
+    TV g[NB][4], ca[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      ca[e] = a[e];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) g[b][e] = (TV)buf[b][j[e]];
+    }
+    if (k + 4 < full) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        a[e] = __ldg(v + (k + 4 + e) * 32);
+        j[e] = __ldg(c + (k + 4 + e) * 32);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+      for (int b = 0; b < NB; ++b) f(e, b, ca[e], g[b][e]);
+  };
+  if (w >= kResWide) {
+    TV acc2[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc2[b] = TV(0);
+#pragma unroll 1
+    for (int k = 0; k < full; k += 4)
+      four(k, [&](int e, int b, TV x, TV y) {
+        if (e & 1) acc2[b] = res_fma<kNegate>(x, y, acc2[b]);
+        else acc[b] = res_fma<kNegate>(x, y, acc[b]);
+      });
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc[b] += acc2[b];
+  } else {
+#pragma unroll 1
+    for (int k = 0; k < full; k += 4)
+      four(k, [&](int, int b, TV x, TV y) { acc[b] = res_fma<kNegate>(x, y, acc[b]); });
+  }
+#pragma unroll 1
+  for (int e = full; e < w; ++e) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc[b] = res_fma<kNegate>(ta[0], (TV)buf[b][tj[0]], acc[b]);
+    ta[0] = ta[1], tj[0] = tj[1];
+    ta[1] = ta[2], tj[1] = tj[2];
+  }
+  if (lg) {  // warp-uniform
+#pragma unroll 1
+    for (int o = 1 << (lg - 1); o > 0; o >>= 1)
+#pragma unroll
+      for (int b = 0; b < NB; ++b) acc[b] += __shfl_xor_sync(0xffffffffu, acc[b], o);
+  }
+}
+
+// One matrix of an LP as a CTA sees it; f(slice, row of this lane or -1) for
+// the CTA's slices of this warp (row -1: a lane without a row of its own).
+// The first slice's descriptor stays in registers, the next one's is loaded
+// ahead.
+struct ResMat {
+  const ResSlice* sl;
+  const uint16_t* col;
+  int slices, s0;
+  int4 first;
+  __device__ __forceinline__ ResMat(const ResSlice* sl_, const uint16_t* col_, int n, int rank, int C)
+      : sl(sl_), col(col_), slices(n), s0(rank + (int)(threadIdx.x >> 5) * C) {
+    first = s0 < n ? __ldg(reinterpret_cast<const int4*>(sl + s0)) : make_int4(0, 0, 0, 0);
+  }
+  template <int C, class F>
+  __device__ __forceinline__ void each(F&& f) const {
+    const int lane = threadIdx.x & 31;
+    int4 q = first;
+    for (int s = s0; s < slices; s += kResWarps * C) {
+      const ResSlice d{q.x, q.y, q.z, q.w};
+      if (s + kResWarps * C < slices) q = __ldg(reinterpret_cast<const int4*>(sl + s + kResWarps * C));
+      const int lg = res_lg(d.wgr), row = lane >> lg;
+      f(d, (lane & ((1 << lg) - 1)) == 0 && row < res_rows(d.wgr) ? row : -1);
+    }
+  }
+};
+
+// Sums of NQ quantities over the cluster, the same bits on every CTA: the
+// block's sums to every CTA's record of this rank, a cluster barrier, then the
+// records in rank order into out[0..NQ) (shared).  `flag` (thread 0's) of rank
+// 0 is returned to every thread.  Ends with a block barrier; the caller meets
+// a cluster barrier before the next call.
+template <int NQ, int C>
+__device__ __forceinline__ bool res_reduce(const ResCluster<C>& cl, const ResSmem& L,
+                                           unsigned char* smem, double (&v)[NQ], double* out,
+                                           bool flag = false) {
+  double* rec = reinterpret_cast<double*>(smem + L.rec);
+  double* red = reinterpret_cast<double*>(smem + L.red);
+  block_sum_scatter<kResThreads, NQ>(v, red, out);
+  if (threadIdx.x < NQ) cl.push(L.rec + (uint32_t)(cl.rank * 18 + threadIdx.x) * 8u, out[threadIdx.x]);
+  if (threadIdx.x == 0) cl.push(L.rec + (uint32_t)(cl.rank * 18 + 16) * 8u, flag ? 1.0 : 0.0);
+  cl.sync();
+  if (threadIdx.x < NQ) {
+    double t = rec[threadIdx.x];
+#pragma unroll
+    for (int r = 1; r < C; ++r) t += rec[r * 18 + threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+  const bool f = rec[16] != 0.0;
+  __syncthreads();
+  return f;
+}
+
+#define RES_DISPATCH_C(c, ...)  \
+  switch (c) {                  \
+    case 1: {                   \
+      constexpr int C_ = 1;     \
+      __VA_ARGS__;              \
+    } break;                    \
+    case 2: {                   \
+      constexpr int C_ = 2;     \
+      __VA_ARGS__;              \
+    } break;                    \
+    case 4: {                   \
+      constexpr int C_ = 4;     \
+      __VA_ARGS__;              \
+    } break;                    \
+    case 8: {                   \
+      constexpr int C_ = 8;     \
+      __VA_ARGS__;              \
+    } break;                    \
+    default: {                  \
+      constexpr int C_ = 16;    \
+      __VA_ARGS__;              \
+    } break;                    \
+  }
+
+inline cudaLaunchConfig_t res_config(int C, int lps, size_t smem, cudaStream_t s,
+                                     cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(lps * C);
+  cfg.blockDim = dim3(kResThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = C;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// ---------------------------------------------------------------------------
+// the solve (resident_solve.cuh)
+// ---------------------------------------------------------------------------
+template <typename T>
+struct ResSolve {
+  const ResLp* lp;
+  const int32_t* list;  // LPs of this launch, one per cluster
+  const ResSlice *a_sl, *t_sl;
+  const uint16_t *a_col, *t_col, *ord_m, *ord_n;
+  const T *a_val, *t_val;
+  const double *a_val64, *t_val64;
+  IterBuffers<T> B;       // the state in natural order
+  int32_t* active;        // LPs not finished
+  unsigned long long slice_ns;
+  unsigned long long wait_ns;  // bound of a wait for another CTA's vector
+  int32_t* err;                // 1 once such a wait ran out
+};
+
+template <typename T>
+const void* res_solve_kernel(int C, bool halpern);
+template <typename T>
+cudaError_t launch_res_solve(const ResSolve<T>& A, int C, int lps, size_t smem, bool halpern,
+                             cudaStream_t s);
+
+}  // namespace pdhg

@@ -497,7 +497,8 @@ static pdhg_status tune_schedules(pdhg_ctx* ctx) {
       cands.push_back({longest <= 256 ? (tn <= -8 ? -8 : -4) : 8, 0});
     else if (tn > 0)
       cands.push_back({tn <= 2044 ? 8 : (tn <= 4092 ? 16 : 32), tn});
-    else if (ctx->opt.autotune && (int64_t)rp[nrows] >= (int64_t)kLongWindowRows * nrows) {
+    else if (ctx->opt.autotune && !ctx->resident &&
+             (int64_t)rp[nrows] >= (int64_t)kLongWindowRows * nrows) {
       // the vector variants were slower than E = 8 on every measured matrix
       // since the window words; they stay available through tile_nnz < 0.
       // E = 16 and 32 are tried only where rows average kLongWindowRows
@@ -944,9 +945,12 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
   CKS(fixed_schedules(ctx));
   stage("float64 schedules");
 
+  CKS(resident_build(ctx));
+  stage("on-chip layout");
+
   // the tuner's E = 16 and E = 32 schedules are host work: build them on a
   // host thread while the GPU runs the power iteration
-  if (ctx->opt.autotune && ctx->opt.tile_nnz == 0) {
+  if (ctx->opt.autotune && ctx->opt.tile_nnz == 0 && !ctx->resident) {
     for (int which = 0; which < 2; ++which)
       for (int q = 0; q < 2; ++q) {
         const int32_t* rp = which == 0 ? ctx->h_a_rp.data() : ctx->h_t_rp.data();
@@ -960,7 +964,9 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
   }
 
   // a3: power iteration on A~^T A~ (float64)
-  {
+  if (ctx->resident) {
+    CKS(resident_power(ctx));
+  } else {
     double *v = ctx->xs64, *u = ctx->ys64, *w = ctx->out_n2;
     launch_pow_init(n, v, ctx->ps, ctx->opt.power_max_iter, ctx->opt.power_rel_tol, ctx->stream);
     ctx->launches += 1;
@@ -1115,6 +1121,7 @@ extern "C" void pdhg_destroy(pdhg_ctx* ctx) {
       if (ctx->ev_k[g][e]) cudaEventDestroy(ctx->ev_k[g][e]);
   }
   pdhg_free_adjoint(ctx);
+  resident_free(ctx);
   for (void* p : ctx->allocs) cudaFree(p);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
@@ -1158,7 +1165,17 @@ extern "C" pdhg_status pdhg_solve(pdhg_ctx* ctx, double eps_rel, int64_t max_ite
   hs.checks = 0;
   hs.rejects = 0;
   CK(cudaMemcpyAsync(ctx->sc, &hs, sizeof(hs), cudaMemcpyHostToDevice, ctx->stream));
-  if (ctx->opt.use_graphs) CKS(build_graphs(ctx));
+  if (ctx->resident) {
+    const pdhg_status rs = ctx->mixed ? resident_solve<float>(ctx, iter_buffers<float>(ctx))
+                                      : resident_solve<double>(ctx, iter_buffers<double>(ctx));
+    CKS(rs);
+    if (rs == PDHG_TIMEOUT) {
+      ctx->last_status = rs;
+      return rs;
+    }
+    k = max_iter;  // every chunk has run
+  }
+  if (ctx->opt.use_graphs && !ctx->resident) CKS(build_graphs(ctx));
   for (double& v : ctx->timing_sum) v = 0.0;
   ctx->timing_n = 0;
 

@@ -1,0 +1,131 @@
+"""LPs solved on chip (a thread-block cluster per LP) against the oracle and
+against the tile kernels, at the edges of the layout: rows of 0, 1, 24, 25,
+256, 257 and 4096 nonzeros (the three row classes and their limit), last
+slices of 1 and 32 rows, more rows than columns, clusters of 1 to 16.
+
+Tolerances as in the other parity tests: float64 states 1e-9 relative in the
+infinity norm (the sums run in another order, about 1e-15 per product, over
+200 iterations of a nonexpansive map); float32-mixed states 1e-4."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+from oracle import pdhg_oracle as O
+from paper_2603_03150_gb300 import build as B
+from paper_2603_03150_gb300 import lpgen
+from paper_2603_03150_gb300 import pdhg
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ["x", "y", "x_avg", "y_avg", "x_last", "y_last", "Ax", "Ax_avg", "Ax_last"]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    B.build()
+
+
+def rel_inf(a, b):
+    a, b = np.asarray(a, float), np.asarray(b, float)
+    return float(np.max(np.abs(a - b)) / max(1e-300, np.max(np.abs(b))))
+
+
+def rows_lp(lengths, n, seed):
+    """One row per entry of `lengths`, planted optimum."""
+    rng = np.random.default_rng(seed)
+    cols = [np.sort(rng.choice(n, size=k, replace=False)) for k in lengths]
+    ptr = np.concatenate([[0], np.cumsum([c.size for c in cols])])
+    val = rng.standard_normal(int(ptr[-1]))
+    A = sp.csr_matrix((val, np.concatenate(cols).astype(int) if cols else [], ptr), shape=(len(lengths), n))
+    x = rng.uniform(0.5, 2, n) * (rng.random(n) < 0.3)
+    z = np.where(x > 0, 0.0, rng.uniform(0.5, 2, n))
+    b, c = A @ x, A.T @ rng.standard_normal(len(lengths)) + z
+    return lpgen.LP(len(lengths), n, A.indptr.astype(np.int32), A.indices.astype(np.int32), A.data, b, c)
+
+
+MAKERS = {
+    "tiny": lambda: lpgen.planted_lp(3, 7, nnz_per_col=2, seed=0),
+    "short_edge": lambda: rows_lp([24] * 33 + [25] * 5 + [0, 1, 0], 64, 1),
+    "mid_edge": lambda: rows_lp([256] * 3 + [257] * 2 + [3] * 40, 300, 2),
+    "longest": lambda: rows_lp([4096, 4095, 31] + [4] * 61, 5000, 3),
+    "tall": lambda: rows_lp(list(range(1, 90)) + [2] * 700, 97, 4),
+    "planted": lambda: lpgen.planted_lp(331, 829, seed=5),
+    "wide_cluster": lambda: lpgen.planted_lp(2311, 5777, seed=6),
+    "transport": lambda: lpgen.transportation_lp(31, 44),
+}
+
+
+def run(lp, iters, **kw):
+    with pdhg.Solver.from_lp(lp, **kw) as s:
+        before = s.launch_count()
+        assert s.solve(0.0, iters) == pdhg.PDHG_MAX_ITER
+        return s.state(), s.log(), s.launch_count() - before
+
+
+@pytest.mark.parametrize("name", list(MAKERS))
+def test_float64_iterates_match_oracle(name):
+    lp = MAKERS[name]()
+    st, lg, launches = run(lp, 100)
+    assert launches < 10  # one launch, not one per half-step
+    r = O.solve(lp, 0.0, 100)
+    for k in KEYS[:6]:
+        assert rel_inf(st[k], getattr(r.state, k)) < 1e-9, k
+    assert [(e["k"], e["restart"], e["cand"]) for e in lg] == \
+           [(e["k"], e["restart"], e["cand"]) for e in r.log]
+
+
+@pytest.mark.parametrize("method,rule", [("averaged", "smooth"), ("halpern", "pid")])
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 1e-4)])
+@pytest.mark.parametrize("name", list(MAKERS))
+def test_states_match_the_tile_kernels(name, precision, tol, method, rule):
+    """200 iterations: an odd last chunk, three evaluations, restarts; the tile
+    kernels are asked for by a forced tile capacity."""
+    lp = MAKERS[name]()
+    kw = dict(precision=precision, method=method, omega_rule=rule)
+    a, la, n_a = run(lp, 200, **kw)
+    b, lb, n_b = run(lp, 200, tile_nnz=2044, **kw)
+    assert n_a < 10 < n_b
+    # the two candidates of an LP that float32 has already solved to its last
+    # digit ("tall" at 192) differ by rounding alone: decisions are float64's
+    if precision == "fp64":
+        assert [(e["k"], e["restart"], e["cand"]) for e in la] == \
+               [(e["k"], e["restart"], e["cand"]) for e in lb]
+    for k in KEYS:
+        assert rel_inf(a[k], b[k]) < tol, k
+
+
+def test_rows_past_the_limit_take_the_tile_kernels():
+    lp = rows_lp([4097] + [3] * 50, 5000, 7)
+    st, _, launches = run(lp, 64)
+    assert launches > 64
+    assert rel_inf(st["x"], O.solve(lp, 0.0, 64).state.x) < 1e-9
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 1e-4)])
+def test_batch_of_every_cluster_size(precision, tol):
+    """LPs from 3 x 7 to 2300 x 5750 in one batch: each LP its own cluster size,
+    several launches side by side; resumed from a stop between evaluations."""
+    lps = [lpgen.planted_lp(3, 7, nnz_per_col=2, seed=0), MAKERS["tall"](), MAKERS["mid_edge"](), lpgen.planted_lp(2300, 5750, seed=1)]
+    lps += [lpgen.planted_lp(m, int(2.5 * m), seed=m) for m in (40, 150, 400, 900)]
+    out = []
+    for persistent in (0, 1):  # the persistent form runs on the tile kernels
+        with pdhg.BatchSolver(lps, precision=precision, persistent=persistent) as s:
+            s.solve(0.0, 100)
+            s.solve(0.0, 200)
+            out.append(s.get())
+    a, b = out
+    assert np.array_equal(a["iters"], b["iters"])
+    assert rel_inf(a["x"], b["x"]) < tol and rel_inf(a["y"], b["y"]) < tol
+
+
+def test_a_stop_between_evaluations_changes_nothing():
+    lp = MAKERS["planted"]()
+    with pdhg.Solver.from_lp(lp) as s:
+        s.solve(0.0, 192)
+        ref = s.state()
+    with pdhg.Solver.from_lp(lp) as s:
+        for k in (1, 37, 100, 192):
+            s.solve(0.0, k)
+        got = s.state()
+    for k in KEYS:
+        np.testing.assert_array_equal(got[k], ref[k], err_msg=k)
