@@ -182,7 +182,8 @@ pdhg_status pdhg_create(pdhg_ctx** out, int32_t m, int32_t n, const int32_t* row
  * widened to float64, A~x~ and A~^T y~ recomputed from the float64 scaled
  * matrices), so a converged float32-mixed solve meets the test at eps_rel
  * exactly as pdhg_get reports it.  If a column-panel SpMV's bounded wait for
- * its bulk copy ran out (options.wait_limit_ms), the call returns
+ * its bulk copy, or an on-chip solve's for another CTA's part of a vector, ran
+ * out (options.wait_limit_ms), the call returns
  * PDHG_TIMEOUT and pdhg_last_error says so; the iterate is then not
  * meaningful, the context stays usable.  */
 pdhg_status pdhg_solve(pdhg_ctx* ctx, double eps_rel, int64_t max_iter);

@@ -11,8 +11,13 @@ namespace pdhg {
 // One cluster per LP, from its stored state until it has finished or slice_ns
 // has passed (the state is stored exactly, so where a launch ends changes
 // nothing).  Bound by the float64 pipe in float64 (2 operations per clock and
-// SM), by shared-memory gathers and the two cluster barriers of an iteration
-// in float32.
+// SM: 512 LPs of 50..5000 rows to 1e-4 in 38.5 ms against 126 ms of the tile
+// kernels' launches, about 0.9 of that pipe while every SM has an LP), by the
+// latency of one pass over a slice and of two exchanges per iteration where an
+// LP has the chip to itself (2000 x 5000 float64 3.7 us per iteration against
+// 11.4, 97 LPs float32-mixed 192 iterations in 1.9 ms against 4.8).  512 threads
+// of up to 128 registers: two CTAs per SM at 64 registers spilled and were 5 to
+// 30% slower.
 template <typename T, int C, bool hal>
 __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
   extern __shared__ __align__(16) unsigned char smem[];
