@@ -303,6 +303,7 @@ struct AdjointData {
   double *mask = nullptr, *w = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *rhs = nullptr,
          *u = nullptr, *rec = nullptr, *xpol = nullptr;
   CgState* cg = nullptr;
+  ResCgData* chip = nullptr;  // the active set's on-chip layout
   bool polished = false;
 };
 
@@ -313,6 +314,7 @@ void pdhg_adjoint_invalidate(pdhg_ctx* ctx) {
 }
 
 void pdhg_free_adjoint(pdhg_ctx* ctx) {
+  if (ctx->adjoint) resident_cg_free(adj_of(ctx)->chip);
   delete adj_of(ctx);
   ctx->adjoint = nullptr;
 }
@@ -336,6 +338,10 @@ static pdhg_status adj_alloc(pdhg_ctx* ctx) {
   CKS(dalloc(ctx, &d->u, m));
   CKS(dalloc(ctx, &d->rec, 2 * (size_t)std::max(ctx->st8.view.ntiles, 1) + 2));
   CKS(dalloc(ctx, &d->cg, (size_t)ctx->count));
+  if (ctx->resident && !(d->chip = resident_cg_new())) {
+    set_error("out of host memory");
+    return PDHG_OOM;
+  }
   for (const void* f : {(const void*)k_adj_mask<kBlock>, (const void*)k_cg_Av<kBlock>,
                         (const void*)k_cg_ATu<kBlock>, (const void*)k_adj_spmv<kBlock>}) {
     CK(set_dyn_adj(f, ctx->smem_optin));
@@ -429,14 +435,19 @@ extern "C" pdhg_status pdhg_batch_polish(pdhg_ctx* ctx, double cg_tol, int32_t c
   CK(cudaMemcpyAsync(lpt.data(), ctx->lp_t8_tiles, sizeof(int32_t) * (count + 1),
                      cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  if (lp_active)
-    for (int l = 0; l < count; ++l) {
-      double s = 0.0;
-      for (int t = lpt[l]; t < lpt[l + 1]; ++t) s += cnt[t];
-      lp_active[l] = (int32_t)s;
-    }
+  std::vector<int32_t> act((size_t)count);
+  for (int l = 0; l < count; ++l) {
+    double s = 0.0;
+    for (int t = lpt[l]; t < lpt[l + 1]; ++t) s += cnt[t];
+    act[l] = (int32_t)s;
+    if (lp_active) lp_active[l] = act[l];
+  }
   std::vector<int32_t> iters;
-  CKS(run_cg(ctx, d, cg_tol, cg_max_iter, &iters, ctx->a_val64, ctx->t_val64));
+  if (d->chip) CKS(resident_cg_layout(ctx, d->chip, d->mask, act.data()));
+  if (resident_cg_ready(d->chip))
+    CKS(resident_cg(ctx, d->chip, false, d->rhs, d->w, cg_tol, cg_max_iter, &iters));
+  else
+    CKS(run_cg(ctx, d, cg_tol, cg_max_iter, &iters, ctx->a_val64, ctx->t_val64));
   if (lp_cg_iters)
     for (int l = 0; l < count; ++l) lp_cg_iters[l] = iters[l];
   // x = D_c x~ (zero off B)
@@ -475,7 +486,10 @@ extern "C" pdhg_status pdhg_batch_adjoint(pdhg_ctx* ctx, const double* grad_x, d
   k_adj_vec<<<eg, 256, 0, ctx->stream>>>(T, 3, nullptr, nullptr, nullptr, d->w);
   ctx->launches += 2;
   std::vector<int32_t> iters;
-  CKS(run_cg(ctx, d, cg_tol, cg_max_iter, &iters, ctx->a_val_orig, ctx->t_val_orig));
+  if (resident_cg_ready(d->chip))
+    CKS(resident_cg(ctx, d->chip, true, d->rhs, d->w, cg_tol, cg_max_iter, &iters));
+  else
+    CKS(run_cg(ctx, d, cg_tol, cg_max_iter, &iters, ctx->a_val_orig, ctx->t_val_orig));
   if (lp_cg_iters)
     for (int l = 0; l < ctx->count; ++l) lp_cg_iters[l] = iters[l];
   // dL/db = A_B w  (w is zero off B)

@@ -242,5 +242,14 @@ void resident_free(pdhg_ctx* ctx);
 pdhg_status resident_power(pdhg_ctx* ctx);
 template <typename T>
 pdhg_status resident_solve(pdhg_ctx* ctx, const IterBuffers<T>& B);
+// conjugate gradients of the adjoint on chip (resident_cg.cu): the layout of an
+// active set (not ready where the LPs are not solved on chip), then the solves
+struct ResCgData;
+ResCgData* resident_cg_new();
+void resident_cg_free(ResCgData* d);
+bool resident_cg_ready(const ResCgData* d);
+pdhg_status resident_cg_layout(pdhg_ctx* ctx, ResCgData* d, const double* mask, const int32_t* active);
+pdhg_status resident_cg(pdhg_ctx* ctx, ResCgData* d, bool original, const double* rhs, double* w,
+                        double tol, int max_iter, std::vector<int32_t>* iters);
 
 }  // namespace pdhg

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <numeric>
 #include <vector>
@@ -14,6 +15,7 @@
 #include "dispatch.cuh"
 #include "eval_rule.cuh"
 #include "resident.cuh"
+#include "resident_host.h"
 
 namespace pdhg {
 
@@ -21,17 +23,7 @@ namespace pdhg {
 // layout build (device; one block per LP and matrix sorts and cuts the slices,
 // then a warp per slice fills it)
 // ---------------------------------------------------------------------------
-struct ResBuild {
-  ResLp* lp;
-  const int32_t *a_rp, *t_rp;   // stacked row pointers
-  ResSlice *a_sl, *t_sl;        // slices of LP l at m_off / n_off (at most one per row)
-  uint16_t *ord_m, *ord_n;      // local row / column at a position
-  uint16_t *pos_m, *pos_n;      // position of a local row / column
-  long long* elems;             // [2 lp]: elements of A~, A~^T
-  int32_t* longest;             // the longest row of any matrix
-};
-
-__global__ void __launch_bounds__(256) k_res_sort(ResBuild B) {
+static __global__ void __launch_bounds__(256) k_res_sort(ResBuild B) {
   constexpr int kBins = kResMid + 2;  // lengths 0..kResMid, and the longer rows
   __shared__ int cursor[kBins];
   __shared__ int n_long, n_mid, longest;
@@ -138,25 +130,14 @@ __global__ void __launch_bounds__(256) k_res_sort(ResBuild B) {
   }
 }
 
-// values and columns of the slices: a warp per slice, grid (x, 2 LPs);
-// entries past a row's end: value 0 and the column of the slot that holds 0
-struct ResFill {
-  const ResLp* lp;
-  const int32_t *a_rp, *t_rp, *a_col, *t_col;  // columns in the stacked numbering
-  const double *a_val, *t_val;
-  const ResSlice *a_sl, *t_sl;
-  const uint16_t *ord_m, *ord_n, *pos_m, *pos_n;
-  uint16_t *a_c, *t_c;   // NULL: columns are in place
-  double *a_v, *t_v;
-  float *a_f, *t_f;      // NULL: no float32 copy
-};
-__global__ void __launch_bounds__(256) k_res_fill(ResFill F) {
+static __global__ void __launch_bounds__(256) k_res_fill(ResFill F) {
   const int l = blockIdx.y >> 1, side = blockIdx.y & 1, lane = threadIdx.x & 31;
   const ResLp lp = F.lp[l];
   const int64_t off = side ? lp.n_off : lp.m_off, coff = side ? lp.m_off : lp.n_off;
   const int32_t* rp = (side ? F.t_rp : F.a_rp) + off;
   const int32_t* col = side ? F.t_col : F.a_col;
   const double* val = side ? F.t_val : F.a_val;
+  const int32_t* src = side ? F.t_src : F.a_src;
   const uint16_t* ord = (side ? F.ord_n : F.ord_m) + off;
   const uint16_t* pos = (side ? F.pos_m : F.pos_n) + coff;
   const ResSlice* sl = (side ? F.t_sl : F.a_sl) + off;
@@ -180,7 +161,7 @@ __global__ void __launch_bounds__(256) k_res_fill(ResFill F) {
       uint16_t c = dummy;
       double v = 0.0;
       if (j < len) {
-        v = val[b + j];
+        v = val[src ? src[b + j] : b + j];
         if (oc) c = pos[col[b + j] - coff];
       }
       const int64_t at = el + d.off + k * 32 + lane;
@@ -189,6 +170,13 @@ __global__ void __launch_bounds__(256) k_res_fill(ResFill F) {
       if (of) of[at] = (float)v;
     }
   }
+}
+
+void launch_res_sort(const ResBuild& B, int count, cudaStream_t s) {
+  k_res_sort<<<2 * count, 256, 0, s>>>(B);
+}
+void launch_res_fill(const ResFill& F, int count, int max_slices, cudaStream_t s) {
+  k_res_fill<<<dim3(std::min((max_slices + 7) / 8, 64), 2 * count), 256, 0, s>>>(F);
 }
 
 // ---------------------------------------------------------------------------
@@ -204,11 +192,12 @@ struct ResPower {
   PowerState* ps;
   int max_iter;
   double rel_tol;
+  unsigned long long wait_ns;
+  int32_t* err;  // 1 once a wait between CTAs ran out
 };
 template <int C>
 __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double tot[2];
   const int l = A.list[blockIdx.x / C];
   const ResLp lp = A.lp[l];
   const ResSmem L = res_smem(lp.m, lp.n, lp.own_m, lp.own_n, 0, 1, 8);
@@ -226,6 +215,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
     X[lp.n] = 0.0;
     Y[lp.m] = 0.0;
   }
+  ResExchange<C> ex(cl, L, smem, A.wait_ns, (uint32_t)lp.n * 8u, (uint32_t)lp.m * 8u, 2, 1);
   double lam = 0.0, lam_prev = 0.0, inv = 0.0;
   int k = 0;
   bool stopped = A.max_iter <= 0;
@@ -235,9 +225,9 @@ __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
       const double* const buf[1] = {X};
       double u[1] = {0.0};
       res_dot<1, false>(s, av, Ma.col, buf, u);
-      if (row >= 0) cl.push(L.Y + (uint32_t)(s.p0 + row) * 8u, u[0]);
+      if (row >= 0) ex.send_y(s.p0 + row, u[0]);
     });
-    cl.sync();
+    ex.wait(1);
     double q[2] = {0.0, 0.0};
     Mt.template each<C>([&](const ResSlice& s, int row) {
       const double* const buf[1] = {Y};
@@ -248,22 +238,32 @@ __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
       q[0] += X[s.p0 + row] * w[0];
       q[1] += w[0] * w[0];
     });
-    res_reduce<2>(cl, L, smem, q, tot);
-    lam = tot[0];
     k += 1;
-    const double nw = sqrt(tot[1]);
-    if (nw == 0.0) {
-      inv = 0.0;
-      break;
-    }
-    inv = 1.0 / nw;
-    stopped = (k > 1 && fabs(lam - lam_prev) <= A.rel_tol * lam) || k >= A.max_iter;
-    lam_prev = lam;
-    Mt.template each<C>([&](const ResSlice& s, int row) {
-      if (row >= 0) cl.push(L.X + (uint32_t)(s.p0 + row) * 8u, wv[s.loc + row] * inv);
+    double t[2][3];
+    ex.sum(q, 0, t, [&](int which, double v, double (&o)[3]) {
+      if (which == 0) {  // lam, and whether it has settled
+        o[0] = v;
+        o[1] = k > 1 && fabs(v - lam_prev) <= A.rel_tol * v ? 1.0 : 0.0;
+      } else {  // |w|^2 = 0, 1 / |w|
+        o[0] = v == 0.0 ? 1.0 : 0.0;
+        o[1] = v == 0.0 ? 0.0 : 1.0 / sqrt(v);
+      }
+      o[2] = 0.0;
     });
-    cl.sync();
+    const bool zero = __double_as_longlong(t[1][0]) != 0;
+    lam = t[0][0];
+    inv = t[1][1];
+    if (!zero) lam_prev = lam;
+    stopped = zero || __double_as_longlong(t[0][1]) != 0 || k >= A.max_iter;
+    if (ex.ends(stopped)) break;
+    Mt.template each<C>([&](const ResSlice& s, int row) {
+      if (row >= 0) ex.send_x(s.p0 + row, wv[s.loc + row] * inv);
+    });
+    ex.wait(0);
+    ex.next();
   }
+  if (__syncthreads_or(ex.lost) && tid == 0) atomicExch(A.err, 1);
+  cl.sync();  // no CTA leaves while another may still write to it
   if (cl.rank == 0 && tid == 0) {
     PowerState p{};
     p.lam = lam;
@@ -280,11 +280,6 @@ __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-struct ResGroup {
-  int C, first, count;  // LPs list[first..first + count)
-  size_t smem_solve = 0, smem_power = 0;
-};
-
 struct ResData {
   ResLp* lp = nullptr;
   int32_t* list = nullptr;
@@ -296,8 +291,7 @@ struct ResData {
   int32_t* active = nullptr;  // [0] LPs not finished, [1] a wait ran out
   int max_slices = 1;
   std::vector<ResGroup> groups;
-  cudaStream_t side[4] = {};  // the groups of a launch run side by side
-  cudaEvent_t fork = nullptr, join[4] = {};
+  ResStreams side;
 };
 static ResData* res_of(const pdhg_ctx* ctx) { return static_cast<ResData*>(ctx->resident); }
 
@@ -312,7 +306,7 @@ static const void* power_kernel(int C) {
 }
 
 // the kernel may run with `smem` bytes in clusters of C (its limits are raised)
-static bool res_fits(const void* f, int C, size_t smem, size_t smem_optin) {
+bool res_fits(const void* f, int C, size_t smem, size_t smem_optin) {
   if (set_max_dyn_smem(f, smem_optin) != cudaSuccess) return false;
   cudaFuncAttributes a;
   if (cudaFuncGetAttributes(&a, f) != cudaSuccess || smem + a.sharedSizeBytes > smem_optin) return false;
@@ -330,11 +324,7 @@ static bool res_fits(const void* f, int C, size_t smem, size_t smem_optin) {
 void resident_free(pdhg_ctx* ctx) {
   ResData* d = res_of(ctx);
   if (!d) return;
-  for (cudaStream_t s : d->side)
-    if (s) cudaStreamDestroy(s);
-  for (cudaEvent_t e : d->join)
-    if (e) cudaEventDestroy(e);
-  if (d->fork) cudaEventDestroy(d->fork);
+  d->side.free();
   delete d;
   ctx->resident = nullptr;
 }
@@ -342,6 +332,66 @@ void resident_free(pdhg_ctx* ctx) {
 static ResSmem solve_smem(const pdhg_ctx* ctx, int m, int n, int C) {
   const bool hal = ctx->opt.method == 1;
   return res_smem(m, n, res_own(m, C), res_own(n, C), hal ? 6 : 4, hal ? 4 : 2, ctx->mixed ? 4 : 8);
+}
+
+// The cluster size of every LP: for each of several shares of the batch's work
+// that a CTA takes at most, the schedule (largest first, each cluster on the
+// SMs that are free first) is played through and the shortest kept.  A CTA gets
+// at least min_ops operations of an iteration and an LP room for its vectors;
+// empty where an LP fits in no cluster.  512 float64 LPs: shares of 1/8 / 1/4 /
+// 1/2 / 1 of an SM's mean 76 / 53 / 47 / 46 ms; 64 LPs of 2000 x 5000 on 152
+// SMs: clusters of 4 run in two waves (11.1 ms), of 2 in one.
+std::vector<int> res_clusters(const pdhg_ctx* ctx, const std::vector<double>& ops, double min_ops,
+                              const std::function<bool(int, int)>& fits) {
+  const int count = (int)ops.size();
+  std::vector<int> least((size_t)count), order((size_t)count), best;
+  double total = 0.0;
+  for (int l = 0; l < count; ++l) {
+    int c = 1;
+    while (c < kResMaxC && !fits(l, c)) c *= 2;
+    if (!fits(l, c)) return {};
+    least[l] = c;
+    total += ops[l];
+  }
+  std::iota(order.begin(), order.end(), 0);
+  double shortest = 0.0;
+  for (double f = 0.25; f < 5.0; f *= 1.41421356) {
+    const double share = std::max(f * total / ctx->nsm, min_ops);
+    std::vector<int> C(least);
+    for (int l = 0; l < count; ++l)
+      while (C[l] < kResMaxC && ops[l] > share * C[l]) C[l] *= 2;
+    std::sort(order.begin(), order.end(), [&](int a, int b) {
+      if (C[a] != C[b]) return C[a] > C[b];
+      if (ops[a] != ops[b]) return ops[a] > ops[b];
+      return a < b;
+    });
+    std::vector<double> busy((size_t)ctx->nsm, 0.0);  // ascending
+    for (int l : order) {
+      // clocks of an iteration: 2 operations per clock and SM, and the exchanges
+      const int c = std::min(C[l], ctx->nsm);
+      const double t = ops[l] / (2.0 * C[l]) + (C[l] > 1 ? 2000.0 : 1500.0);
+      const double end = busy[c - 1] + t;
+      busy.erase(busy.begin(), busy.begin() + c);
+      busy.insert(std::upper_bound(busy.begin(), busy.end(), end), (size_t)c, end);
+    }
+    if (best.empty() || busy.back() < shortest) {
+      shortest = busy.back();
+      best = C;
+    }
+  }
+  return best;
+}
+
+// the LPs by cluster size, then work (a launch group is a run of one size)
+std::vector<int32_t> res_order(const std::vector<ResLp>& lps, const std::vector<double>& ops) {
+  std::vector<int32_t> list(lps.size());
+  std::iota(list.begin(), list.end(), 0);
+  std::sort(list.begin(), list.end(), [&](int a, int b) {
+    if (lps[a].C != lps[b].C) return lps[a].C > lps[b].C;
+    if (ops[a] != ops[b]) return ops[a] > ops[b];
+    return a < b;
+  });
+  return list;
 }
 
 // Chooses the cluster size of every LP and builds the layout; leaves
@@ -355,7 +405,6 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
   const int count = ctx->count;
   std::vector<ResLp> lps((size_t)count);
   std::vector<double> ops((size_t)count);
-  double total = 0.0;
   for (int l = 0; l < count; ++l) {
     ResLp& p = lps[l];
     p = ResLp{};
@@ -365,27 +414,18 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
     p.n = ctx->batch ? (int)(ctx->h_n_off[l + 1] - p.n_off) : ctx->n;
     const int64_t z = (int64_t)ctx->h_a_rp[p.m_off + p.m] - ctx->h_a_rp[p.m_off];
     if (p.m > 65534 || p.n > 65534 || z > kResMaxNnz) return PDHG_OK;
-    ops[l] = 2.0 * (double)z + 4.0 * p.n + 7.0 * p.m;
-    total += ops[l];
+    ops[l] = 2.0 * (double)z + 3.0 * p.n + 7.0 * p.m;
   }
-  // A cluster's size: a CTA's share of an LP at most an SM's share of the
-  // whole batch (so no LP is left running alone on few SMs), at least
-  // kResMinOps operations of an iteration, and room for its vectors.
-  const double share = std::max(total / ctx->nsm, ctx->mixed ? kResMinOps32 : kResMinOps64);
+  auto fits = [&](int l, int c) {
+    const size_t need = std::max<size_t>(
+        solve_smem(ctx, lps[l].m, lps[l].n, c).total,
+        res_smem(lps[l].m, lps[l].n, res_own(lps[l].m, c), res_own(lps[l].n, c), 0, 1, 8).total);
+    return need + 2048 <= ctx->smem_optin;  // the kernels' static shared memory
+  };
+  const std::vector<int> Cs = res_clusters(ctx, ops, ctx->mixed ? kResMinOps32 : kResMinOps64, fits);
+  if (Cs.empty()) return PDHG_OK;
+  for (int l = 0; l < count; ++l) lps[l].C = Cs[l];
   bool use[5] = {};
-  for (int l = 0; l < count; ++l) {
-    int C = 1;
-    while (C < kResMaxC && ops[l] > share * C) C *= 2;
-    auto fits = [&](int c) {
-      const size_t need = std::max<size_t>(
-          solve_smem(ctx, lps[l].m, lps[l].n, c).total,
-          res_smem(lps[l].m, lps[l].n, res_own(lps[l].m, c), res_own(lps[l].n, c), 0, 1, 8).total);
-      return need + 2048 <= ctx->smem_optin;  // the kernels' static shared memory
-    };
-    while (C < kResMaxC && !fits(C)) C *= 2;
-    if (!fits(C)) return PDHG_OK;
-    lps[l].C = C;
-  }
   // the cluster sizes the device runs (16 may not be available)
   for (int l = 0; l < count; ++l) use[(int)std::lround(std::log2(lps[l].C))] = true;
   for (int q = 0; q < 5; ++q) {
@@ -421,13 +461,7 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
   CKS(dalloc(ctx, &elems, 2 * (size_t)count));
   CK(cudaMemsetAsync(d->active, 0, 2 * sizeof(int32_t), ctx->stream));
   // launch groups by cluster size, the largest LPs first
-  std::vector<int32_t> list((size_t)count);
-  std::iota(list.begin(), list.end(), 0);
-  std::sort(list.begin(), list.end(), [&](int a, int b) {
-    if (lps[a].C != lps[b].C) return lps[a].C > lps[b].C;
-    if (ops[a] != ops[b]) return ops[a] > ops[b];
-    return a < b;
-  });
+  std::vector<int32_t> list = res_order(lps, ops);
   for (int i = 0; i < count; ++i) {
     ResLp& p = lps[list[i]];
     p.own_m = res_own(p.m, p.C);
@@ -443,7 +477,7 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
   CK(cudaMemcpyAsync(d->list, list.data(), sizeof(int32_t) * count, cudaMemcpyHostToDevice, ctx->stream));
   ResBuild b{d->lp, ctx->a_rp, ctx->t_rp, d->a_sl, d->t_sl, d->ord_m, d->ord_n, d->pos_m, d->pos_n, elems,
              d->active};
-  k_res_sort<<<2 * count, 256, 0, ctx->stream>>>(b);
+  launch_res_sort(b, count, ctx->stream);
   std::vector<long long> el(2 * (size_t)count);
   CK(cudaMemcpyAsync(el.data(), elems, sizeof(long long) * el.size(), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(lps.data(), d->lp, sizeof(ResLp) * count, cudaMemcpyDeviceToHost, ctx->stream));
@@ -471,51 +505,38 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
     CKS(dalloc(ctx, &d->t_f, (size_t)et));
   }
   CK(cudaMemcpyAsync(d->lp, lps.data(), sizeof(ResLp) * count, cudaMemcpyHostToDevice, ctx->stream));
-  const ResFill f{d->lp,    ctx->a_rp, ctx->t_rp, ctx->a_col, ctx->t_col, ctx->a_val64, ctx->t_val64,
-                  d->a_sl,  d->t_sl,   d->ord_m,  d->ord_n,   d->pos_m,   d->pos_n,     d->a_col,
-                  d->t_col, d->a_val,  d->t_val,  d->a_f,     d->t_f};
-  k_res_fill<<<dim3(std::min((d->max_slices + 7) / 8, 64), 2 * count), 256, 0, ctx->stream>>>(f);
+  launch_res_fill(ResFill{d->lp, ctx->a_rp, ctx->t_rp, ctx->a_col, ctx->t_col, ctx->a_val64,
+                          ctx->t_val64, nullptr, nullptr, d->a_sl, d->t_sl, d->ord_m, d->ord_n,
+                          d->pos_m, d->pos_n, d->a_col, d->t_col, d->a_val, d->t_val, d->a_f, d->t_f},
+                  count, d->max_slices, ctx->stream);
   ctx->launches += 2;
   CK(cudaGetLastError());
-  if (d->groups.size() > 1) {
-    CK(cudaEventCreateWithFlags(&d->fork, cudaEventDisableTiming));
-    for (size_t g = 1; g < d->groups.size(); ++g) {
-      CK(cudaStreamCreateWithFlags(&d->side[g - 1], cudaStreamNonBlocking));
-      CK(cudaEventCreateWithFlags(&d->join[g - 1], cudaEventDisableTiming));
-    }
-  }
+  CK(d->side.make((int)d->groups.size()));
   CK(cudaStreamSynchronize(ctx->stream));  // the host vectors go out of scope
-  return PDHG_OK;
-}
-
-// launch(group, stream) for every group, side by side
-template <class F>
-static pdhg_status res_groups(pdhg_ctx* ctx, F&& launch) {
-  ResData* d = res_of(ctx);
-  if (d->groups.size() > 1) CK(cudaEventRecord(d->fork, ctx->stream));
-  for (size_t g = 0; g < d->groups.size(); ++g) {
-    cudaStream_t s = g == 0 ? ctx->stream : d->side[g - 1];
-    if (g) CK(cudaStreamWaitEvent(s, d->fork, 0));
-    CK(launch(d->groups[g], s));
-    ctx->launches += 1;
-    if (g) CK(cudaEventRecord(d->join[g - 1], s));
-  }
-  for (size_t g = 1; g < d->groups.size(); ++g) CK(cudaStreamWaitEvent(ctx->stream, d->join[g - 1], 0));
   return PDHG_OK;
 }
 
 pdhg_status resident_power(pdhg_ctx* ctx) {
   ResData* d = res_of(ctx);
-  ResPower A{d->lp,    nullptr,  d->a_sl,  d->t_sl, d->a_col, d->t_col,
-             d->a_val, d->t_val, ctx->ps,  ctx->opt.power_max_iter, ctx->opt.power_rel_tol};
-  return res_groups(ctx, [&](const ResGroup& g, cudaStream_t s) {
+  ResPower A{d->lp,    nullptr,  d->a_sl, d->t_sl, d->a_col, d->t_col,
+             d->a_val, d->t_val, ctx->ps, ctx->opt.power_max_iter, ctx->opt.power_rel_tol,
+             (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull, d->active + 1};
+  CKS(res_groups(ctx, d->groups, d->side, [&](const ResGroup& g, cudaStream_t s) {
     A.list = d->list + g.first;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = res_config(g.C, g.count, g.smem_power, s, &attr);
     cudaError_t e = cudaSuccess;
     RES_DISPATCH_C(g.C, e = cudaLaunchKernelEx(&cfg, k_res_power<C_>, A));
     return e;
-  });
+  }));
+  int32_t err = 0;
+  CK(cudaMemcpyAsync(&err, d->active + 1, sizeof(err), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  if (err) {
+    set_error("power iteration: a CTA waited longer than options.wait_limit_ms for another's vector");
+    return PDHG_CUDA_ERROR;
+  }
+  return PDHG_OK;
 }
 
 template <typename T>
@@ -543,7 +564,7 @@ static pdhg_status res_solve(pdhg_ctx* ctx, const IterBuffers<T>& B, int32_t* ac
   A.slice_ns = 100000000ull;
   A.wait_ns = (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull;
   A.err = d->active + 1;
-  return res_groups(ctx, [&](const ResGroup& g, cudaStream_t s) {
+  return res_groups(ctx, d->groups, d->side, [&](const ResGroup& g, cudaStream_t s) {
     A.list = d->list + g.first;
     return launch_res_solve<T>(A, g.C, g.count, g.smem_solve, ctx->opt.method == 1, s);
   });

@@ -81,9 +81,9 @@ __host__ __device__ inline ResSmem res_smem(int m, int n, int own_m, int own_n, 
   };
   r.sc = take(sizeof(Scalars));
   r.rec = take(kResMaxC * 18 * 8);   // one record per CTA: 16 sums, 1 flag
-  r.red = take(16 * kResWarps * 8);
+  r.red = take(nvm ? 16 * kResWarps * 8 : (2 * kResThreads + 8) * 8);  // (no vectors of rows: ResExchange)
   r.tab = take(64 * 8);              // averaging weights of 64 iterations
-  r.bar = take(16);                  // transaction barriers of X and Y
+  r.bar = take(32);                  // transaction barriers: X, Y and two sums
   r.X = take((uint32_t)(((m > n ? m : n) + 1) * es));
   r.Y = take((uint32_t)((m + 1) * es));
   r.own_n = take((uint32_t)(own_n * nvn * es));
@@ -176,6 +176,15 @@ struct ResCluster {
             "r"(__float_as_int(v)), "r"(at(q, bar))
             : "memory");
     }
+  }
+  __device__ __forceinline__ void send_to(int q, uint32_t off, uint32_t bar, double v) const {
+    if constexpr (C == 1)
+      push(off, v);
+    else
+      asm volatile(
+          "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(at(q, off)),
+          "l"(__double_as_longlong(v)), "r"(at(q, bar))
+          : "memory");
   }
   // waits until the vector counted by barrier `bar` has arrived (phase parity)
   // and lets thread 0 expect the next one; false (for the whole warp) once a
@@ -350,6 +359,108 @@ __device__ __forceinline__ bool res_reduce(const ResCluster<C>& cl, const ResSme
   return f;
 }
 
+// Exchanges of an iteration that needs sums besides the two vectors (the power
+// iteration, the conjugate gradients): barrier 0 counts X, 1 Y, 2 and 3 the
+// records of two sums.  Each barrier goes through one phase per iteration.  A
+// CTA may be one exchange ahead of another, never two: each exchange waits for
+// every CTA's part, so a record is read everywhere before its slot is written
+// again.
+template <int C>
+struct ResExchange {
+  const ResCluster<C>& cl;
+  const ResSmem& L;
+  unsigned char* smem;
+  unsigned long long wait_ns;
+  uint32_t bytes_x, bytes_y;
+  int nq0, nq1;        // quantities of the two sums
+  uint32_t phase = 0;
+  bool lost = false;  // a wait ran out (uniform in a warp)
+  __device__ __forceinline__ ResExchange(const ResCluster<C>& c, const ResSmem& l, unsigned char* s,
+                                         unsigned long long limit, uint32_t bx, uint32_t by,
+                                         int q0, int q1)
+      : cl(c), L(l), smem(s), wait_ns(limit), bytes_x(bx), bytes_y(by), nq0(q0), nq1(q1) {
+    if (C > 1 && threadIdx.x == 0)
+      for (int b = 0; b < 4; ++b) {
+        mbar_init(cl.base + L.bar + 8u * b);
+        mbar_arrive_expect(cl.base + L.bar + 8u * b, expect(b));
+      }
+  }
+  __device__ __forceinline__ uint32_t expect(int b) const {
+    return b == 0 ? bytes_x : b == 1 ? bytes_y : (uint32_t)(C * 8 * (b == 2 ? nq0 : nq1));
+  }
+  __device__ __forceinline__ void send_x(int p, double v) const { cl.send(L.X + 8u * p, L.bar, v); }
+  __device__ __forceinline__ void send_y(int p, double v) const { cl.send(L.Y + 8u * p, L.bar + 8u, v); }
+  __device__ __forceinline__ void wait(int b) {
+    if constexpr (C == 1)
+      __syncthreads();
+    else if (!lost)
+      lost = !cl.arrived(L.bar + 8u * b, phase, expect(b), wait_ns);
+  }
+  // NQ sums over the cluster, the same bits in every thread; slot 0 or 1, each
+  // once per iteration.  The threads' shares go through shared memory to one
+  // warp per quantity (16 values a lane, then a tree): every warp summing its
+  // own by shuffles took 5 float64 operations of 16 clocks per warp and
+  // quantity, 3600 clocks a sum; this takes about 1100.  What follows from a
+  // total (a quotient, a root, a test) is taken there too, once instead of by
+  // all 16 warps: fin(quantity, total, o) sets o[0..2], which every thread gets
+  // in res[quantity][0..2].
+  template <int NQ, class F>
+  __device__ __forceinline__ void sum(const double (&v)[NQ], int slot, double (&res)[NQ][3], F&& fin) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* red = reinterpret_cast<double*>(smem + L.red);
+    double* out = red + 2 * kResThreads;  // the totals
+    const double* rec = reinterpret_cast<const double*>(smem + L.rec) + slot * 2 * kResMaxC;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) red[q * kResThreads + threadIdx.x] = v[q];
+    __syncthreads();
+    if (warp < NQ) {
+      const double* mine = red + warp * kResThreads + lane;
+      double t[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        t[e] = mine[e * 32];
+#pragma unroll
+        for (int k = 1; k < kResWarps / 4; ++k) t[e] += mine[(e + 4 * k) * 32];
+      }
+      t[0] = (t[0] + t[1]) + (t[2] + t[3]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+      const uint32_t bar = L.bar + 16u + 8u * slot;
+      if (lane < C)
+        cl.send_to(lane, L.rec + (uint32_t)(slot * 2 * kResMaxC + warp * kResMaxC + cl.rank) * 8u, bar, t[0]);
+      if (C > 1) {
+        // the records of every CTA, in a tree
+        wait(2 + slot);
+        double r = lane < C ? rec[warp * kResMaxC + lane] : 0.0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        t[0] = r;
+      }
+      if (lane == 0) {
+        double o[3];
+        fin(warp, t[0], o);
+        out[4 * warp] = o[0];
+        out[4 * warp + 1] = o[1];
+        out[4 * warp + 2] = o[2];
+      }
+    } else if (C > 1) {
+      wait(2 + slot);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      res[q][0] = out[4 * q];
+      res[q][1] = out[4 * q + 1];
+      res[q][2] = out[4 * q + 2];
+    }
+  }
+  // whether the loop ends, the same for all of the CTA's threads (after a lost
+  // wait its warps may have read different sums)
+  __device__ __forceinline__ bool ends(bool stop) const { return __syncthreads_or(stop || lost); }
+  // ends an iteration that used every barrier once
+  __device__ __forceinline__ void next() { phase ^= 1u; }
+};
+
 #define RES_DISPATCH_C(c, ...)  \
   switch (c) {                  \
     case 1: {                   \
@@ -388,6 +499,35 @@ inline cudaLaunchConfig_t res_config(int C, int lps, size_t smem, cudaStream_t s
   cfg.numAttrs = 1;
   return cfg;
 }
+
+// ---------------------------------------------------------------------------
+// building and launching (resident.cu)
+// ---------------------------------------------------------------------------
+struct ResBuild {
+  ResLp* lp;
+  const int32_t *a_rp, *t_rp;   // stacked row pointers
+  ResSlice *a_sl, *t_sl;        // slices of LP l at m_off / n_off (at most one per row)
+  uint16_t *ord_m, *ord_n;      // local row / column at a position
+  uint16_t *pos_m, *pos_n;      // position of a local row / column
+  long long* elems;             // [2 lp]: elements of A~, A~^T
+  int32_t* longest;             // the longest row of any matrix
+};
+
+// values and columns of the slices: a warp per slice, grid (x, 2 LPs);
+// entries past a row's end: value 0 and the column of the slot that holds 0
+struct ResFill {
+  const ResLp* lp;
+  const int32_t *a_rp, *t_rp, *a_col, *t_col;  // columns in the stacked numbering
+  const double *a_val, *t_val;
+  const int32_t *a_src, *t_src;  // NULL, or where the values of entry k are
+  const ResSlice *a_sl, *t_sl;
+  const uint16_t *ord_m, *ord_n, *pos_m, *pos_n;
+  uint16_t *a_c, *t_c;   // NULL: columns are in place
+  double *a_v, *t_v;
+  float *a_f, *t_f;      // NULL: no float32 copy
+};
+void launch_res_sort(const ResBuild& B, int count, cudaStream_t s);
+void launch_res_fill(const ResFill& F, int count, int max_slices, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // the solve (resident_solve.cuh)

@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
           const long long tt = tt0 + i + tid;
           tab[tid] = hal ? (T)((double)(tt + 1) / (double)(tt + 2)) : (T)(1.0 / (double)(tt + 1));
         }
-        __syncthreads();
+        lost = __syncthreads_or(lost);
+        if (lost) break;
       }
       const T w = tab[i & 63];
       const bool first = tt0 + i == 0;
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
         }
       });
       if constexpr (C == 1) cl.sync();
-      else lost |= !cl.arrived(bar_x, phase, bytes_x, A.wait_ns);
+      else if (!lost) lost = !cl.arrived(bar_x, phase, bytes_x, A.wait_ns);
       Ma.template each<C>([&](const ResSlice& s, int row) {
         const T* const buf[1] = {X};
         T h1[1] = {T(0)};
@@ -160,9 +161,8 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
         }
       });
       if constexpr (C == 1) cl.sync();
-      else lost |= !cl.arrived(bar_y, phase, bytes_y, A.wait_ns);
+      else if (!lost) lost = !cl.arrived(bar_y, phase, bytes_y, A.wait_ns);
       phase ^= 1u;
-      if (lost) break;
     }
     // a wait that ran out: tell every CTA (each comes to the next cluster
     // barrier, since all its waits are bounded)

@@ -129,3 +129,39 @@ def test_a_stop_between_evaluations_changes_nothing():
         got = s.state()
     for k in KEYS:
         np.testing.assert_array_equal(got[k], ref[k], err_msg=k)
+
+
+def test_polish_and_adjoint_match_the_tile_kernels():
+    """Conjugate gradients on chip, cut down to the active columns, against the
+    tile kernels': LPs of every row class, more rows than columns, no active
+    column at all (b = 0), and one large enough for a wide cluster.  Both stop
+    at a relative residual of 1e-12 of normal equations of condition up to 1e4
+    or so: 1e-8 relative."""
+    lps = [MAKERS[k]() for k in ("planted", "short_edge", "mid_edge", "tall", "wide_cluster")]
+    lps.append(lpgen.planted_lp(30, 80, seed=3, n_pos=0))
+    g = np.random.default_rng(0).standard_normal(sum(lp.n for lp in lps))
+    out = []
+    for kw in ({}, {"tile_nnz": 2044}):
+        with pdhg.BatchSolver(lps, **kw) as s:
+            s.solve(1e-4, 20_000)
+            before = s.launch_count()
+            p = s.polish()
+            out.append((p["active"], p["x"], s.adjoint(g)["grad_b"], s.launch_count() - before, p["cg_iters"]))
+            if not kw:  # a second active set in the same context
+                s.set_rhs(np.concatenate([lp.b for lp in lps]), np.concatenate([lp.c for lp in lps]))
+                s.solve(1e-4, 20_000)
+                np.testing.assert_array_equal(s.polish()["x"], p["x"])
+                np.testing.assert_array_equal(s.adjoint(g)["grad_b"], out[0][2])
+    a, b = out
+    np.testing.assert_array_equal(a[0], b[0])
+    assert a[0][-1] == 0 and a[4][-1] == 0
+    assert a[3] < b[3]
+    assert rel_inf(a[1], b[1]) < 1e-8
+    # the adjoint is A_B (A_B^T A_B)^-1 g: with more active columns than rows
+    # ("mid_edge") that matrix is singular and no solution exists to compare
+    first = np.concatenate([[0], np.cumsum([lp.m for lp in lps])])
+    defined = [i for i, lp in enumerate(lps) if a[0][i] <= lp.m]
+    assert len(defined) == len(lps) - 1
+    for i in defined:
+        u, v = a[2][first[i]:first[i + 1]], b[2][first[i]:first[i + 1]]
+        assert np.array_equal(u, v) or rel_inf(u, v) < 1e-8, i
