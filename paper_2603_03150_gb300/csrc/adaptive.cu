@@ -44,7 +44,7 @@ struct AdaptPrimalEpi {
   T acc;  // this thread's sum of dx_j^2 over rows finished in one tile
   __device__ __forceinline__ void row(int j, const T (&s)[1], int group) {
     const T xo = x[j], xa = x_avg[j];
-    const T xn = fmax(T(0), xo - tau * (c[j] - s[0]));
+    const T xn = max0(xo - tau * (c[j] - s[0]));
     const T d = xn - xo;
     x_avg_prev[j] = xa;
     x[j] = xn;

@@ -58,12 +58,12 @@ struct BPrimalEpi {
     if (s.done) return false;
     const long long tt = s.t + i;
     tau = (T)s.tau;
-    w = (T)(1.0 / (double)(tt + 1));
+    w = avg_weight(tt + 1, T(0));
     first = tt == 0;
     return true;
   }
   __device__ __forceinline__ void row(int j, const T (&s)[1], int) {
-    const T xn = fmax(T(0), x[j] - tau * (c[j] - s[0]));
+    const T xn = max0(x[j] - tau * (c[j] - s[0]));
     x[j] = xn;
     x_avg[j] = first ? xn : x_avg[j] + (xn - x_avg[j]) * w;
   }
@@ -85,7 +85,7 @@ struct BDualEpi {
     if (s.done) return false;
     const long long tt = s.t + i;
     sigma = (T)s.sigma;
-    w = (T)(1.0 / (double)(tt + 1));
+    w = avg_weight(tt + 1, T(0));
     first = tt == 0;
     return true;
   }

@@ -380,6 +380,58 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mb, uint32_t parity, unsigned
   }
 }
 
+// max(0, v) and min(0, v) of doubles with integer tests (fmax / fmin would
+// take the float64 pipe); NaN gives 0 as fmax(0, NaN) does.
+__device__ __forceinline__ double max0(double v) {
+  return (unsigned long long)__double_as_longlong(v) > 0x7ff0000000000000ull ? 0.0 : v;
+}
+__device__ __forceinline__ float max0(float v) { return fmaxf(0.f, v); }
+__device__ __forceinline__ double min0(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull ? v : 0.0;
+}
+
+// 1 / n and n / (n + 1), the averaging weight and the Halpern weight after n - 1
+// iterations, n >= 1.  For float the division runs in float up to n = 2^24: both
+// operands are exact, and no quotient of two numbers of 24 bits lies within
+// 2^-49 of the middle of two floats, so rounding the float64 quotient (2^-53)
+// gives the same bits.
+__device__ __forceinline__ float avg_weight(long long n, float) {
+  return n < (1 << 24) ? 1.f / (float)(int)n : (float)(1.0 / (double)n);
+}
+__device__ __forceinline__ double avg_weight(long long n, double) { return 1.0 / (double)n; }
+__device__ __forceinline__ float halpern_weight(long long n, float) {
+  return n < (1 << 24) ? (float)(int)n / (float)(int)(n + 1) : (float)((double)n / (double)(n + 1));
+}
+__device__ __forceinline__ double halpern_weight(long long n, double) {
+  return (double)n / (double)(n + 1);
+}
+
+// A step's two scalars for a whole block.  A float64 division by every thread
+// (about 12 operations of 16 clocks per warp on GB300's float64 pipe) is work of
+// the pipe that bounds the float64 kernels: one warp divides and shares the
+// quotient (power-law LP, 64 iterations 6.54 -> 6.38 ms, with max0 above), and
+// float weights are divided in float (transportation LP, 64 Halpern iterations
+// 4.92 -> 4.89 ms).  Ends with a block barrier in float64.
+template <typename T>
+struct StepScalars {
+  T step, w;
+};
+template <typename T>
+__device__ __forceinline__ StepScalars<T> step_scalars(double step, long long n, bool halpern) {
+  if constexpr (sizeof(T) == 4) {
+    return {(T)step, halpern ? halpern_weight(n, T(0)) : avg_weight(n, T(0))};
+  } else {
+    __shared__ T weight;
+    if (threadIdx.x < 32) {
+      const T v = halpern ? halpern_weight(n, T(0)) : avg_weight(n, T(0));
+      if (threadIdx.x == 0) weight = v;
+    }
+    __syncthreads();
+    return {(T)step, weight};
+  }
+}
+
 __device__ __forceinline__ float fmadd(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
 

@@ -6,6 +6,7 @@
 // with load(i) and writes with apply(i, in, s): the panel row pass issues
 // load(i) before the partial sums arrive; row() is the two in sequence.
 #pragma once
+#include "common.cuh"
 
 namespace pdhg {
 
@@ -24,7 +25,7 @@ struct PrimalEpi {
     return In{x[j], c[j], first ? T(0) : x_avg[j]};
   }
   __device__ __forceinline__ void apply(int j, const In& in, T s) {
-    const T xn = fmax(T(0), in.x - tau * (in.c - s));
+    const T xn = max0(in.x - tau * (in.c - s));
     x[j] = xn;
     x_avg[j] = first ? xn : in.xa + (xn - in.xa) * w;
   }
@@ -123,7 +124,7 @@ struct HalpernPrimalEpi {
   };
   __device__ __forceinline__ In load(int j) const { return In{x[j], c[j], x0[j]}; }
   __device__ __forceinline__ void apply(int j, const In& in, T s) {
-    const T xh = fmax(T(0), in.xo - tau * (in.c - s));
+    const T xh = max0(in.xo - tau * (in.c - s));
     x_hat[j] = xh;
     x[j] = lam * ((T(1) + rho) * xh - rho * in.xo) + (T(1) - lam) * in.x0;
   }

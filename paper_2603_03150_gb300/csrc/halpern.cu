@@ -25,8 +25,8 @@ __global__ void __launch_bounds__(BLOCK) k_hprimal(IterBuffers<T> B, int i) {
   if (B.sc->done) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const long long tt = B.sc->t + i;  // iterations since restart before this one
-  const double lam = (double)(tt + 1) / (double)(tt + 2);
-  HalpernPrimalEpi<T> epi{B.x, B.x_avg, B.c_t, B.x_last, (T)B.sc->tau, (T)lam, (T)B.rho};
+  const StepScalars<T> st = step_scalars<T>(B.sc->tau, tt + 1, true);
+  HalpernPrimalEpi<T> epi{B.x, B.x_avg, B.c_t, B.x_last, st.step, st.w, (T)B.rho};
   Gather<T, 1> g{{B.y}};
   run_sched<T, 1, BLOCK, E>(B.t_sched, B.t_rp, B.t_col, B.t_val, g, epi, smem);
 }
@@ -38,9 +38,9 @@ __global__ void __launch_bounds__(BLOCK) k_hdual(IterBuffers<T> B, int i) {
   if (B.sc->done) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const long long tt = B.sc->t + i;
-  const double lam = (double)(tt + 1) / (double)(tt + 2);
-  HalpernDualEpi<T> epi{B.y,      B.b_t,       B.Ax,    B.y_avg,           B.Ax_avg,
-                        B.y_last, B.Ax_last,   (T)B.sc->sigma, (T)lam,     (T)B.rho};
+  const StepScalars<T> st = step_scalars<T>(B.sc->sigma, tt + 1, true);
+  HalpernDualEpi<T> epi{B.y,      B.b_t,     B.Ax,    B.y_avg, B.Ax_avg,
+                        B.y_last, B.Ax_last, st.step, st.w,    (T)B.rho};
   Gather<T, 1> g{{B.x_avg}};  // x^ of this iteration
   run_sched<T, 1, BLOCK, E>(B.a_sched, B.a_rp, B.a_col, B.a_val, g, epi, smem);
 }

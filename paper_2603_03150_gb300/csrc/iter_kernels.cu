@@ -22,7 +22,8 @@ __global__ void __launch_bounds__(BLOCK) k_primal(IterBuffers<T> B, int i) {
   if (B.sc->done) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const long long tt = B.sc->t + i;  // iterations since restart before this one
-  PrimalEpi<T> epi{B.x, B.c_t, B.x_avg, (T)B.sc->tau, (T)(1.0 / (double)(tt + 1)), tt == 0};
+  const StepScalars<T> st = step_scalars<T>(B.sc->tau, tt + 1, false);
+  PrimalEpi<T> epi{B.x, B.c_t, B.x_avg, st.step, st.w, tt == 0};
   Gather<T, 1> g{{B.y}};
   run_sched<T, 1, BLOCK, E>(B.t_sched, B.t_rp, B.t_col, B.t_val, g, epi, smem);
 }
@@ -38,8 +39,8 @@ __global__ void __launch_bounds__(BLOCK) k_dual(IterBuffers<T> B, int i) {
   if (B.sc->done) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const long long tt = B.sc->t + i;
-  DualEpi<T> epi{B.y,   B.b_t, B.Ax, B.y_avg, B.Ax_avg, (T)B.sc->sigma, (T)(1.0 / (double)(tt + 1)),
-                 tt == 0};
+  const StepScalars<T> st = step_scalars<T>(B.sc->sigma, tt + 1, false);
+  DualEpi<T> epi{B.y, B.b_t, B.Ax, B.y_avg, B.Ax_avg, st.step, st.w, tt == 0};
   Gather<T, 1> g{{B.x}};
   run_sched<T, 1, BLOCK, E>(B.a_sched, B.a_rp, B.a_col, B.a_val, g, epi, smem);
 }

@@ -420,7 +420,7 @@ __device__ __forceinline__ void row_scalars(const IterBuffers<float>& B, int i, 
     const long long tt = sc->t + i;  // iterations since restart before this one
     out->done = sc->done;
     out->a = (float)(dual ? sc->sigma : sc->tau);
-    out->b = halpern ? (float)((double)(tt + 1) / (double)(tt + 2)) : (float)(1.0 / (double)(tt + 1));
+    out->b = halpern ? halpern_weight(tt + 1, 0.f) : avg_weight(tt + 1, 0.f);
     out->first = tt == 0;
   }
 }

@@ -92,17 +92,6 @@ __host__ __device__ inline ResSmem res_smem(int m, int n, int own_m, int own_n, 
   return r;
 }
 
-// max(0, v) and min(0, v) of doubles with integer tests (fmax / fmin would
-// take the float64 pipe); NaN gives 0 as fmax(0, NaN) does.
-__device__ __forceinline__ double max0(double v) {
-  return (unsigned long long)__double_as_longlong(v) > 0x7ff0000000000000ull ? 0.0 : v;
-}
-__device__ __forceinline__ float max0(float v) { return fmaxf(0.f, v); }
-__device__ __forceinline__ double min0(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull ? v : 0.0;
-}
-
 // A cluster of C CTAs, one of its CTAs (rank) with its shared memory window.
 template <int C>
 struct ResCluster {

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
       if ((i & 63) == 0) {  // the next 64 weights (one float64 division each)
         if (tid < 64) {
           const long long tt = tt0 + i + tid;
-          tab[tid] = hal ? (T)((double)(tt + 1) / (double)(tt + 2)) : (T)(1.0 / (double)(tt + 1));
+          tab[tid] = hal ? halpern_weight(tt + 1, T(0)) : avg_weight(tt + 1, T(0));
         }
         lost = __syncthreads_or(lost);
         if (lost) break;
