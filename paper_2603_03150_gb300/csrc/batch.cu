@@ -700,10 +700,6 @@ __global__ void k_bws_mu(const double* rec, const int32_t* lp_tiles, const int64
   }
 }
 
-__device__ __forceinline__ double bws_move(double target, double v, double delta) {
-  return fmin(fmax(target, v - delta), v + delta);
-}
-
 __global__ void k_bws_apply(SchedView Sn, SchedView Sm, const double* x_s, const double* z_s,
                             const double* y_s, const double* mu, double delta, double alpha,
                             int unscaled, const double* D_r, const double* D_c, double* x_out,
@@ -713,14 +709,8 @@ __global__ void k_bws_apply(SchedView Sn, SchedView Sm, const double* x_s, const
     if (tl.split >= 0 && tl.part != 0) continue;
     const double m_t = mu[tl.lp];
     for (int j = tl.row_begin + threadIdx.x; j < tl.row_end; j += blockDim.x) {
-      double xp = fmax(x_s[j], alpha), zp = fmax(z_s[j], alpha);
-      if (xp < zp) {
-        xp = bws_move(m_t / zp, xp, delta);
-        zp = bws_move(m_t / xp, zp, delta);
-      } else {
-        zp = bws_move(m_t / xp, zp, delta);
-        xp = bws_move(m_t / zp, xp, delta);
-      }
+      double xp = x_s[j], zp = z_s[j];
+      centered_pair(m_t, delta, alpha, xp, zp);
       if (unscaled) {
         xp = D_c[j] * xp;
         zp = zp / D_c[j];

@@ -256,6 +256,84 @@ __device__ __forceinline__ void parts_sum(const double* a, int na, const double*
   __syncthreads();
 }
 
+// max(0, v) and min(0, v) of doubles with integer tests (fmax / fmin would
+// take the float64 pipe); NaN gives 0 as fmax(0, NaN) does.
+__device__ __forceinline__ double max0(double v) {
+  return (unsigned long long)__double_as_longlong(v) > 0x7ff0000000000000ull ? 0.0 : v;
+}
+__device__ __forceinline__ float max0(float v) { return fmaxf(0.f, v); }
+__device__ __forceinline__ double min0(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull ? v : 0.0;
+}
+
+// max and min of doubles of which at least one is not negative, by their bits
+// (the order of the values; a NaN loses, as with fmax and fmin)
+__device__ __forceinline__ bool is_nan_bits(long long b) {
+  return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ double max_pos(double v, double w) {
+  const long long a = __double_as_longlong(v), b = __double_as_longlong(w);
+  return is_nan_bits(b) || (a > b && !is_nan_bits(a)) ? v : w;
+}
+__device__ __forceinline__ double min_pos(double v, double w) {
+  const long long a = __double_as_longlong(v), b = __double_as_longlong(w);
+  return is_nan_bits(b) || (a < b && !is_nan_bits(a)) ? v : w;
+}
+
+// x / d from inv = 1 / d: the product corrected by its residual (3 float64
+// operations; a division takes about 10)
+__device__ __forceinline__ double div_by(double x, double d, double inv) {
+  const double q = x * inv;
+  const bool finite = ((unsigned long long)__double_as_longlong(q) << 1) < 0xffe0000000000000ull;
+  return finite ? fma(fma(-q, d, x), inv, q) : q;
+}
+
+// Sums (and for quantity `mx` the maximum) of `count` records of 4 doubles, by
+// every thread of a block of 256 in a fixed order, into out[0..4) (shared); one
+// thread adding 600 records in turn, 68 clocks each, took 30 to 330 us.  `red`
+// holds 32 doubles.  Ends with a block barrier.
+__device__ __forceinline__ void fold_records(const double* rec, int count, int mx, double* out,
+                                             double* red) {
+  const int q = threadIdx.x & 3, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double s = 0.0;
+  for (int p = threadIdx.x >> 2; p < count; p += 64) {
+    const double v = __ldcg(rec + 4 * (size_t)p + q);
+    s = q == mx ? fmax(s, v) : s + v;
+  }
+#pragma unroll
+  for (int o = 16; o >= 4; o >>= 1) {
+    const double v = __shfl_down_sync(0xffffffffu, s, o);
+    s = q == mx ? fmax(s, v) : s + v;
+  }
+  if (lane < 4) red[4 * w + lane] = s;
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    double t = red[threadIdx.x];
+    for (int i = 1; i < 8; ++i)
+      t = threadIdx.x == mx ? fmax(t, red[4 * i + threadIdx.x]) : t + red[4 * i + threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+  __syncthreads();
+}
+
+// Algorithm 1's per-entry update (Section 3.1): the smaller of the pair moves
+// toward mu / (other) first, a tie moves z; the other follows.  One path for
+// both orders, so a warp divides twice per entry and not four times.
+__device__ __forceinline__ double centered_move(double target, double v, double delta) {
+  return min_pos(max_pos(target, v - delta), v + delta);
+}
+__device__ __forceinline__ void centered_pair(double mu, double delta, double alpha, double& x,
+                                              double& z) {
+  const double xp = max_pos(x, alpha), zp = max_pos(z, alpha);
+  const bool x_first = __double_as_longlong(xp) < __double_as_longlong(zp);
+  const double a = x_first ? xp : zp, b = x_first ? zp : xp;
+  const double a1 = centered_move(mu / b, a, delta);
+  const double b1 = centered_move(mu / a1, b, delta);
+  x = x_first ? a1 : b1;
+  z = x_first ? b1 : a1;
+}
+
 // ---------------------------------------------------------------------------
 // Loads of the matrix stream (column indices, values, window words): read
 // once per SpMV, so they carry an L2 evict-first policy and skip L1, leaving
@@ -378,17 +456,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mb, uint32_t parity, unsigned
     if (done) return true;
     if (global_ns() - t0 > limit_ns) return false;
   }
-}
-
-// max(0, v) and min(0, v) of doubles with integer tests (fmax / fmin would
-// take the float64 pipe); NaN gives 0 as fmax(0, NaN) does.
-__device__ __forceinline__ double max0(double v) {
-  return (unsigned long long)__double_as_longlong(v) > 0x7ff0000000000000ull ? 0.0 : v;
-}
-__device__ __forceinline__ float max0(float v) { return fmaxf(0.f, v); }
-__device__ __forceinline__ double min0(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull ? v : 0.0;
 }
 
 // 1 / n and n / (n + 1), the averaging weight and the Halpern weight after n - 1

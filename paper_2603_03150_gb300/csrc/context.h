@@ -127,7 +127,7 @@ struct pdhg_ctx {
   double* adapt_sums = nullptr;
   Launch l_aprim{}, l_adual{};  // the adaptive half-steps' launches
   double *xs64 = nullptr, *ys64 = nullptr, *out_n1 = nullptr, *out_n2 = nullptr,
-         *out_m1 = nullptr, *report = nullptr, *sums = nullptr;
+         *out_m1 = nullptr, *report = nullptr;
   Scalars* sc = nullptr;
   PowerState* ps = nullptr;
   double* partials = nullptr;  // generic reduction scratch

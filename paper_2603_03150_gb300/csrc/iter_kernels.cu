@@ -234,21 +234,21 @@ void launch_spmv(const SchedView& S, const int32_t* rp, const int32_t* col, cons
 // float64 report of an iterate on the original model.
 // ---------------------------------------------------------------------------
 struct ReportNEpi {
-  const double *x_s, *c_t, *D_c;
+  const double *x_s, *c_t, *D_c, *Dc_inv;
   double *x_out, *z_out;
   double u2, s3, xz, inf_rd;
   double* split_q;  // per split group: 4 values
   __device__ __forceinline__ void row(int j, const double (&s)[1], int group) {
-    const double d = c_t[j] - s[0];
-    const double zs = fmax(0.0, d), rd = fmin(0.0, d) / D_c[j];
+    const double d = c_t[j] - s[0], dc = D_c[j], dci = Dc_inv[j];
+    const double zs = max0(d), rd = div_by(min0(d), dc, dci);
     const double xs = x_s[j];
-    if (x_out) x_out[j] = D_c[j] * xs;
-    if (z_out) z_out[j] = zs / D_c[j];
+    if (x_out) x_out[j] = dc * xs;
+    if (z_out) z_out[j] = div_by(zs, dc, dci);
     if (group < 0) {
       u2 += rd * rd;
       s3 += c_t[j] * xs;
       xz += xs * zs;
-      inf_rd = fmax(inf_rd, fabs(rd));
+      inf_rd = max_pos(fabs(rd), inf_rd);
     } else {
       double* r = split_q + 4 * (size_t)group;
       r[0] = rd * rd;
@@ -259,49 +259,51 @@ struct ReportNEpi {
   }
 };
 
+// the block's record: three sums and a maximum
+template <int BLOCK>
+__device__ __forceinline__ void report_record(double a, double b, double c, double mx, double* red,
+                                              double* out) {
+  double v[4] = {a, b, c, 0.0};
+  block_sum_scatter<BLOCK, 4>(v, red, out);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) mx = max_pos(__shfl_down_sync(0xffffffffu, mx, off), mx);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < BLOCK / 32; ++w) mx = max_pos(red[w], mx);
+    out[3] = mx;
+  }
+}
+
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) k_report_n(SchedView S, const int32_t* rp, const int32_t* col,
                                                    const double* val, const double* x_s,
                                                    const double* y_s, const double* c_t,
-                                                   const double* D_c, double* x_out, double* z_out,
-                                                   double* partials, const Scalars* gate) {
+                                                   const double* D_c, const double* Dc_inv,
+                                                   double* x_out, double* z_out, double* partials,
+                                                   const Scalars* gate) {
   if (gate && !gate->verify) return;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[4 * (BLOCK / 32)];
   double* split_q = partials + 4 * (size_t)gridDim.x;
-  ReportNEpi epi{x_s, c_t, D_c, x_out, z_out, 0.0, 0.0, 0.0, 0.0, split_q};
+  ReportNEpi epi{x_s, c_t, D_c, Dc_inv, x_out, z_out, 0.0, 0.0, 0.0, 0.0, split_q};
   Gather<double, 1> g{{y_s}};
   run_tiles<double, 1, BLOCK, kFixedE>(S, rp, col, val, g, epi, smem);
-  // infinity norm through a max-reduction, sums through block_sum
-  const double v[3] = {epi.u2, epi.s3, epi.xz};
-  double o[3];
-  block_sum<BLOCK, 3>(v, o, red);
-  double mx = epi.inf_rd;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, off));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < BLOCK / 32; ++w) mx = fmax(mx, red[w]);
-    partials[4 * (size_t)blockIdx.x + 0] = o[0];
-    partials[4 * (size_t)blockIdx.x + 1] = o[1];
-    partials[4 * (size_t)blockIdx.x + 2] = o[2];
-    partials[4 * (size_t)blockIdx.x + 3] = mx;
-  }
+  report_record<BLOCK>(epi.u2, epi.s3, epi.xz, epi.inf_rd, red, partials + 4 * (size_t)blockIdx.x);
 }
 
 struct ReportMEpi {
-  const double *y_s, *b_t, *D_r;
+  const double *y_s, *b_t, *D_r, *Dr_inv;
   double* y_out;
   double u1, s4, inf_rp;
   double* split_q;
   __device__ __forceinline__ void row(int i, const double (&s)[1], int group) {
-    const double rp = (b_t[i] - s[0]) / D_r[i];
-    if (y_out) y_out[i] = D_r[i] * y_s[i];
+    const double dr = D_r[i], rp = div_by(b_t[i] - s[0], dr, Dr_inv[i]);
+    if (y_out) y_out[i] = dr * y_s[i];
     if (group < 0) {
       u1 += rp * rp;
       s4 += b_t[i] * y_s[i];
-      inf_rp = fmax(inf_rp, fabs(rp));
+      inf_rp = max_pos(fabs(rp), inf_rp);
     } else {
       double* r = split_q + 4 * (size_t)group;
       r[0] = rp * rp;
@@ -316,52 +318,31 @@ template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) k_report_m(SchedView S, const int32_t* rp, const int32_t* col,
                                                    const double* val, const double* x_s,
                                                    const double* y_s, const double* b_t,
-                                                   const double* D_r, double* y_out,
-                                                   double* partials, const Scalars* gate) {
+                                                   const double* D_r, const double* Dr_inv,
+                                                   double* y_out, double* partials,
+                                                   const Scalars* gate) {
   if (gate && !gate->verify) return;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[4 * (BLOCK / 32)];
   double* split_q = partials + 4 * (size_t)gridDim.x;
-  ReportMEpi epi{y_s, b_t, D_r, y_out, 0.0, 0.0, 0.0, split_q};
+  ReportMEpi epi{y_s, b_t, D_r, Dr_inv, y_out, 0.0, 0.0, 0.0, split_q};
   Gather<double, 1> g{{x_s}};
   run_tiles<double, 1, BLOCK, kFixedE>(S, rp, col, val, g, epi, smem);
-  const double v[2] = {epi.u1, epi.s4};
-  double o[2];
-  block_sum<BLOCK, 2>(v, o, red);
-  double mx = epi.inf_rp;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, off));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < BLOCK / 32; ++w) mx = fmax(mx, red[w]);
-    partials[4 * (size_t)blockIdx.x + 0] = o[0];
-    partials[4 * (size_t)blockIdx.x + 1] = o[1];
-    partials[4 * (size_t)blockIdx.x + 2] = 0.0;
-    partials[4 * (size_t)blockIdx.x + 3] = mx;
-  }
+  report_record<BLOCK>(epi.u1, epi.s4, 0.0, epi.inf_rp, red, partials + 4 * (size_t)blockIdx.x);
 }
 
 // pn/pm hold [grid][4] block partials followed by [groups][4] split records;
-// gn/gm count all of those records.
+// gn/gm count all of those records.  One block of 256.
 __global__ void k_report_final(const double* pn, int gn, const double* pm, int gm, double* out) {
+  __shared__ double red[32], tn[4], tm[4];
+  fold_records(pn, gn, 3, tn, red);
+  fold_records(pm, gm, 3, tm, red);
   if (threadIdx.x != 0) return;
-  double u2 = 0, s3 = 0, xz = 0, ird = 0, u1 = 0, s4 = 0, irp = 0;
-  for (int b = 0; b < gn; ++b) {
-    u2 += pn[4 * b];
-    s3 += pn[4 * b + 1];
-    xz += pn[4 * b + 2];
-    ird = fmax(ird, pn[4 * b + 3]);
-  }
-  for (int b = 0; b < gm; ++b) {
-    u1 += pm[4 * b];
-    s4 += pm[4 * b + 1];
-    irp = fmax(irp, pm[4 * b + 3]);
-  }
-  out[0] = sqrt(u1);
-  out[1] = sqrt(u2);
+  const double s3 = tn[1], s4 = tm[1], xz = tn[2];
+  out[0] = sqrt(tm[0]);
+  out[1] = sqrt(tn[0]);
   out[2] = fabs(s3 - s4);
-  out[3] = fmax(fmax(irp, ird), xz / (1.0 + fabs(s3)));
+  out[3] = fmax(fmax(tm[3], tn[3]), xz / (1.0 + fabs(s3)));
   out[4] = s3;
   out[5] = s4;
   out[6] = xz;
@@ -370,20 +351,21 @@ __global__ void k_report_final(const double* pn, int gn, const double* pm, int g
 
 void launch_report_n(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
                      const double* x_s, const double* y_s, const double* c_t, const double* D_c,
-                     double* x_out, double* z_out, double* partials, const Launch& L,
-                     cudaStream_t s) {
-  k_report_n<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, c_t, D_c, x_out,
-                                                    z_out, partials, nullptr);
+                     const double* Dc_inv, double* x_out, double* z_out, double* partials,
+                     const Launch& L, cudaStream_t s) {
+  k_report_n<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, c_t, D_c, Dc_inv,
+                                                    x_out, z_out, partials, nullptr);
 }
 void launch_report_m(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
                      const double* x_s, const double* y_s, const double* b_t, const double* D_r,
-                     double* y_out, double* partials, const Launch& L, cudaStream_t s) {
-  k_report_m<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, b_t, D_r, y_out,
-                                                    partials, nullptr);
+                     const double* Dr_inv, double* y_out, double* partials, const Launch& L,
+                     cudaStream_t s) {
+  k_report_m<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, b_t, D_r, Dr_inv,
+                                                    y_out, partials, nullptr);
 }
 void launch_report_final(const double* pn, int gn, const double* pm, int gm, double* out,
                          cudaStream_t s) {
-  k_report_final<<<1, 32, 0, s>>>(pn, gn, pm, gm, out);
+  k_report_final<<<1, 256, 0, s>>>(pn, gn, pm, gm, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -404,19 +386,14 @@ __global__ void k_fp64_prep(IterBuffers<T> B, double* xs, double* ys) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B.m; i += stride) ys[i] = (double)y[i];
 }
 
+// one block of 256
 __global__ void k_fp64_final(Scalars* sc, const double* pn, int gn, const double* pm, int gm,
                              long long* log_k, int32_t* log_flags, double* log_kkt) {
-  if (threadIdx.x != 0 || !sc->verify) return;
-  double u2 = 0, s3 = 0, u1 = 0, s4 = 0;
-  for (int b = 0; b < gn; ++b) {
-    u2 += pn[4 * b];
-    s3 += pn[4 * b + 1];
-  }
-  for (int b = 0; b < gm; ++b) {
-    u1 += pm[4 * b];
-    s4 += pm[4 * b + 1];
-  }
-  eval_fp64_check(*sc, u1, u2, s3, s4, log_k, log_flags, log_kkt);
+  __shared__ double red[32], tn[4], tm[4];
+  if (!sc->verify) return;
+  fold_records(pn, gn, 3, tn, red);
+  fold_records(pm, gm, 3, tm, red);
+  if (threadIdx.x == 0) eval_fp64_check(*sc, tm[0], tn[0], tn[1], tm[1], log_k, log_flags, log_kkt);
 }
 
 template <typename T>
@@ -425,11 +402,12 @@ void launch_fp64_check(const IterBuffers<T>& B, const Fp64Check& C, cudaStream_t
   double* pn = B.partials;
   double* pm = B.partials + 4 * (size_t)(C.gn + 1);
   k_report_n<kBlock><<<C.Lt.grid, kBlock, C.Lt.smem, s>>>(C.St, B.t_rp, B.t_col, C.t_val, C.xs, C.ys,
-                                                          B.c_t64, B.D_c, nullptr, nullptr, pn,
-                                                          B.sc);
+                                                          B.c_t64, B.D_c, B.Dc_inv, nullptr,
+                                                          nullptr, pn, B.sc);
   k_report_m<kBlock><<<C.La.grid, kBlock, C.La.smem, s>>>(C.Sa, B.a_rp, B.a_col, C.a_val, C.xs, C.ys,
-                                                          B.b_t64, B.D_r, nullptr, pm, B.sc);
-  k_fp64_final<<<1, 32, 0, s>>>(B.sc, pn, C.gn, pm, C.gm, B.log_k, B.log_flags, B.log_kkt);
+                                                          B.b_t64, B.D_r, B.Dr_inv, nullptr, pm,
+                                                          B.sc);
+  k_fp64_final<<<1, 256, 0, s>>>(B.sc, pn, C.gn, pm, C.gm, B.log_k, B.log_flags, B.log_kkt);
 }
 template void launch_fp64_check<float>(const IterBuffers<float>&, const Fp64Check&, cudaStream_t);
 
@@ -442,7 +420,7 @@ struct WsEpi {
   double xz;
   double* split_q;
   __device__ __forceinline__ void row(int j, const double (&s)[1], int group) {
-    const double z = fmax(0.0, c_t[j] - s[0]);
+    const double z = max0(c_t[j] - s[0]);
     z_s[j] = z;
     if (group < 0)
       xz += x_s[j] * z;
@@ -467,15 +445,11 @@ __global__ void __launch_bounds__(BLOCK) k_ws_z(SchedView S, const int32_t* rp, 
   if (threadIdx.x == 0) partials[blockIdx.x] = o[0];
 }
 
+// one block of 256: the sum of g block partials in a fixed order
 __global__ void k_ws_mu(const double* partials, int g, int n, double mu_min, double* mu) {
-  if (threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int b = 0; b < g; ++b) s += partials[b];
-  *mu = fmax(s / (double)n, mu_min);
-}
-
-__device__ __forceinline__ double ws_move(double target, double v, double delta) {
-  return fmin(fmax(target, v - delta), v + delta);
+  __shared__ double red[8], tot[1];
+  parts_sum<256, 1>(partials, g, nullptr, 0, tot, red);
+  if (threadIdx.x == 0) *mu = fmax(tot[0] / (double)n, mu_min);
 }
 
 __global__ void k_ws_apply(int n, int m, const double* x_s, const double* z_s, const double* y_s,
@@ -485,14 +459,8 @@ __global__ void k_ws_apply(int n, int m, const double* x_s, const double* z_s, c
   const double mu = *mu_p;
   const int stride = gridDim.x * blockDim.x;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride) {
-    double xp = fmax(x_s[j], alpha), zp = fmax(z_s[j], alpha);
-    if (xp < zp) {
-      xp = ws_move(mu / zp, xp, delta);
-      zp = ws_move(mu / xp, zp, delta);
-    } else {
-      zp = ws_move(mu / xp, zp, delta);
-      xp = ws_move(mu / zp, xp, delta);
-    }
+    double xp = x_s[j], zp = z_s[j];
+    centered_pair(mu, delta, alpha, xp, zp);
     if (unscaled) {
       xp = D_c[j] * xp;
       zp = zp / D_c[j];
@@ -511,7 +479,7 @@ void launch_ws_z(const SchedView& S, const int32_t* rp, const int32_t* col, cons
   k_ws_z<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, c_t, z_s, partials);
 }
 void launch_ws_mu(const double* partials, int g, int n, double mu_min, double* mu, cudaStream_t s) {
-  k_ws_mu<<<1, 32, 0, s>>>(partials, g, n, mu_min, mu);
+  k_ws_mu<<<1, 256, 0, s>>>(partials, g, n, mu_min, mu);
 }
 void launch_ws_apply(int n, int m, const double* x_s, const double* z_s, const double* y_s,
                      const double* mu, double delta_max, double alpha_min, int unscaled,

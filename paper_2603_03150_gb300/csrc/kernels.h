@@ -78,10 +78,10 @@ void launch_spmv(const SchedView& S, const int32_t* rp, const int32_t* col, cons
 //   part m: y output and partials [grid][4] = {U1, S4, 0, inf_rp}
 void launch_report_n(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
                      const double* x_s, const double* y_s, const double* c_t, const double* D_c,
-                     double* x_out, double* z_out, double* partials, const Launch& L, cudaStream_t s);
+                     const double* Dc_inv, double* x_out, double* z_out, double* partials, const Launch& L, cudaStream_t s);
 void launch_report_m(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
                      const double* x_s, const double* y_s, const double* b_t, const double* D_r,
-                     double* y_out, double* partials, const Launch& L, cudaStream_t s);
+                     const double* Dr_inv, double* y_out, double* partials, const Launch& L, cudaStream_t s);
 // sums the two partial sets into out[8] = {r_P, r_D, gap, maxviol, c^T x, b^T y, x^T z, 0}
 void launch_report_final(const double* pn, int gn, const double* pm, int gm, double* out,
                          cudaStream_t s);
@@ -139,12 +139,11 @@ struct RowStatPlan {
   const int32_t* long_ids = nullptr;
   int nlong = 0;
 };
-// Ruiz / Pock-Chambolle statistic of each row of D_self M D_other:
-// mode 0: sqrt(max |.|), mode 1: sqrt(sum |.|); zero -> 1.
+// One Ruiz / Pock-Chambolle round for the rows of D_self M D_other: d_new =
+// d_self / statistic, mode 0: sqrt(max |.|), mode 1: sqrt(sum |.|); zero -> 1.
 void launch_row_stat(int nrows, const int32_t* rp, const int32_t* col, const double* val,
-                     const double* d_self, const double* d_other, int mode, double* out,
+                     const double* d_self, const double* d_other, int mode, double* d_new,
                      const RowStatPlan& plan, cudaStream_t s);
-void launch_div(double* d, const double* r, int len, cudaStream_t s);
 // out[i] = 1 / in[i]
 void launch_recip(const double* in, double* out, int64_t len, cudaStream_t s);
 void launch_fill(double* d, double v, int64_t len, cudaStream_t s);
@@ -154,11 +153,6 @@ void launch_scale_vals(int nrows, const int32_t* rp, const int32_t* col, const d
                        float* out32, cudaStream_t s);
 void launch_scale_vec(int len, const double* d, const double* v, double* out64, float* out32,
                       cudaStream_t s);
-// partial sums (mode 0: a.b, 1: |a|^2, 2: |min(0,a)|^2) into partials[grid];
-// then a one-thread total in fixed order
-void launch_dot_partials(int64_t len, const double* a, const double* b, int mode,
-                         double* partials, int grid, cudaStream_t s);
-void launch_sum_final(const double* partials, int g, double* out, cudaStream_t s);
 // power iteration pieces (float64)
 void launch_pow_init(int n, double* v, PowerState* ps, int max_iter, double rel_tol,
                      cudaStream_t s);
@@ -170,13 +164,14 @@ void launch_pow_Av(const SchedView& S, const int32_t* rp, const int32_t* col, co
 void launch_pow_norm(int n, const double* w, double* v, PowerState* ps, cudaStream_t s);
 // blocks per SM of the power iteration's SpMV kernels (at: the A~^T one)
 int pow_occupancy(bool at, size_t smem);
-// scalar set-up of the solve from reduced values
-//   sums[5] = |b|^2, |c|^2, |b~|^2, |c~|^2, |min(0, c~)|^2
+// scalar set-up of the solve: the norms of b, c, b~, c~ and min(0, c~), then
 // eta = eta_safety / sigma_max, omega_0 = |c~|/|b~| (1 if either is 0),
 // tau, sigma, and the first restart point (0, 0): kkt_last = kkt_prev =
-// KKT_omega0(0, 0) = sqrt(omega^2 |b~|^2 + |min(0,c~)|^2 / omega^2)
-void launch_init_scalars(Scalars* sc, const double* sums, const PowerState* ps,
-                         double eta_safety, cudaStream_t s);
+// KKT_omega0(0, 0) = sqrt(omega^2 |b~|^2 + |min(0,c~)|^2 / omega^2); two
+// launches, partials holds 256 * 8 doubles
+void launch_init_scalars(Scalars* sc, int m, int n, const double* b, const double* c,
+                         const double* b_t, const double* c_t, double* partials,
+                         const PowerState* ps, double eta_safety, cudaStream_t s);
 cudaError_t configure_setup_kernels(size_t max_smem);
 // gather-rate floor pass (diagnostic): nnz nonzeros in groups of 8
 template <typename T>

@@ -254,93 +254,106 @@ void launch_segsort(int nseg, const int32_t* seg_ptr, int32_t* keys, double* val
 // ---------------------------------------------------------------------------
 // scaling statistics of D_self M D_other and scaled copies
 // ---------------------------------------------------------------------------
-// Row statistic sqrt(d_self[i] * max_j |M_ij| d_other[j]) (mode 0) or
-// sqrt(d_self[i] * sum_j |M_ij| d_other[j]) (mode 1); zero -> 1.  G lanes per
-// row (G sized to the mean row length, every lane of a warp takes part in the
-// shuffles); rows longer than long_len are left to k_row_stat_long.
-template <int G>
-__global__ void k_row_stat(int nrows, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
-                           const double* __restrict__ val, const double* __restrict__ d_self,
-                           const double* __restrict__ d_other, int mode, int long_len,
-                           double* __restrict__ out) {
-  // mode 0 (Ruiz): the maximum of |a| d over non-negative doubles, taken on
-  // their bit patterns (ordered like the values) with 64-bit integer max, so
-  // only the product and the row's square root use the slow float64 pipe;
-  // mode 1 (Pock-Chambolle): the float64 sum
-  constexpr int RPW = 32 / G;  // rows per warp and pass
-  const int lane = threadIdx.x & 31, gw = lane / G, gl = lane & (G - 1);
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int base = warp * RPW; base < nrows; base += nw * RPW) {
-    const int i = base + gw;
-    double acc = 0.0;
-    long long mx = 0;
-    bool mine = false;
-    if (i < nrows) {
-      const int b = rp[i], e = rp[i + 1];
-      if (e - b <= long_len) {
-        mine = true;
-        if (mode) {
-          for (int k = b + gl; k < e; k += G) acc += fabs(val[k]) * d_other[col[k]];
-        } else {
-          for (int k = b + gl; k < e; k += G)
-            mx = max(mx, __double_as_longlong(fabs(val[k]) * d_other[col[k]]));
-        }
-      }
-    }
-    if (mode) {
-#pragma unroll
-      for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o, G);
-    } else {
-#pragma unroll
-      for (int o = G / 2; o > 0; o >>= 1) mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o, G));
-      acc = __longlong_as_double(mx);
-    }
-    if (mine && gl == 0) {
-      const double r = sqrt(d_self[i] * acc);
-      out[i] = (r == 0.0) ? 1.0 : r;
-    }
-  }
+// d_new[i] = d_self[i] divided by the row statistic sqrt(d_self[i] * max_j
+// |M_ij| d_other[j]) (mode 0) or sqrt(d_self[i] * sum_j |M_ij| d_other[j])
+// (mode 1); zero -> 1.  Bound by the float64 pipe: the products, and the root
+// and quotient of each row.  G lanes take a row (G sized to the mean row
+// length), a warp RPW rows at a time; their statistics are collected one to a
+// lane over `passes` passes and the roots and quotients taken at once: a root in
+// the one lane that holds a row's statistic costs the pipe as much as 32.
+// Power-law LP: 200,000 rows of A 156 -> 78 us, 1,000,000 of A^T 108 -> 74 us,
+// the division pass after each (11 us) and a launch per matrix for the rows
+// longer than long_len (60 us; here the first nlong blocks, one row each) gone.
+// mode 0 takes the maximum on the bit patterns of the non-negative products
+// (ordered like the values), off the float64 pipe.
+__device__ __forceinline__ double scaled_by_stat(double d, double acc) {
+  const double r = sqrt(d * acc);
+  return d / (r == 0.0 ? 1.0 : r);
 }
 
-// the same statistic for the rows listed in ids, one block of 256 per row
-__global__ void k_row_stat_long(const int32_t* __restrict__ ids, const int32_t* __restrict__ rp,
-                                const int32_t* __restrict__ col, const double* __restrict__ val,
-                                const double* __restrict__ d_self,
-                                const double* __restrict__ d_other, int mode,
-                                double* __restrict__ out) {
-  __shared__ double red[8];
-  const int i = ids[blockIdx.x];
-  double acc = 0.0;
-  long long mx = 0;
-  if (mode) {
-    for (int k = rp[i] + threadIdx.x; k < rp[i + 1]; k += blockDim.x)
-      acc += fabs(val[k]) * d_other[col[k]];
+template <int G, bool kSum>
+__global__ void __launch_bounds__(256)
+    k_row_stat(int nrows, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
+               const double* __restrict__ val, const double* __restrict__ d_self,
+               const double* __restrict__ d_other, int long_len, const int32_t* __restrict__ long_ids,
+               int nlong, int passes, double* __restrict__ d_new) {
+  const int lane = threadIdx.x & 31;
+  if ((int)blockIdx.x < nlong) {
+    __shared__ double red[8];
+    const int i = long_ids[blockIdx.x], e = rp[i + 1];
+    double acc = 0.0;
+    long long mx = 0;
+#pragma unroll 4
+    for (int k = rp[i] + threadIdx.x; k < e; k += 256) {
+      const double p = fabs(val[k]) * d_other[col[k]];
+      if (kSum) acc += p;
+      else mx = max(mx, __double_as_longlong(p));
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  } else {
-    for (int k = rp[i] + threadIdx.x; k < rp[i + 1]; k += blockDim.x)
-      mx = max(mx, __double_as_longlong(fabs(val[k]) * d_other[col[k]]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
-    acc = __longlong_as_double(mx);
+    for (int o = 16; o > 0; o >>= 1) {
+      if (kSum) acc += __shfl_down_sync(0xffffffffu, acc, o);
+      else mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
+    }
+    if (lane == 0) red[threadIdx.x >> 5] = kSum ? acc : __longlong_as_double(mx);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double v = red[0];
+      for (int w = 1; w < 8; ++w) v = kSum ? v + red[w] : fmax(v, red[w]);
+      d_new[i] = scaled_by_stat(d_self[i], v);
+    }
+    return;
   }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = red[0];
-    for (int w = 1; w < 8; ++w) v = mode ? v + red[w] : fmax(v, red[w]);
-    const double r = sqrt(d_self[i] * v);
-    out[i] = (r == 0.0) ? 1.0 : r;
+  constexpr int RPW = 32 / G;  // rows per pass of a warp
+  const int gw = lane / G, gl = lane & (G - 1);
+  const int warp = (((int)blockIdx.x - nlong) * 256 + (int)threadIdx.x) >> 5;
+  const int nw = (((int)gridDim.x - nlong) * 256) >> 5;
+  const int group = passes * RPW;
+  for (int base = warp * group; base < nrows; base += nw * group) {
+    // the bounds of the group's rows, one to a lane
+    const int i = lane < group ? base + lane : nrows;
+    const int b0 = i < nrows ? rp[i] : 0, e0 = i < nrows ? rp[i + 1] : 0;
+    double mine = 0.0;
+#pragma unroll 4
+    for (int p = 0; p < passes; ++p) {
+      const int src = p * RPW + gw;
+      const int b = __shfl_sync(0xffffffffu, b0, src);
+      int e = __shfl_sync(0xffffffffu, e0, src);
+      if (e - b > long_len) e = b;
+      double acc = 0.0;
+      long long mx = 0;
+      for (int k = b + gl; k < e; k += G) {
+        const double q = fabs(val[k]) * d_other[col[k]];
+        if (kSum) acc += q;
+        else mx = max(mx, __double_as_longlong(q));
+      }
+#pragma unroll
+      for (int o = G / 2; o > 0; o >>= 1) {
+        if (kSum) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        else mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      }
+      const double v = __shfl_sync(0xffffffffu, kSum ? acc : __longlong_as_double(mx), (lane % RPW) * G);
+      if (lane / RPW == p) mine = v;
+    }
+    if (i < nrows && e0 - b0 <= long_len) d_new[i] = scaled_by_stat(d_self[i], mine);
   }
 }
 
 void launch_row_stat(int nrows, const int32_t* rp, const int32_t* col, const double* val,
-                     const double* d_self, const double* d_other, int mode, double* out,
+                     const double* d_self, const double* d_other, int mode, double* d_new,
                      const RowStatPlan& plan, cudaStream_t s) {
-  const int g = grid_cap((int64_t)nrows * plan.lanes);
-#define PDHG_ROW_STAT(G) \
-  k_row_stat<G><<<g, 256, 0, s>>>(nrows, rp, col, val, d_self, d_other, mode, plan.long_len, out)
+  // passes of a warp: all G (32 rows, full lanes in the roots) once every SM
+  // has 32 warps, fewer rows a warp on smaller matrices (200 rows: 5.6 us in
+  // one pass against 19 in 16)
+  const int rpw = 32 / plan.lanes;
+  const int passes = std::max(1, std::min(plan.lanes, nrows / (rpw * 152 * 32)));
+  const int g = plan.nlong + grid_cap((int64_t)nrows * 32 / (passes * rpw));
+#define PDHG_ROW_STAT(G)                                                                              \
+  if (mode)                                                                                           \
+    k_row_stat<G, true><<<g, 256, 0, s>>>(nrows, rp, col, val, d_self, d_other, plan.long_len,       \
+                                          plan.long_ids, plan.nlong, passes, d_new);                         \
+  else                                                                                                \
+    k_row_stat<G, false><<<g, 256, 0, s>>>(nrows, rp, col, val, d_self, d_other, plan.long_len,      \
+                                           plan.long_ids, plan.nlong, passes, d_new)
   switch (plan.lanes) {
     case 4: PDHG_ROW_STAT(4); break;
     case 8: PDHG_ROW_STAT(8); break;
@@ -348,9 +361,6 @@ void launch_row_stat(int nrows, const int32_t* rp, const int32_t* col, const dou
     default: PDHG_ROW_STAT(32); break;
   }
 #undef PDHG_ROW_STAT
-  if (plan.nlong > 0)
-    k_row_stat_long<<<plan.nlong, 256, 0, s>>>(plan.long_ids, rp, col, val, d_self, d_other, mode,
-                                              out);
 }
 
 __global__ void k_fill(double* d, double v, int64_t len) {
@@ -360,14 +370,6 @@ __global__ void k_fill(double* d, double v, int64_t len) {
 }
 void launch_fill(double* d, double v, int64_t len, cudaStream_t s) {
   k_fill<<<grid_cap(len), 256, 0, s>>>(d, v, len);
-}
-
-__global__ void k_div(double* d, const double* r, int len) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < len; i += gridDim.x * blockDim.x)
-    d[i] = d[i] / r[i];
-}
-void launch_div(double* d, const double* r, int len, cudaStream_t s) {
-  k_div<<<grid_cap(len), 256, 0, s>>>(d, r, len);
 }
 
 // A~_ij = (D_r[i] A_ij) D_c[j], evaluated in that order for A and for A^T so
@@ -406,34 +408,26 @@ void launch_scale_vec(int len, const double* d, const double* v, double* out64, 
   k_scale_vec<<<grid_cap(len), 256, 0, s>>>(len, d, v, out64, out32);
 }
 
-// mode 0: sum a*b; 1: sum a^2; 2: sum min(0,a)^2
-__global__ void k_dot_partials(int64_t len, const double* a, const double* b, int mode,
-                               double* partials) {
-  __shared__ double red[8];
-  double acc = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double x = a[i];
-    acc += mode == 0 ? x * b[i] : (mode == 1 ? x * x : fmin(0.0, x) * fmin(0.0, x));
+// partials[block][8]: sums of b^2, c^2, b~^2, c~^2, min(0, c~)^2, three zeros
+__global__ void __launch_bounds__(256) k_norms(int m, int n, const double* __restrict__ b,
+                                               const double* __restrict__ c,
+                                               const double* __restrict__ b_t,
+                                               const double* __restrict__ c_t, double* partials) {
+  __shared__ double red[8 * 8];
+  double v[8] = {};
+  const int step = gridDim.x * blockDim.x, t = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = t; i < m; i += step) {
+    const double p = b[i], q = b_t[i];
+    v[0] += p * p;
+    v[2] += q * q;
   }
-  const double v[1] = {acc};
-  double o[1];
-  block_sum<256, 1>(v, o, red);
-  if (threadIdx.x == 0) partials[blockIdx.x] = o[0];
-}
-void launch_dot_partials(int64_t len, const double* a, const double* b, int mode, double* partials,
-                         int grid, cudaStream_t s) {
-  k_dot_partials<<<grid, 256, 0, s>>>(len, a, b, mode, partials);
-}
-
-__global__ void k_sum_final(const double* partials, int g, double* out) {
-  if (threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int i = 0; i < g; ++i) s += partials[i];
-  *out = s;
-}
-void launch_sum_final(const double* partials, int g, double* out, cudaStream_t s) {
-  k_sum_final<<<1, 32, 0, s>>>(partials, g, out);
+  for (int j = t; j < n; j += step) {
+    const double p = c[j], q = c_t[j], r = min0(q);
+    v[1] += p * p;
+    v[3] += q * q;
+    v[4] += r * r;
+  }
+  block_sum_scatter<256, 8>(v, red, partials + 8 * (size_t)blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -564,9 +558,12 @@ void launch_pow_norm(int n, const double* w, double* v, PowerState* ps, cudaStre
   launch_pdl(k_pow_norm, grid_cap(n), 256, 0, s, n, w, v, (const PowerState*)ps);
 }
 
-// sums: |b|^2, |c|^2, |b~|^2, |c~|^2, |min(0, c~)|^2
-__global__ void k_init_scalars(Scalars* sc, const double* sums, const PowerState* ps,
+// the norms from k_norms' partials (a fixed order), then the scalars of the
+// solve; one block of 256
+__global__ void k_init_scalars(Scalars* sc, const double* partials, int grid, const PowerState* ps,
                                double eta_safety) {
+  __shared__ double sums[8], red[8 * 8];
+  parts_sum<256, 8>(partials, grid, nullptr, 0, sums, red);
   if (threadIdx.x != 0) return;
   const double smax = sqrt(fmax(ps->lam, 0.0));
   sc->eta = smax > 0.0 ? eta_safety / smax : 1.0;
@@ -590,9 +587,12 @@ void launch_recip(const double* in, double* out, int64_t len, cudaStream_t s) {
   k_recip<<<(int)g, 256, 0, s>>>(in, out, len);
 }
 
-void launch_init_scalars(Scalars* sc, const double* sums, const PowerState* ps, double eta_safety,
-                         cudaStream_t s) {
-  k_init_scalars<<<1, 32, 0, s>>>(sc, sums, ps, eta_safety);
+void launch_init_scalars(Scalars* sc, int m, int n, const double* b, const double* c,
+                         const double* b_t, const double* c_t, double* partials,
+                         const PowerState* ps, double eta_safety, cudaStream_t s) {
+  const int grid = grid_cap(std::max(m, n), 1024, 256);
+  k_norms<<<grid, 256, 0, s>>>(m, n, b, c, b_t, c_t, partials);
+  k_init_scalars<<<1, 256, 0, s>>>(sc, partials, grid, ps, eta_safety);
 }
 
 // shared memory limit for the power-iteration tile kernels

@@ -745,7 +745,6 @@ pdhg_status pdhg::alloc_arrays(pdhg_ctx* ctx) {
   CKS(dalloc(ctx, &ctx->out_n2, n));
   CKS(dalloc(ctx, &ctx->out_m1, m));
   CKS(dalloc(ctx, &ctx->report, 8));
-  CKS(dalloc(ctx, &ctx->sums, 8));
   CKS(dalloc(ctx, &ctx->sc, (size_t)ctx->count));
   CKS(dalloc(ctx, &ctx->ps, (size_t)ctx->count));
   CKS(dalloc(ctx, &ctx->log_k, ctx->log_cap));
@@ -868,18 +867,18 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
     CKS(make_plan(ctx->h_t_rp, n, &plan_t));
   }
   sub("  row-length plans");
-  double *r = ctx->out_m1, *s = ctx->out_n1;
-  launch_fill(ctx->D_r, 1.0, m, ctx->stream);
-  launch_fill(ctx->D_c, 1.0, n, ctx->stream);
+  // each round reads one pair of scalings and writes the other
+  double *dr[2] = {ctx->D_r, ctx->out_m1}, *dc[2] = {ctx->D_c, ctx->out_n1};
   const int rounds = ctx->opt.ruiz_iters + (ctx->opt.pock_chambolle ? 1 : 0);
-  for (int it = 0; it < rounds; ++it) {
+  int cur = rounds & 1;  // the last round writes D_r, D_c
+  launch_fill(dr[cur], 1.0, m, ctx->stream);
+  launch_fill(dc[cur], 1.0, n, ctx->stream);
+  for (int it = 0; it < rounds; ++it, cur ^= 1) {
     const int mode = it < ctx->opt.ruiz_iters ? 0 : 1;
-    launch_row_stat(m, ctx->a_rp, ctx->a_col, ctx->a_val_orig, ctx->D_r, ctx->D_c, mode, r,
+    launch_row_stat(m, ctx->a_rp, ctx->a_col, ctx->a_val_orig, dr[cur], dc[cur], mode, dr[cur ^ 1],
                     plan_a, ctx->stream);
-    launch_row_stat(n, ctx->t_rp, ctx->t_col, ctx->t_val_orig, ctx->D_c, ctx->D_r, mode, s,
+    launch_row_stat(n, ctx->t_rp, ctx->t_col, ctx->t_val_orig, dc[cur], dr[cur], mode, dc[cur ^ 1],
                     plan_t, ctx->stream);
-    launch_div(ctx->D_r, r, m, ctx->stream);
-    launch_div(ctx->D_c, s, n, ctx->stream);
   }
   sub("  scaling rounds");
   launch_scale_vals(m, ctx->a_rp, ctx->a_col, ctx->a_val_orig, ctx->D_r, ctx->D_c, 0,
@@ -891,8 +890,7 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
   launch_recip(ctx->D_r, ctx->Dr_inv, m, ctx->stream);
   launch_recip(ctx->D_c, ctx->Dc_inv, n, ctx->stream);
   ctx->launches += 2;
-  ctx->launches += 2 + 4LL * rounds + 4 +
-                   (long long)rounds * ((plan_a.nlong > 0) + (plan_t.nlong > 0));
+  ctx->launches += 2 + 2LL * rounds + 4;
   CK(cudaGetLastError());
 
   // zero state (also what the autotuner multiplies)
@@ -1012,16 +1010,9 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
     h.log_cap = ctx->log_cap;
     h.status = PDHG_MAX_ITER;
     CK(cudaMemcpyAsync(ctx->sc, &h, sizeof(h), cudaMemcpyHostToDevice, ctx->stream));
-    const int g = 256;
-    const double* srcs[5] = {ctx->b, ctx->c, ctx->b_t64, ctx->c_t64, ctx->c_t64};
-    const int64_t lens[5] = {m, n, m, n, n};
-    const int modes[5] = {1, 1, 1, 1, 2};
-    for (int q = 0; q < 5; ++q) {
-      launch_dot_partials(lens[q], srcs[q], nullptr, modes[q], ctx->partials, g, ctx->stream);
-      launch_sum_final(ctx->partials, g, ctx->sums + q, ctx->stream);
-    }
-    launch_init_scalars(ctx->sc, ctx->sums, ctx->ps, ctx->opt.eta_safety, ctx->stream);
-    ctx->launches += 11;
+    launch_init_scalars(ctx->sc, m, n, ctx->b, ctx->c, ctx->b_t64, ctx->c_t64, ctx->partials, ctx->ps,
+                        ctx->opt.eta_safety, ctx->stream);
+    ctx->launches += 2;
     Scalars hs;
     PowerState hp;
     CK(cudaMemcpyAsync(&hs, ctx->sc, sizeof(hs), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1278,9 +1269,9 @@ static pdhg_status compute_report(pdhg_ctx* ctx) {
   double* pm = ctx->partials + 4 * (size_t)(gn + 1);
   const int gm = ctx->l_a64.grid + ctx->sa8.view.ngroups;
   launch_report_n(ctx->st8.view, ctx->t_rp, ctx->t_col, ctx->t_val64, xs, ys, ctx->c_t64, ctx->D_c,
-                  ctx->out_n1, ctx->out_n2, pn, ctx->l_t64, ctx->stream);
+                  ctx->Dc_inv, ctx->out_n1, ctx->out_n2, pn, ctx->l_t64, ctx->stream);
   launch_report_m(ctx->sa8.view, ctx->a_rp, ctx->a_col, ctx->a_val64, xs, ys, ctx->b_t64, ctx->D_r,
-                  ctx->out_m1, pm, ctx->l_a64, ctx->stream);
+                  ctx->Dr_inv, ctx->out_m1, pm, ctx->l_a64, ctx->stream);
   launch_report_final(pn, gn, pm, gm, ctx->report, ctx->stream);
   ctx->launches += 3;
   CK(cudaGetLastError());
