@@ -20,7 +20,7 @@ LIBPATH = os.path.join(LIBDIR, "libpdhg.so")
 
 SOURCES = ["setup_kernels.cu", "iter_kernels.cu", "halpern.cu", "adaptive.cu", "solver.cu", "noalloc.cu",
            "batch.cu", "adjoint.cu", "diag.cu", "panel.cu", "resident.cu",
-           "resident_f32.cu", "resident_f64.cu", "resident_cg.cu"]
+           "resident_f32.cu", "resident_f64.cu", "resident_cg.cu", "slices.cu"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O3",

@@ -27,7 +27,7 @@
 // sums do not depend on the order in which blocks finish.
 #include "dispatch.cuh"
 #include "kernels.h"
-#include "spmv_tile.cuh"
+#include "spmv_slice.cuh"
 
 namespace pdhg {
 
@@ -210,11 +210,11 @@ __global__ void k_adapt_revert(IterBuffers<T> B) {
 
 template <typename T>
 void launch_adapt_primal(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_E(B.t_sched.e, launch_pdl(k_aprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(B.t_sched.e, launch_pdl(k_aprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_adapt_dual(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_E(B.a_sched.e, launch_pdl(k_adual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(B.a_sched.e, launch_pdl(k_adual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_adapt_revert(const IterBuffers<T>& B, int grid, cudaStream_t s) {
@@ -244,7 +244,8 @@ cudaError_t configure_adaptive_kernels(size_t max_smem) {
   cudaError_t e = cudaSuccess;
   for (int w = 0; w < 4; ++w)
     for (const void* f : {adaptive_kernel<8>(w), adaptive_kernel<16>(w), adaptive_kernel<32>(w),
-                          adaptive_kernel<-4>(w), adaptive_kernel<-8>(w)}) {
+                          adaptive_kernel<-4>(w), adaptive_kernel<-8>(w),
+                          adaptive_kernel<kSliced>(w)}) {
       cudaError_t r = set_max_dyn_smem(f, max_smem);
       if (r != cudaSuccess) e = r;
     }
@@ -253,7 +254,7 @@ cudaError_t configure_adaptive_kernels(size_t max_smem) {
 
 int adaptive_occupancy(int which, int e, size_t smem) {
   const void* f = nullptr;
-  PDHG_DISPATCH_E(e, f = adaptive_kernel<E_>(which));
+  PDHG_DISPATCH_S(e, f = adaptive_kernel<E_>(which));
   int nb = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, kBlock, smem);
   return nb < 1 ? 1 : nb;

@@ -41,9 +41,24 @@ struct SchedView {
   int32_t tile_nnz;  // nonzero capacity of a tile (block * e - 4)
   int32_t max_rows;  // rows per tile at most
   int32_t ngroups;   // split groups (records appended after block partials)
-  int32_t e;         // nonzeros per thread (4, 8 or 16)
-  int32_t pad;
+  int32_t e;         // nonzeros per thread (8, 16 or 32), kSliced: slices
+  // slices (spmv_slice.cuh), a warp each; ntiles counts blocks of them
+  int32_t nslices;
+  const int4* slices;         // first element; steps, lanes, rows; place in slice_ord; first row of the window
+  const uint8_t* slice_ord;   // [window][max_rows]: row (in the window) at a position
+  const int32_t* slice_col;
+  const void* slice_val;
 };
+
+constexpr int kSliced = 64;       // SchedView::e of a sliced schedule
+constexpr int kSliceRows = 64;    // rows sorted together
+constexpr int kSliceShort = 24;   // a lane per row up to this many nonzeros
+constexpr int kSliceWarps = 8;    // per SM, or short rows take more lanes
+// Float32 half-steps: slices up to this many nonzeros (A~^T of the planted LP
+// 100,000 x 250,000 8.6 -> 6.9 us, of 20,000 x 50,000 5.2 -> 3.5), tiles above
+// (A~^T of the 2000 x 2000 transportation LP 24.8 us against 32.9).
+constexpr int kSliceMaxNnz32 = 1 << 21;
+constexpr int kSliceMaxRow = 256; // 8 lanes per row up to this many; none longer
 
 // ---------------------------------------------------------------------------
 // Column-panel layout of one matrix (float32 iterations).  The columns are cut

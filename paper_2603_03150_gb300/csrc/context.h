@@ -10,7 +10,7 @@
 
 #include "kernels.h"
 #include "pdhg.h"
-#include "spmv_tile.cuh"
+#include "spmv_slice.cuh"
 
 namespace pdhg {
 void set_error(const char* fmt, ...);
@@ -60,6 +60,7 @@ struct DevSched {
   int32_t* counters = nullptr;
   double* slots = nullptr;
   uint32_t* wd = nullptr;
+  float* v32 = nullptr;  // sliced: the values in float32 (float32-mixed contexts)
   SchedView view{};
 };
 
@@ -106,6 +107,7 @@ struct pdhg_ctx {
   double *a_val_orig = nullptr, *t_val_orig = nullptr, *a_val64 = nullptr, *t_val64 = nullptr;
   float *a_val32 = nullptr, *t_val32 = nullptr;
   std::vector<int32_t> h_a_rp, h_t_rp;
+  int longest_a = 0, longest_t = 0;  // nonzeros of the longest row of A / A^T
   // [A, A^T][E = 16, 32]: the tuner's other whole-row schedules, built on a
   // host thread while the GPU runs the power iteration (declared after the
   // row pointers they read, so an early destruction joins them first)
@@ -229,6 +231,8 @@ pdhg_status polling_resources(pdhg_ctx* ctx);
 // panels do not apply (float64, batches, or dense partial sums above about
 // twice the nonzeros); the device layout
 bool panel_shape(const pdhg_ctx* ctx, bool on_a, int* P, int* npanels, int pscap = 256);
+// the sliced schedule of A~ or A~^T (slices.cu): no row above kSliceMaxRow
+pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d);
 pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out);
 // batched solve from iteration k0 to max_iter in one cooperative launch
 // (PDHG_TIMEOUT if a grid barrier's bounded wait ran out)

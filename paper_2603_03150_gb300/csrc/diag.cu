@@ -2,7 +2,7 @@
 // half-step SpMVs, used to report how far the fused kernels sit from the cost of
 // their loads and gathers alone.
 #include "kernels.h"
-#include "spmv_tile.cuh"
+#include "spmv_slice.cuh"
 
 namespace pdhg {
 

@@ -4,7 +4,7 @@
 
 // SpMV variant of a schedule -> template instantiation: segmented with
 // E = 8, 16, 32 nonzeros per thread, or vector with 4 / 8 lanes per row
-// (E_ = -4, -8).
+// (E_ = -4, -8); PDHG_DISPATCH_S also the slices of single LPs.
 #define PDHG_DISPATCH_E(e, ...)                 \
   switch (e) {                                  \
     case -4: {                                  \
@@ -27,6 +27,23 @@
       constexpr int E_ = 8;                     \
       __VA_ARGS__;                              \
     } break;                                    \
+  }
+
+#define PDHG_DISPATCH_S(e, ...)                 \
+  if ((e) == kSliced) {                         \
+    constexpr int E_ = kSliced;                 \
+    __VA_ARGS__;                                \
+  } else {                                      \
+    PDHG_DISPATCH_E(e, __VA_ARGS__)             \
+  }
+// the float64 report, Algorithm 1 and power iteration: E = 8 tiles or slices
+#define PDHG_DISPATCH_FIXED(e, ...)             \
+  if ((e) == kSliced) {                         \
+    constexpr int E_ = kSliced;                 \
+    __VA_ARGS__;                                \
+  } else {                                      \
+    constexpr int E_ = kFixedE;                 \
+    __VA_ARGS__;                                \
   }
 
 namespace pdhg {

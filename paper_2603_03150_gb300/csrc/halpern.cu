@@ -14,7 +14,7 @@
 #include "dispatch.cuh"
 #include "epilogues.cuh"
 #include "kernels.h"
-#include "spmv_tile.cuh"
+#include "spmv_slice.cuh"
 
 namespace pdhg {
 
@@ -47,11 +47,11 @@ __global__ void __launch_bounds__(BLOCK) k_hdual(IterBuffers<T> B, int i) {
 
 template <typename T>
 void launch_hprimal(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_E(B.t_sched.e, launch_pdl(k_hprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(B.t_sched.e, launch_pdl(k_hprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_hdual(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_E(B.a_sched.e, launch_pdl(k_hdual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(B.a_sched.e, launch_pdl(k_hdual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template void launch_hprimal<float>(const IterBuffers<float>&, const Launch&, int, cudaStream_t);
 template void launch_hprimal<double>(const IterBuffers<double>&, const Launch&, int, cudaStream_t);
@@ -73,7 +73,8 @@ cudaError_t configure_halpern_kernels(size_t max_smem) {
   cudaError_t e = cudaSuccess;
   for (int w = 0; w < 4; ++w)
     for (const void* f : {halpern_kernel<8>(w), halpern_kernel<16>(w), halpern_kernel<32>(w),
-                          halpern_kernel<-4>(w), halpern_kernel<-8>(w)}) {
+                          halpern_kernel<-4>(w), halpern_kernel<-8>(w),
+                          halpern_kernel<kSliced>(w)}) {
       cudaError_t r = set_max_dyn_smem(f, max_smem);
       if (r != cudaSuccess) e = r;
     }
@@ -82,7 +83,7 @@ cudaError_t configure_halpern_kernels(size_t max_smem) {
 
 int halpern_occupancy(int which, int e, size_t smem) {
   const void* f = nullptr;
-  PDHG_DISPATCH_E(e, f = halpern_kernel<E_>(which));
+  PDHG_DISPATCH_S(e, f = halpern_kernel<E_>(which));
   int nb = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, kBlock, smem);
   return nb < 1 ? 1 : nb;

@@ -8,7 +8,7 @@
 #include "epilogues.cuh"
 #include "eval_rule.cuh"
 #include "kernels.h"
-#include "spmv_tile.cuh"
+#include "spmv_slice.cuh"
 
 namespace pdhg {
 
@@ -191,15 +191,15 @@ __global__ void k_restart(IterBuffers<T> B) {
 
 template <typename T>
 void launch_primal(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_E(B.t_sched.e, launch_pdl(k_primal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(B.t_sched.e, launch_pdl(k_primal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_dual(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_E(B.a_sched.e, launch_pdl(k_dual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(B.a_sched.e, launch_pdl(k_dual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_eval(const IterBuffers<T>& B, const Launch& L, int chunk, cudaStream_t s) {
-  PDHG_DISPATCH_E(B.t_sched.e, k_eval<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(B, chunk));
+  PDHG_DISPATCH_S(B.t_sched.e, k_eval<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(B, chunk));
 }
 template <typename T>
 void launch_restart(const IterBuffers<T>& B, int grid, cudaStream_t s) {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(BLOCK) k_spmv(SchedView S, const int32_t* rp, 
 template <typename T>
 void launch_spmv(const SchedView& S, const int32_t* rp, const int32_t* col, const T* val,
                  const T* v, T* out, const Launch& L, cudaStream_t s) {
-  PDHG_DISPATCH_E(S.e, k_spmv<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, v, out));
+  PDHG_DISPATCH_S(S.e, k_spmv<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, v, out));
 }
 
 // ---------------------------------------------------------------------------
@@ -275,7 +275,7 @@ __device__ __forceinline__ void report_record(double a, double b, double c, doub
   }
 }
 
-template <int BLOCK>
+template <int BLOCK, int E>
 __global__ void __launch_bounds__(BLOCK) k_report_n(SchedView S, const int32_t* rp, const int32_t* col,
                                                    const double* val, const double* x_s,
                                                    const double* y_s, const double* c_t,
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(BLOCK) k_report_n(SchedView S, const int32_t* 
   double* split_q = partials + 4 * (size_t)gridDim.x;
   ReportNEpi epi{x_s, c_t, D_c, Dc_inv, x_out, z_out, 0.0, 0.0, 0.0, 0.0, split_q};
   Gather<double, 1> g{{y_s}};
-  run_tiles<double, 1, BLOCK, kFixedE>(S, rp, col, val, g, epi, smem);
+  run_sched<double, 1, BLOCK, E>(S, rp, col, val, g, epi, smem);
   report_record<BLOCK>(epi.u2, epi.s3, epi.xz, epi.inf_rd, red, partials + 4 * (size_t)blockIdx.x);
 }
 
@@ -314,7 +314,7 @@ struct ReportMEpi {
   }
 };
 
-template <int BLOCK>
+template <int BLOCK, int E>
 __global__ void __launch_bounds__(BLOCK) k_report_m(SchedView S, const int32_t* rp, const int32_t* col,
                                                    const double* val, const double* x_s,
                                                    const double* y_s, const double* b_t,
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(BLOCK) k_report_m(SchedView S, const int32_t* 
   double* split_q = partials + 4 * (size_t)gridDim.x;
   ReportMEpi epi{y_s, b_t, D_r, Dr_inv, y_out, 0.0, 0.0, 0.0, split_q};
   Gather<double, 1> g{{x_s}};
-  run_tiles<double, 1, BLOCK, kFixedE>(S, rp, col, val, g, epi, smem);
+  run_sched<double, 1, BLOCK, E>(S, rp, col, val, g, epi, smem);
   report_record<BLOCK>(epi.u1, epi.s4, 0.0, epi.inf_rp, red, partials + 4 * (size_t)blockIdx.x);
 }
 
@@ -353,15 +353,16 @@ void launch_report_n(const SchedView& S, const int32_t* rp, const int32_t* col, 
                      const double* x_s, const double* y_s, const double* c_t, const double* D_c,
                      const double* Dc_inv, double* x_out, double* z_out, double* partials,
                      const Launch& L, cudaStream_t s) {
-  k_report_n<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, c_t, D_c, Dc_inv,
-                                                    x_out, z_out, partials, nullptr);
+  PDHG_DISPATCH_FIXED(S.e, k_report_n<kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(
+                               S, rp, col, val, x_s, y_s, c_t, D_c, Dc_inv, x_out, z_out, partials,
+                               nullptr));
 }
 void launch_report_m(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
                      const double* x_s, const double* y_s, const double* b_t, const double* D_r,
                      const double* Dr_inv, double* y_out, double* partials, const Launch& L,
                      cudaStream_t s) {
-  k_report_m<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, b_t, D_r, Dr_inv,
-                                                    y_out, partials, nullptr);
+  PDHG_DISPATCH_FIXED(S.e, k_report_m<kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(
+                               S, rp, col, val, x_s, y_s, b_t, D_r, Dr_inv, y_out, partials, nullptr));
 }
 void launch_report_final(const double* pn, int gn, const double* pm, int gm, double* out,
                          cudaStream_t s) {
@@ -401,12 +402,12 @@ void launch_fp64_check(const IterBuffers<T>& B, const Fp64Check& C, cudaStream_t
   k_fp64_prep<T><<<C.conv_grid, 256, 0, s>>>(B, C.xs, C.ys);
   double* pn = B.partials;
   double* pm = B.partials + 4 * (size_t)(C.gn + 1);
-  k_report_n<kBlock><<<C.Lt.grid, kBlock, C.Lt.smem, s>>>(C.St, B.t_rp, B.t_col, C.t_val, C.xs, C.ys,
-                                                          B.c_t64, B.D_c, B.Dc_inv, nullptr,
-                                                          nullptr, pn, B.sc);
-  k_report_m<kBlock><<<C.La.grid, kBlock, C.La.smem, s>>>(C.Sa, B.a_rp, B.a_col, C.a_val, C.xs, C.ys,
-                                                          B.b_t64, B.D_r, B.Dr_inv, nullptr, pm,
-                                                          B.sc);
+  PDHG_DISPATCH_FIXED(C.St.e, k_report_n<kBlock, E_><<<C.Lt.grid, kBlock, C.Lt.smem, s>>>(
+                                  C.St, B.t_rp, B.t_col, C.t_val, C.xs, C.ys, B.c_t64, B.D_c, B.Dc_inv,
+                                  nullptr, nullptr, pn, B.sc));
+  PDHG_DISPATCH_FIXED(C.Sa.e, k_report_m<kBlock, E_><<<C.La.grid, kBlock, C.La.smem, s>>>(
+                                  C.Sa, B.a_rp, B.a_col, C.a_val, C.xs, C.ys, B.b_t64, B.D_r, B.Dr_inv,
+                                  nullptr, pm, B.sc));
   k_fp64_final<<<1, 256, 0, s>>>(B.sc, pn, C.gn, pm, C.gm, B.log_k, B.log_flags, B.log_kkt);
 }
 template void launch_fp64_check<float>(const IterBuffers<float>&, const Fp64Check&, cudaStream_t);
@@ -429,7 +430,7 @@ struct WsEpi {
   }
 };
 
-template <int BLOCK>
+template <int BLOCK, int E>
 __global__ void __launch_bounds__(BLOCK) k_ws_z(SchedView S, const int32_t* rp, const int32_t* col,
                                                const double* val, const double* x_s,
                                                const double* y_s, const double* c_t, double* z_s,
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(BLOCK) k_ws_z(SchedView S, const int32_t* rp, 
   __shared__ double red[BLOCK / 32];
   WsEpi epi{x_s, c_t, z_s, 0.0, partials + gridDim.x};
   Gather<double, 1> g{{y_s}};
-  run_tiles<double, 1, BLOCK, kFixedE>(S, rp, col, val, g, epi, smem);
+  run_sched<double, 1, BLOCK, E>(S, rp, col, val, g, epi, smem);
   const double v[1] = {epi.xz};
   double o[1];
   block_sum<BLOCK, 1>(v, o, red);
@@ -476,7 +477,8 @@ __global__ void k_ws_apply(int n, int m, const double* x_s, const double* z_s, c
 void launch_ws_z(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
                  const double* x_s, const double* y_s, const double* c_t, double* z_s,
                  double* partials, const Launch& L, cudaStream_t s) {
-  k_ws_z<kBlock><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s, c_t, z_s, partials);
+  PDHG_DISPATCH_FIXED(S.e, k_ws_z<kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, x_s, y_s,
+                                                                             c_t, z_s, partials));
 }
 void launch_ws_mu(const double* partials, int g, int n, double mu_min, double* mu, cudaStream_t s) {
   k_ws_mu<<<1, 256, 0, s>>>(partials, g, n, mu_min, mu);
@@ -526,9 +528,10 @@ PDHG_INST(double)
 #undef PDHG_INST
 
 // shared memory of the tile kernels (NV vectors, precision, rows per tile,
-// schedule variant: e < 0 is the vector kernel)
+// schedule variant: e < 0 is the vector kernel, which stages its sums as the
+// slices do)
 size_t tile_smem(int nv, bool f32, int max_rows, int e) {
-  if (e < 0) {
+  if (e < 0 || e == kSliced) {
     if (nv == 1)
       return f32 ? tile_vec_smem_bytes<float, 1, kBlock>(max_rows)
                  : tile_vec_smem_bytes<double, 1, kBlock>(max_rows);
@@ -555,11 +558,12 @@ static const void* tile_kernel(int which) {
     default: return nullptr;
   }
 }
+template <int E>
 static const void* fixed_kernel(int which) {
   switch (which) {
-    case 0: return (const void*)k_report_n<kBlock>;
-    case 1: return (const void*)k_report_m<kBlock>;
-    case 2: return (const void*)k_ws_z<kBlock>;
+    case 0: return (const void*)k_report_n<kBlock, E>;
+    case 1: return (const void*)k_report_m<kBlock, E>;
+    case 2: return (const void*)k_ws_z<kBlock, E>;
     default: return nullptr;
   }
 }
@@ -569,14 +573,15 @@ cudaError_t configure_tile_kernels(size_t max_smem) {
   cudaError_t e = cudaSuccess;
   for (int w = 0; w < 8; ++w)
     for (const void* f : {tile_kernel<8>(w), tile_kernel<16>(w), tile_kernel<32>(w),
-                          tile_kernel<-4>(w), tile_kernel<-8>(w)}) {
+                          tile_kernel<-4>(w), tile_kernel<-8>(w), tile_kernel<kSliced>(w)}) {
       cudaError_t r = set_max_dyn_smem(f, max_smem);
       if (r != cudaSuccess) e = r;
     }
-  for (int w = 0; w < 3; ++w) {
-    cudaError_t r = set_max_dyn_smem(fixed_kernel(w), max_smem);
-    if (r != cudaSuccess) e = r;
-  }
+  for (int w = 0; w < 3; ++w)
+    for (const void* f : {fixed_kernel<kFixedE>(w), fixed_kernel<kSliced>(w)}) {
+      cudaError_t r = set_max_dyn_smem(f, max_smem);
+      if (r != cudaSuccess) e = r;
+    }
   return e;
 }
 
@@ -585,7 +590,9 @@ cudaError_t configure_tile_kernels(size_t max_smem) {
 int tile_occupancy(int which, int e, size_t smem) {
   const void* f = nullptr;
   if (which >= 8)
-    f = fixed_kernel(0);
+    f = e == kSliced ? fixed_kernel<kSliced>(0) : fixed_kernel<kFixedE>(0);
+  else if (e == kSliced)
+    f = tile_kernel<kSliced>(which);
   else if (e == 32)
     f = tile_kernel<32>(which);
   else if (e == -4)

@@ -5,7 +5,7 @@
 
 #include "dispatch.cuh"
 #include "kernels.h"
-#include "spmv_tile.cuh"
+#include "spmv_slice.cuh"
 
 namespace pdhg {
 
@@ -431,17 +431,18 @@ __global__ void __launch_bounds__(256) k_norms(int m, int n, const double* __res
 }
 
 // ---------------------------------------------------------------------------
-// power iteration on A~^T A~ (float64).  Its three kernels are launched with
-// programmatic dependent launch and wait on entry, so each launch is set up
-// while the previous kernel drains.
+// power iteration on A~^T A~ (float64): u = A~ v with v = w / |w| kept as w and
+// the factor, then w <- A~^T u in place with v . w and |w|^2.  Both kernels are
+// launched with programmatic dependent launch and wait on entry, so each launch
+// is set up while the previous kernel drains.
 // ---------------------------------------------------------------------------
-__global__ void k_pow_init(int n, double* v, PowerState* ps, int max_iter, double rel_tol) {
+__global__ void k_pow_init(int n, double* w, PowerState* ps, int max_iter, double rel_tol) {
   const double v0 = 1.0 / sqrt((double)n);
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) v[j] = v0;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) w[j] = v0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ps->lam = 0.0;
     ps->lam_prev = 0.0;
-    ps->inv_norm = 0.0;
+    ps->inv_norm = 1.0;
     ps->k = 0;
     ps->max_iter = max_iter;
     ps->stopped = (max_iter <= 0 || n == 0) ? 1 : 0;
@@ -449,63 +450,67 @@ __global__ void k_pow_init(int n, double* v, PowerState* ps, int max_iter, doubl
     ps->rel_tol = rel_tol;
   }
 }
-void launch_pow_init(int n, double* v, PowerState* ps, int max_iter, double rel_tol,
+void launch_pow_init(int n, double* w, PowerState* ps, int max_iter, double rel_tol,
                      cudaStream_t s) {
-  k_pow_init<<<grid_cap(n), 256, 0, s>>>(n, v, ps, max_iter, rel_tol);
+  k_pow_init<<<grid_cap(n), 256, 0, s>>>(n, w, ps, max_iter, rel_tol);
 }
 
-template <int BLOCK>
+struct PowAvEpi {
+  double* u;
+  double inv;
+  __device__ __forceinline__ void row(int r, const double (&s)[1], int) { u[r] = s[0] * inv; }
+};
+
+template <int BLOCK, int E>
 __global__ void __launch_bounds__(BLOCK) k_pow_Av(SchedView S, const int32_t* rp, const int32_t* col,
-                                                 const double* val, const double* v, double* u,
+                                                 const double* val, const double* w, double* u,
                                                  const PowerState* ps) {
   pdl_enter();
   if (ps->stopped) return;
   extern __shared__ __align__(16) unsigned char smem[];
-  struct E {
-    double* u;
-    __device__ void row(int r, const double (&s)[1], int) { u[r] = s[0]; }
-  } epi{u};
-  Gather<double, 1> g{{v}};
-  run_tiles<double, 1, BLOCK, kFixedE>(S, rp, col, val, g, epi, smem);
+  PowAvEpi epi{u, ps->inv_norm};
+  Gather<double, 1> g{{w}};
+  run_sched<double, 1, BLOCK, E>(S, rp, col, val, g, epi, smem);
 }
 
 struct PowEpi {
-  const double* v;
   double* w;
-  double lam, nw2;
+  double inv, lam, nw2;
   double* split_q;
+  __device__ __forceinline__ double load(int j) const { return w[j]; }
+  __device__ __forceinline__ void apply(int j, double old, double s) {
+    w[j] = s;
+    lam += (old * inv) * s;
+    nw2 += s * s;
+  }
   __device__ __forceinline__ void row(int j, const double (&s)[1], int group) {
-    w[j] = s[0];
     if (group < 0) {
-      lam += v[j] * s[0];
-      nw2 += s[0] * s[0];
+      apply(j, load(j), s[0]);
     } else {
-      split_q[2 * group] = v[j] * s[0];
+      const double v = w[j] * inv;
+      w[j] = s[0];
+      split_q[2 * group] = v * s[0];
       split_q[2 * group + 1] = s[0] * s[0];
     }
   }
 };
 
-template <int BLOCK>
+template <int BLOCK, int E>
 __global__ void __launch_bounds__(BLOCK) k_pow_ATu(SchedView S, const int32_t* rp, const int32_t* col,
-                                                  const double* val, const double* u,
-                                                  const double* v, double* w, double* partials,
-                                                  PowerState* ps, int ngroups) {
+                                                  const double* val, const double* u, double* w,
+                                                  double* partials, PowerState* ps, int ngroups) {
   pdl_enter();
   if (ps->stopped) return;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[2 * (BLOCK / 32)];
   __shared__ int is_last;
   double* split_q = partials + 2 * (size_t)gridDim.x;
-  PowEpi epi{v, w, 0.0, 0.0, split_q};
+  PowEpi epi{w, ps->inv_norm, 0.0, 0.0, split_q};
   Gather<double, 1> g{{u}};
-  run_tiles<double, 1, BLOCK, kFixedE>(S, rp, col, val, g, epi, smem);
-  const double vv[2] = {epi.lam, epi.nw2};
-  double o[2];
-  block_sum<BLOCK, 2>(vv, o, red);
+  run_sched<double, 1, BLOCK, E>(S, rp, col, val, g, epi, smem);
+  double vv[2] = {epi.lam, epi.nw2};
+  block_sum_scatter<BLOCK, 2>(vv, red, partials + 2 * (size_t)blockIdx.x);
   if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = o[0];
-    partials[2 * blockIdx.x + 1] = o[1];
     __threadfence();
     is_last = (atomicAdd(&ps->ticket, 1) == (int)gridDim.x - 1);
   }
@@ -531,31 +536,26 @@ __global__ void __launch_bounds__(BLOCK) k_pow_ATu(SchedView S, const int32_t* r
   if (ps->k >= ps->max_iter) ps->stopped = 1;
 }
 
-__global__ void k_pow_norm(int n, const double* w, double* v, const PowerState* ps) {
-  pdl_enter();
-  const double s = ps->inv_norm;
-  if (s == 0.0) return;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) v[j] = w[j] * s;
-}
-
 void launch_pow_Av(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
-                   const double* v, double* u, PowerState* ps, const Launch& L, cudaStream_t s) {
-  launch_pdl(k_pow_Av<kBlock>, L.grid, kBlock, L.smem, s, S, rp, col, val, v, u, (const PowerState*)ps);
+                   const double* w, double* u, PowerState* ps, const Launch& L, cudaStream_t s) {
+  PDHG_DISPATCH_FIXED(S.e, launch_pdl(k_pow_Av<kBlock, E_>, L.grid, kBlock, L.smem, s, S, rp, col, val, w,
+                                      u, (const PowerState*)ps));
 }
 void launch_pow_ATu(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
-                    const double* u, const double* v, double* w, double* partials,
-                    PowerState* ps, const Launch& L, cudaStream_t s) {
-  launch_pdl(k_pow_ATu<kBlock>, L.grid, kBlock, L.smem, s, S, rp, col, val, u, v, w, partials, ps,
-             (int)S.ngroups);
+                    const double* u, double* w, double* partials, PowerState* ps, const Launch& L,
+                    cudaStream_t s) {
+  PDHG_DISPATCH_FIXED(S.e, launch_pdl(k_pow_ATu<kBlock, E_>, L.grid, kBlock, L.smem, s, S, rp, col, val, u,
+                                      w, partials, ps, (int)S.ngroups));
 }
-int pow_occupancy(bool at, size_t smem) {
-  const void* f = at ? (const void*)k_pow_ATu<kBlock> : (const void*)k_pow_Av<kBlock>;
+template <int E>
+static const void* pow_kernel(bool at) {
+  return at ? (const void*)k_pow_ATu<kBlock, E> : (const void*)k_pow_Av<kBlock, E>;
+}
+int pow_occupancy(bool at, int e, size_t smem) {
+  const void* f = e == kSliced ? pow_kernel<kSliced>(at) : pow_kernel<kFixedE>(at);
   int nb = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, kBlock, smem);
   return nb < 1 ? 1 : nb;
-}
-void launch_pow_norm(int n, const double* w, double* v, PowerState* ps, cudaStream_t s) {
-  launch_pdl(k_pow_norm, grid_cap(n), 256, 0, s, n, w, v, (const PowerState*)ps);
 }
 
 // the norms from k_norms' partials (a fixed order), then the scalars of the
@@ -598,7 +598,8 @@ void launch_init_scalars(Scalars* sc, int m, int n, const double* b, const doubl
 // shared memory limit for the power-iteration tile kernels
 cudaError_t configure_setup_kernels(size_t max_smem) {
   cudaError_t e = cudaSuccess;
-  for (const void* f : {(const void*)k_pow_Av<kBlock>, (const void*)k_pow_ATu<kBlock>}) {
+  for (const void* f : {pow_kernel<kFixedE>(false), pow_kernel<kFixedE>(true), pow_kernel<kSliced>(false),
+        pow_kernel<kSliced>(true)}) {
     cudaFuncAttributes a;
     cudaError_t r = cudaFuncGetAttributes(&a, f);
     if (r == cudaSuccess)

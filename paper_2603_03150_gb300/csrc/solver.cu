@@ -195,6 +195,13 @@ Launch pdhg::make_launch(pdhg_ctx* ctx, int occ_kind, int e, size_t smem, int nt
 }
 
 
+// A matrix may be sliced (spmv_slice.cuh) from 2^16 nonzeros on where the LP is
+// not solved on chip, no row is long and no tile capacity is forced.
+static bool sliced(const pdhg_ctx* ctx, bool on_a) {
+  return !ctx->batch && !ctx->resident && ctx->opt.tile_nnz == 0 && ctx->nnz >= (1 << 16) &&
+         (on_a ? ctx->longest_a : ctx->longest_t) <= kSliceMaxRow;
+}
+
 // Float64 schedules (report, Algorithm 1, power iteration) and reduction
 // scratch sized for any iteration schedule the tuner may pick.
 static pdhg_status fixed_schedules(pdhg_ctx* ctx) {
@@ -208,14 +215,17 @@ static pdhg_status fixed_schedules(pdhg_ctx* ctx) {
     const bool on_a = which == 0;
     const std::vector<int32_t>& rp = on_a ? ctx->h_a_rp : ctx->h_t_rp;
     const int nrows = on_a ? ctx->m : ctx->n;
-    HostSched h = build_sched(rp.data(), nrows, kFixedE);
-    CKS(upload_sched(ctx, h, on_a ? &ctx->sa8 : &ctx->st8, on_a ? ctx->a_rp : ctx->t_rp));
-    for (int r = 0; r < nrows; ++r) long_rows += (rp[r + 1] - rp[r]) > cap_min;
+    DevSched* d = on_a ? &ctx->sa8 : &ctx->st8;
+    if (sliced(ctx, on_a)) CKS(build_slices(ctx, on_a, d));
+    if (d->view.e != kSliced)
+      CKS(upload_sched(ctx, build_sched(rp.data(), nrows, kFixedE), d, on_a ? ctx->a_rp : ctx->t_rp));
+    if ((on_a ? ctx->longest_a : ctx->longest_t) > cap_min)
+      for (int r = 0; r < nrows; ++r) long_rows += (rp[r + 1] - rp[r]) > cap_min;
   }
   const bool mx = ctx->mixed;
   const SchedView &A8 = ctx->sa8.view, &T8 = ctx->st8.view;
-  ctx->l_a64 = make_launch(ctx, 8, kFixedE, smem_for(2, mx, A8.max_rows, A8.e), A8.ntiles);
-  ctx->l_t64 = make_launch(ctx, 8, kFixedE, smem_for(2, mx, T8.max_rows, T8.e), T8.ntiles);
+  ctx->l_a64 = make_launch(ctx, 8, A8.e, smem_for(2, mx, A8.max_rows, A8.e), A8.ntiles);
+  ctx->l_t64 = make_launch(ctx, 8, T8.e, smem_for(2, mx, T8.max_rows, T8.e), T8.ntiles);
   ctx->restart_grid = std::max(1, std::min(ctx->nsm * 8, (std::max(ctx->m, ctx->n) + 255) / 256));
   // grids never exceed SMs x 8 resident blocks of 256 threads
   const int64_t gmax = std::max<int64_t>({(int64_t)ctx->nsm * 8, ctx->l_a64.grid, ctx->l_t64.grid, 4096});
@@ -507,13 +517,22 @@ static pdhg_status tune_schedules(pdhg_ctx* ctx) {
     } else {
       cands = {{8, 0}};
     }
+    // sliced: in float64 slices were the faster ones on every measured matrix;
+    // in float32 8 nonzeros per thread stays a candidate
+    const DevSched& fixed = on_a ? ctx->sa8 : ctx->st8;
+    if (fixed.view.e == kSliced) {
+      cands.clear();
+      if (mx) cands.push_back({8, 0});
+      if (!mx || (fixed.v32 && ctx->opt.autotune)) cands.push_back({kSliced, 0});
+    }
     DevSched best{};
     float best_ms = 1e30f;
     for (const auto& cand : cands) {
       const int e = cand.first;
       DevSched d;
-      if (e == kFixedE && cand.second == 0) {
-        d = on_a ? ctx->sa8 : ctx->st8;
+      if (e == fixed.view.e && cand.second == 0) {
+        d = fixed;
+        if (e == kSliced && mx) d.view.slice_val = d.v32;
       } else {
         std::future<HostSched>& pre = ctx->presched[which][e == 16 ? 0 : 1];
         HostSched h = (cand.second == 0 && (e == 16 || e == 32) && pre.valid())
@@ -845,13 +864,19 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
   RowStatPlan plan_a, plan_t;
   {
     constexpr int kLongRow = 1024;
-    auto make_plan = [&](const std::vector<int32_t>& rp, int nrows, RowStatPlan* pl) -> pdhg_status {
+    auto make_plan = [&](const std::vector<int32_t>& rp, int nrows, int* longest,
+                         RowStatPlan* pl) -> pdhg_status {
       const double mean = nrows > 0 ? (double)rp[nrows] / nrows : 0.0;
       pl->lanes = mean <= 6 ? 4 : mean <= 12 ? 8 : mean <= 24 ? 16 : 32;
       pl->long_len = kLongRow;
+      int32_t most = 0;
+      const int32_t* r = rp.data();
+      for (int i = 0; i < nrows; ++i) most = std::max(most, r[i + 1] - r[i]);
+      *longest = most;
       std::vector<int32_t> ids;
-      for (int i = 0; i < nrows; ++i)
-        if (rp[i + 1] - rp[i] > kLongRow) ids.push_back(i);
+      if (most > kLongRow)
+        for (int i = 0; i < nrows; ++i)
+          if (r[i + 1] - r[i] > kLongRow) ids.push_back(i);
       pl->nlong = (int)ids.size();
       if (!ids.empty()) {
         int32_t* d = nullptr;
@@ -863,8 +888,8 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
       }
       return PDHG_OK;
     };
-    CKS(make_plan(ctx->h_a_rp, m, &plan_a));
-    CKS(make_plan(ctx->h_t_rp, n, &plan_t));
+    CKS(make_plan(ctx->h_a_rp, m, &ctx->longest_a, &plan_a));
+    CKS(make_plan(ctx->h_t_rp, n, &ctx->longest_t, &plan_t));
   }
   sub("  row-length plans");
   // each round reads one pair of scalings and writes the other
@@ -939,12 +964,12 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
   CKS(prepare_matrix(ctx));
   stage("validate/transpose/scale");
 
+  CKS(resident_build(ctx));
+  stage("on-chip layout");
+
   // float64 schedules (the iteration schedules are tuned once the scalars exist)
   CKS(fixed_schedules(ctx));
   stage("float64 schedules");
-
-  CKS(resident_build(ctx));
-  stage("on-chip layout");
 
   // the tuner's E = 16 and E = 32 schedules are host work: build them on a
   // host thread while the GPU runs the power iteration
@@ -953,7 +978,9 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
       for (int q = 0; q < 2; ++q) {
         const int32_t* rp = which == 0 ? ctx->h_a_rp.data() : ctx->h_t_rp.data();
         const int nrows = which == 0 ? m : n;
-        if ((int64_t)rp[nrows] < (int64_t)kLongWindowRows * nrows) continue;  // not tried
+        if ((int64_t)rp[nrows] < (int64_t)kLongWindowRows * nrows ||
+            (which == 0 ? ctx->sa8 : ctx->st8).view.e == kSliced)
+          continue;  // not tried
         const int e = q == 0 ? 16 : 32;
         ctx->presched[which][q] = std::async(std::launch::async, [rp, nrows, e] {
           return build_sched(rp, nrows, e, nullptr, 1, 0);
@@ -965,22 +992,21 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
   if (ctx->resident) {
     CKS(resident_power(ctx));
   } else {
-    double *v = ctx->xs64, *u = ctx->ys64, *w = ctx->out_n2;
-    launch_pow_init(n, v, ctx->ps, ctx->opt.power_max_iter, ctx->opt.power_rel_tol, ctx->stream);
+    double *w = ctx->xs64, *u = ctx->ys64;
+    launch_pow_init(n, w, ctx->ps, ctx->opt.power_max_iter, ctx->opt.power_rel_tol, ctx->stream);
     ctx->launches += 1;
     // grids from the power kernels' own occupancy (the float64 report
     // kernel's, which l_a64 / l_t64 follow, holds more registers)
-    const Launch la{std::max(1, std::min(ctx->sa8.view.ntiles, ctx->nsm * pow_occupancy(false, ctx->l_a64.smem))),
+    const SchedView &A8 = ctx->sa8.view, &T8 = ctx->st8.view;
+    const Launch la{std::max(1, std::min(A8.ntiles, ctx->nsm * pow_occupancy(false, A8.e, ctx->l_a64.smem))),
                     ctx->l_a64.smem};
-    const Launch lt{std::max(1, std::min(ctx->st8.view.ntiles, ctx->nsm * pow_occupancy(true, ctx->l_t64.smem))),
+    const Launch lt{std::max(1, std::min(T8.ntiles, ctx->nsm * pow_occupancy(true, T8.e, ctx->l_t64.smem))),
                     ctx->l_t64.smem};
     for (int it = 0; it < ctx->opt.power_max_iter; ++it) {
-      launch_pow_Av(ctx->sa8.view, ctx->a_rp, ctx->a_col, ctx->a_val64, v, u, ctx->ps, la,
-                    ctx->stream);
-      launch_pow_ATu(ctx->st8.view, ctx->t_rp, ctx->t_col, ctx->t_val64, u, v, w, ctx->partials,
-                     ctx->ps, lt, ctx->stream);
-      launch_pow_norm(n, w, v, ctx->ps, ctx->stream);
-      ctx->launches += 3;
+      launch_pow_Av(A8, ctx->a_rp, ctx->a_col, ctx->a_val64, w, u, ctx->ps, la, ctx->stream);
+      launch_pow_ATu(T8, ctx->t_rp, ctx->t_col, ctx->t_val64, u, w, ctx->partials, ctx->ps, lt,
+                     ctx->stream);
+      ctx->launches += 2;
       if ((it & 15) == 15) {
         PowerState hp;
         CK(cudaMemcpyAsync(&hp, ctx->ps, sizeof(hp), cudaMemcpyDeviceToHost, ctx->stream));

@@ -482,19 +482,6 @@ __device__ __forceinline__ void run_tiles_vec(const SchedView& S, const int32_t*
   }
 }
 
-// Schedule variant V: V > 0 segmented with E = V nonzeros per thread,
-// V < 0 vector with G = -V lanes per row.
-template <typename T, int NV, int BLOCK, int V, class Epi, class Gv>
-__device__ __forceinline__ void run_sched(const SchedView& S, const int32_t* __restrict__ row_ptr,
-                                          const int32_t* __restrict__ col,
-                                          const T* __restrict__ val, const Gv& g,
-                                          Epi& epi, unsigned char* smem) {
-  if constexpr (V > 0)
-    run_tiles<T, NV, BLOCK, V>(S, row_ptr, col, val, g, epi, smem);
-  else
-    run_tiles_vec<T, NV, BLOCK, -V>(S, row_ptr, col, val, g, epi, smem);
-}
-
 // Shared memory of run_tiles_vec (staged row sums, split-tile block sums).
 template <typename T, int NV, int BLOCK>
 __host__ __device__ constexpr size_t tile_vec_smem_bytes(int max_rows) {

@@ -1,0 +1,96 @@
+"""Large matrices without long rows in slices (a warp per slice of up to 32 rows
+sorted in windows of 64) against the tile kernels, which a forced tile capacity
+asks for: rows at the edges of the classes (24, 48 or 96 nonzeros with 1, 2 or 4
+lanes per short row, 256 the longest), empty rows, last windows of 1 row, tails
+of 0 to 3 steps; and matrices that keep the tiles.
+
+Tolerances as in the other parity tests: float64 states 1e-9 relative in the
+infinity norm (the sums run in another order, about 1e-15 per product, over 100
+iterations of a nonexpansive map); float32-mixed states 1e-4.  The adaptive step
+feeds its sums back into the step length, which is no such map (two capacities of
+the tile kernels drift apart as fast): 10 attempts instead of 100."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+from paper_2603_03150_gb300 import build as B
+from paper_2603_03150_gb300 import lpgen
+from paper_2603_03150_gb300 import pdhg
+
+pytestmark = pytest.mark.gpu
+
+SLICED = 64
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    B.build()
+
+
+def rel_inf(a, b):
+    a, b = np.asarray(a, float), np.asarray(b, float)
+    return float(np.max(np.abs(a - b)) / max(1e-300, np.max(np.abs(b))))
+
+
+def rows_lp(lengths, n, seed):
+    """One row per entry of `lengths` at random columns, planted optimum."""
+    rng = np.random.default_rng(seed)
+    lengths = np.asarray(lengths)
+    m, nnz = lengths.size, int(lengths.sum())
+    ptr = np.concatenate([[0], np.cumsum(lengths)])
+    # distinct columns of a row: a random start and a stride coprime to n (n prime)
+    k = np.arange(nnz) - np.repeat(ptr[:-1], lengths)
+    start, stride = rng.integers(0, n, m), rng.integers(1, n, m)
+    cols = (np.repeat(start, lengths) + k * np.repeat(stride, lengths)) % n
+    A = sp.csr_matrix((rng.standard_normal(nnz), cols, ptr), shape=(m, n))
+    A.sort_indices()
+    x = rng.uniform(0.5, 2, n) * (rng.random(n) < 0.3)
+    z = np.where(x > 0, 0.0, rng.uniform(0.5, 2, n))
+    b, c = A @ x, A.T @ rng.standard_normal(m) + z
+    return lpgen.LP(m, n, A.indptr.astype(np.int32), A.indices.astype(np.int32), A.data, b, c)
+
+
+def lengths(m, seed):
+    """Runs of 32 equal lengths from the edges of every class, long ones rare."""
+    rng = np.random.default_rng(seed)
+    pool = [0, 1, 2, 3, 4, 5, 7, 8, 23, 24, 25, 47, 48, 49, 95, 96, 97, 255, 256]
+    p = np.array([1.0] * 16 + [0.5, 0.2, 0.2])
+    return np.repeat(rng.choice(pool, size=m // 32 + 1, p=p / p.sum()), 32)[:m]
+
+
+MAKERS = {  # 4, 2 and 1 lanes per short row of A; A^T's rows follow
+    "lanes_4": lambda: rows_lp(lengths(14017, 1), 10007, 1),
+    "lanes_2": lambda: rows_lp(lengths(20033, 2), 30011, 2),
+    "lanes_1": lambda: rows_lp(lengths(44993, 3), 60013, 3),
+    "planted": lambda: lpgen.planted_lp(33_001, 82_507, seed=5),
+}
+
+
+@pytest.mark.parametrize("method,precision,tol", [
+    (q, *p) for q in ("averaged", "halpern", "adaptive") for p in (("fp64", 1e-9), ("fp32", 1e-4))])
+@pytest.mark.parametrize("name", list(MAKERS))
+def test_states_match_the_tile_kernels(name, precision, tol, method):
+    lp = MAKERS[name]()
+    kw, iters = dict(precision=precision), 10 if method == "adaptive" else 100
+    kw.update({"step_rule": "adaptive"} if method == "adaptive" else {"method": method})
+    with pdhg.Solver.from_lp(lp, **kw) as s, pdhg.Solver.from_lp(lp, tile_nnz=2044, **kw) as t:
+        if precision == "fp64":  # float32-mixed schedules are chosen by their measured times
+            assert s.schedule()["a_variant"] == s.schedule()["at_variant"] == SLICED
+        assert t.schedule()["a_variant"] != SLICED and t.schedule()["at_variant"] != SLICED
+        sa, sb = s.scaling()["sigma_max"], t.scaling()["sigma_max"]
+        assert abs(sa - sb) < 1e-12 * sb
+        for q in (s, t):
+            assert q.solve(0.0, iters) == pdhg.PDHG_MAX_ITER
+        a, b = s.state(), t.state()
+        for k in ("x", "y", "x_avg", "y_avg"):
+            assert rel_inf(a[k], b[k]) < tol, k
+
+
+@pytest.mark.parametrize("name,rows", [
+    ("too_long", np.r_[257, np.full(21000, 17)]),
+    ("too_ragged", np.where(np.arange(40000) % 64 == 0, 250, 4)),  # padded above 2 x
+])
+def test_matrices_that_keep_the_tiles(name, rows):
+    lp = rows_lp(rows, 30011, 4)
+    with pdhg.Solver.from_lp(lp) as s:
+        assert s.schedule()["a_variant"] != SLICED and s.schedule()["at_variant"] == SLICED
