@@ -154,6 +154,7 @@ struct Scalars {
   int32_t pad2;
   double avg_w;
   double eta_sum;
+  double step_pow[4];  // the attempt's (j+1)^-0.3 and (j+1)^-0.6, two attempts' pairs
   long long step_rejects;
 };
 

@@ -337,8 +337,7 @@ static void launch_dual_step(pdhg_ctx* ctx, const IterBuffers<T>& B, int i,
   if (between) cudaEventRecordWithFlags(between, ctx->stream, cudaEventRecordExternal);
 }
 // the half-steps a solve runs: the adaptive step's own kernels (its dual
-// half-step ends with the acceptance test of the attempt, then the undo of a rejected
-// one), else the above
+// half-step ends with the acceptance test of the attempt), else the above
 template <typename T>
 static void launch_prim_half(pdhg_ctx* ctx, const IterBuffers<T>& B, int i,
                              cudaEvent_t between = nullptr) {
@@ -352,16 +351,15 @@ static void launch_dual_half(pdhg_ctx* ctx, const IterBuffers<T>& B, int i,
   if (ctx->opt.step_rule != 1) return launch_dual_step<T>(ctx, B, i, between);
   launch_adapt_dual<T>(B, ctx->l_adual, i, ctx->stream);
   if (between) cudaEventRecordWithFlags(between, ctx->stream, cudaEventRecordExternal);
-  launch_adapt_revert<T>(B, ctx->restart_grid, ctx->stream);
 }
 static int prim_launches(const pdhg_ctx* ctx) { return ctx->pt.on ? 2 : 1; }
 static int dual_launches(const pdhg_ctx* ctx) { return ctx->pa.on ? 2 : 1; }
 // kernels of a chunk of `len` iterations: the half-steps, the evaluation, the
 // float64 check (float32-mixed) and the restart
 static long long chunk_launches(const pdhg_ctx* ctx, int len) {
-  // adaptive step: the two half-steps and the undo of a rejected attempt
-  const int per = ctx->opt.step_rule == 1 ? 3 : prim_launches(ctx) + dual_launches(ctx);
-  return (long long)per * len + 2 + (ctx->mixed ? kFp64CheckLaunches : 0);
+  // adaptive step: the undo of the last attempt
+  return (long long)(prim_launches(ctx) + dual_launches(ctx)) * len + 2 +
+         (ctx->opt.step_rule == 1 ? 1 : 0) + (ctx->mixed ? kFp64CheckLaunches : 0);
 }
 
 // what the float64 check of a float32-mixed candidate reads and writes
@@ -398,6 +396,7 @@ static void enqueue_chunk(pdhg_ctx* ctx, int len, cudaEvent_t* timing) {
     launch_dual_half<T>(ctx, B, i, sample ? timing[4] : nullptr);
     if (sample) cudaEventRecordWithFlags(timing[5], ctx->stream, cudaEventRecordExternal);
   }
+  if (ctx->opt.step_rule == 1) launch_adapt_revert<T>(B, ctx->restart_grid, ctx->stream);
   launch_eval<T>(B, ctx->l_eval, len, ctx->stream);
   if constexpr (sizeof(T) == 4) launch_fp64_check<T>(B, fp64_check_args(ctx), ctx->stream);
   launch_restart<T>(B, ctx->restart_grid, ctx->stream);
@@ -420,7 +419,7 @@ static void set_adaptive_launch(pdhg_ctx* ctx, bool on_a, const SchedView& S) {
   (on_a ? ctx->l_adual : ctx->l_aprim) = Launch{std::max(1, std::min(S.ntiles, ctx->nsm * occ)), sm};
 }
 static int half_launches(const pdhg_ctx* ctx, bool dual) {
-  if (ctx->opt.step_rule == 1) return dual ? 2 : 1;
+  if (ctx->opt.step_rule == 1) return 1;
   return dual ? dual_launches(ctx) : prim_launches(ctx);
 }
 
@@ -1689,7 +1688,7 @@ static pdhg_status time_kernels_impl(pdhg_ctx* ctx, int reps, double* ms) {
     if ((which == 3 && !(ctx->mixed && ctx->pt.on)) || (which == 4 && !(ctx->mixed && ctx->pa.on)))
       continue;
     const bool ad = ctx->opt.step_rule == 1;
-    const long long np = ad ? 1 : prim_launches(ctx), nd = ad ? 2 : dual_launches(ctx);
+    const long long np = ad ? 1 : prim_launches(ctx), nd = ad ? 1 : dual_launches(ctx);
     const long long per = which == 0 ? np : which == 1 ? nd : which == 2 ? np + nd : 1;
     ctx->launches += per * (warm + reps);
     for (int it = 0; it < warm + reps; ++it) {

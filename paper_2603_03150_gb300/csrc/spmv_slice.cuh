@@ -113,8 +113,10 @@ template <typename T, int NV, class Epi, class In>
 __device__ __forceinline__ void epi_apply(Epi& e, int r, const In& in, const T (&s)[NV]) {
   if constexpr (std::is_same<In, NoOperands>::value)
     e.row(r, s, -1);
-  else
+  else if constexpr (NV == 1)
     e.apply(r, in, s[0]);
+  else
+    e.apply(r, in, s);
 }
 
 template <typename T, int NV, int BLOCK, class Epi, class Gv>
