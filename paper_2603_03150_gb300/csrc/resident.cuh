@@ -403,31 +403,21 @@ struct ResExchange {
     for (int q = 0; q < NQ; ++q) red[q * kResThreads + threadIdx.x] = v[q];
     __syncthreads();
     if (warp < NQ) {
-      const double* mine = red + warp * kResThreads + lane;
-      double t[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        t[e] = mine[e * 32];
-#pragma unroll
-        for (int k = 1; k < kResWarps / 4; ++k) t[e] += mine[(e + 4 * k) * 32];
-      }
-      t[0] = (t[0] + t[1]) + (t[2] + t[3]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+      double t = block_share(red + warp * kResThreads + lane);
       const uint32_t bar = L.bar + 16u + 8u * slot;
       if (lane < C)
-        cl.send_to(lane, L.rec + (uint32_t)(slot * 2 * kResMaxC + warp * kResMaxC + cl.rank) * 8u, bar, t[0]);
+        cl.send_to(lane, L.rec + (uint32_t)(slot * 2 * kResMaxC + warp * kResMaxC + cl.rank) * 8u, bar, t);
       if (C > 1) {
         // the records of every CTA, in a tree
         wait(2 + slot);
         double r = lane < C ? rec[warp * kResMaxC + lane] : 0.0;
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-        t[0] = r;
+        t = r;
       }
       if (lane == 0) {
         double o[3];
-        fin(warp, t[0], o);
+        fin(warp, t, o);
         out[4 * warp] = o[0];
         out[4 * warp + 1] = o[1];
         out[4 * warp + 2] = o[2];
@@ -442,6 +432,63 @@ struct ResExchange {
       res[q][1] = out[4 * q + 1];
       res[q][2] = out[4 * q + 2];
     }
+  }
+  // The same in two parts: the last NQ warps add the CTA's shares and send them
+  // in sum_begin; in sum_end, later in the loop, they add the CTAs' and call fin
+  // (o[0..1]).  `slot` alternates between iterations, so a record is read before
+  // its slot is written again although a CTA may be an iteration ahead; `parity`
+  // is that of the slot's uses.  sum_end: whether a warp's wait ran out.
+  template <int NQ>
+  __device__ __forceinline__ void sum_begin(const double (&v)[NQ], int slot) {
+    const int lane = threadIdx.x & 31, q = (int)(threadIdx.x >> 5) - (kResWarps - NQ);
+    double* red = reinterpret_cast<double*>(smem + L.red);
+#pragma unroll
+    for (int e = 0; e < NQ; ++e) red[e * kResThreads + threadIdx.x] = v[e];
+    __syncthreads();
+    if (q < 0) return;
+    const double t = block_share(red + q * kResThreads + lane);
+    if (lane < C)
+      cl.send_to(lane, L.rec + (uint32_t)(slot * 2 * kResMaxC + q * kResMaxC + cl.rank) * 8u,
+                 L.bar + 16u + 8u * slot, t);
+  }
+  template <int NQ, class F>
+  __device__ __forceinline__ bool sum_end(int slot, uint32_t parity, double (&res)[NQ][2], F&& fin) {
+    const int lane = threadIdx.x & 31, q = (int)(threadIdx.x >> 5) - (kResWarps - NQ);
+    double* out = reinterpret_cast<double*>(smem + L.red) + 2 * kResThreads;
+    const double* rec = reinterpret_cast<const double*>(smem + L.rec) + slot * 2 * kResMaxC;
+    if (C > 1 && !lost) lost = !cl.arrived(L.bar + 16u + 8u * slot, parity, expect(2 + slot), wait_ns);
+    if (q >= 0) {
+      double r = lane < C ? rec[q * kResMaxC + lane] : 0.0;
+#pragma unroll
+      for (int o = C / 2; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+      if (lane == 0) {
+        double o[2];
+        fin(q, r, o);
+        out[4 * q] = o[0];
+        out[4 * q + 1] = o[1];
+      }
+    }
+    const bool ran_out = __syncthreads_or(lost);
+#pragma unroll
+    for (int e = 0; e < NQ; ++e) {
+      res[e][0] = out[4 * e];
+      res[e][1] = out[4 * e + 1];
+    }
+    return ran_out;
+  }
+  // the sum of 512 shares, 32 apart, of this lane and of its warp
+  __device__ __forceinline__ double block_share(const double* mine) const {
+    double t[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      t[e] = mine[e * 32];
+#pragma unroll
+      for (int k = 1; k < kResWarps / 4; ++k) t[e] += mine[(e + 4 * k) * 32];
+    }
+    t[0] = (t[0] + t[1]) + (t[2] + t[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+    return t[0];
   }
   // whether the loop ends, the same for all of the CTA's threads (after a lost
   // wait its warps may have read different sums)
