@@ -31,7 +31,7 @@ static __global__ void __launch_bounds__(256) k_res_sort(ResBuild B) {
   __shared__ int wsum[8];
   const int l = blockIdx.x >> 1, side = blockIdx.x & 1;
   ResLp& lp = B.lp[l];
-  const int N = side ? lp.n : lp.m, C = lp.C;
+  const int N = side ? lp.n : lp.m, C = lp.C, lg1 = side ? lp.lg_t : lp.lg_a, per = 32 >> lg1;
   const int64_t off = side ? lp.n_off : lp.m_off;
   const int32_t* rp = (side ? B.t_rp : B.a_rp) + off;
   uint16_t* ord = (side ? B.ord_n : B.ord_m) + off;
@@ -82,7 +82,7 @@ static __global__ void __launch_bounds__(256) k_res_sort(ResBuild B) {
     }
   }
   __syncthreads();
-  const int sL = n_long, sM = (n_mid + 3) / 4, n1 = N - n_long - n_mid, sS = (n1 + 31) / 32;
+  const int sL = n_long, sM = (n_mid + 3) / 4, n1 = N - n_long - n_mid, sS = (n1 + per - 1) / per;
   const int S = sL + sM + sS;
   for (int base = 0; base < S; base += 256) {
     const int s = base + tid;
@@ -97,11 +97,11 @@ static __global__ void __launch_bounds__(256) k_res_sort(ResBuild B) {
       } else if (s < sL + sM) {
         lg = 3, d.p0 = n_long + 4 * (s - sL), rows = min(4, n_long + n_mid - d.p0);
       } else {
-        lg = 0, d.p0 = n_long + n_mid + 32 * (s - sL - sM), rows = min(32, N - d.p0);
+        lg = lg1, d.p0 = n_long + n_mid + per * (s - sL - sM), rows = min(per, N - d.p0);
       }
       const int c1 = mine(min(s, sL)), c2 = mine(min(s, sL + sM)) - mine(min(s, sL)),
                 c3 = mine(s) - mine(min(s, sL + sM));
-      d.loc = c1 + 4 * c2 + 32 * c3;
+      d.loc = c1 + 4 * c2 + per * c3;
       const int i = ord[d.p0], len = rp[i + 1] - rp[i];  // the slice's longest row
       w = (len + (1 << lg) - 1) >> lg;
       d.wgr = w | (lg << 16) | (rows << 20);
@@ -429,7 +429,13 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
   };
   const std::vector<int> Cs = res_clusters(ctx, ops, ctx->mixed ? kResMinOps32 : kResMinOps64, fits);
   if (Cs.empty()) return PDHG_OK;
-  for (int l = 0; l < count; ++l) lps[l].C = Cs[l];
+  for (int l = 0; l < count; ++l) {
+    ResLp& q = lps[l];
+    const int64_t z = (int64_t)ctx->h_a_rp[q.m_off + q.m] - ctx->h_a_rp[q.m_off];
+    q.C = Cs[l];
+    q.lg_a = res_lanes(q.m, z, q.C);
+    q.lg_t = res_lanes(q.n, z, q.C);
+  }
   bool use[5] = {};
   // the cluster sizes the device runs (16 may not be available)
   for (int l = 0; l < count; ++l) use[(int)std::lround(std::log2(lps[l].C))] = true;

@@ -4,8 +4,8 @@
 //
 // Layout.  Each matrix of an LP (A~ and A~^T) is stored in slices of one warp:
 // the rows are sorted by length (longest first, stable, so the order is
-// fixed), rows of up to kResShort nonzeros go 32 to a slice (a lane each),
-// rows of up to kResMid 4 to a slice (8 lanes each), longer ones one to a
+// fixed), rows of up to kResShort nonzeros go 32 to a slice (a lane each; 16 or 8
+// in small LPs), rows of up to kResMid 4 to a slice (8 lanes each), longer ones one to a
 // slice.  Step k of a slice is 32 consecutive values and 16-bit columns, so
 // the loads coalesce and a row costs one fused multiply-add per nonzero and,
 // for the longer classes, the shuffle sum: GB300 runs 2 float64 operations per
@@ -59,7 +59,22 @@ struct ResLp {
   int32_t C;             // CTAs of its cluster
   int32_t a_slices, t_slices;
   int32_t own_m, own_n;  // slots of a CTA's own rows and columns (bounds)
+  int32_t lg_a, lg_t;    // log2 of the lanes of a short row of A~ / A~^T
 };
+
+// Lanes (log2) of a short row of a matrix whose slices are few: an iteration then
+// waits for the chains of dependent additions (68 clocks each), not for the
+// float64 pipe (a warp's operation takes 16 clocks of it).  Twice the lanes while
+// a CTA has less than 3 slices (it has less than 6 after) and a lane 6 nonzeros.
+// us per iteration with 1 / 2 / 4 lanes for the rows of A~ (12.5 nonzeros),
+// float64: 30 x 80 2.18 / 1.79 / 1.64, 60 x 150 2.38 / 1.94 / 2.11, 200 x 500
+// 2.55 / 2.14 / 2.16, 2000 x 5000 3.94 / 4.24 / 5.02; 2 lanes for the rows of
+// A~^T (5 nonzeros) 200 x 500 2.14 -> 2.20.
+__host__ inline int res_lanes(int rows, int64_t nnz, int C) {
+  int lg = 0;
+  while (lg < 2 && ((int64_t)rows << lg) <= 90LL * C && nnz >= ((int64_t)rows * 6 << lg)) ++lg;
+  return lg;
+}
 
 // Slots of one CTA's own rows of a matrix of `rows` rows: a class of slices
 // dealt to C CTAs gives a CTA at most one slice above the mean.
