@@ -153,14 +153,17 @@ void launch_scale_vals(int nrows, const int32_t* rp, const int32_t* col, const d
                        float* out32, cudaStream_t s);
 void launch_scale_vec(int len, const double* d, const double* v, double* out64, float* out32,
                       cudaStream_t s);
-// power iteration pieces (float64): w in place of v (v = w * ps->inv_norm)
+// power iteration pieces (float64): nparts block sums of the step before (0:
+// the first step) are added in launch_pow_Av, those of the last in launch_pow_end
 void launch_pow_init(int n, double* w, PowerState* ps, int max_iter, double rel_tol,
                      cudaStream_t s);
-void launch_pow_ATu(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
-                    const double* u, double* w, double* partials, PowerState* ps, const Launch& L,
-                    cudaStream_t s);
 void launch_pow_Av(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
-                   const double* w, double* u, PowerState* ps, const Launch& L, cudaStream_t s);
+                   const double* w, double* u, PowerState* ps, const double* partials, int nparts,
+                   const Launch& L, cudaStream_t s);
+void launch_pow_ATu(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
+                    const double* u, double* w, double* partials, const PowerState* ps, const Launch& L,
+                    cudaStream_t s);
+void launch_pow_end(PowerState* ps, const double* partials, int nparts, cudaStream_t s);
 // blocks per SM of the power iteration's SpMV kernels (at: the A~^T one)
 int pow_occupancy(bool at, int e, size_t smem);
 // scalar set-up of the solve: the norms of b, c, b~, c~ and min(0, c~), then

@@ -431,10 +431,13 @@ __global__ void __launch_bounds__(256) k_norms(int m, int n, const double* __res
 }
 
 // ---------------------------------------------------------------------------
-// power iteration on A~^T A~ (float64): u = A~ v with v = w / |w| kept as w and
-// the factor, then w <- A~^T u in place with v . w and |w|^2.  Both kernels are
-// launched with programmatic dependent launch and wait on entry, so each launch
-// is set up while the previous kernel drains.
+// power iteration on A~^T A~ (float64): u = A~ w, then w <- (A~^T u) / |w| in
+// place with v . w and |w|^2, v = w / |w| of the step before.  The factor is
+// applied a kernel late, so the last block of the next k_pow_Av adds a step's
+// block sums (loads, a tree, a root, two divisions: 4 us, the power-law LP's
+// steps 83 -> 79 us) while the others multiply.  Both kernels are launched with
+// programmatic dependent launch and wait on entry, so each launch is set up
+// while the previous kernel drains.
 // ---------------------------------------------------------------------------
 __global__ void k_pow_init(int n, double* w, PowerState* ps, int max_iter, double rel_tol) {
   const double v0 = 1.0 / sqrt((double)n);
@@ -457,18 +460,40 @@ void launch_pow_init(int n, double* w, PowerState* ps, int max_iter, double rel_
 
 struct PowAvEpi {
   double* u;
-  double inv;
-  __device__ __forceinline__ void row(int r, const double (&s)[1], int) { u[r] = s[0] * inv; }
+  __device__ __forceinline__ void row(int r, const double (&s)[1], int) { u[r] = s[0]; }
 };
+
+// ends the step whose nparts block sums are in `partials`; one block
+template <int BLOCK>
+__device__ __forceinline__ void pow_step(PowerState* ps, const double* partials, int nparts) {
+  __shared__ double red[2 * (BLOCK / 32)], tot[2];
+  parts_sum<BLOCK, 2>(partials, nparts, nullptr, 0, tot, red);
+  if (threadIdx.x != 0) return;
+  const double lam = tot[0], nw = sqrt(tot[1]);
+  ps->k += 1;
+  ps->lam = lam;
+  ps->inv_norm = nw == 0.0 ? 0.0 : 1.0 / nw;
+  bool stop = nw == 0.0 || ps->k >= ps->max_iter;
+  if (nw != 0.0) {
+    stop = stop || (ps->k > 1 && fabs(lam - ps->lam_prev) <= ps->rel_tol * lam);
+    ps->lam_prev = lam;
+  }
+  if (stop) ps->stopped = 1;
+}
+// the last step of power_max_iter
+__global__ void __launch_bounds__(256) k_pow_end(PowerState* ps, const double* partials, int nparts) {
+  if (!ps->stopped) pow_step<256>(ps, partials, nparts);
+}
 
 template <int BLOCK, int E>
 __global__ void __launch_bounds__(BLOCK) k_pow_Av(SchedView S, const int32_t* rp, const int32_t* col,
                                                  const double* val, const double* w, double* u,
-                                                 const PowerState* ps) {
+                                                 PowerState* ps, const double* partials, int nparts) {
   pdl_enter();
   if (ps->stopped) return;
+  if (nparts && blockIdx.x == gridDim.x - 1) pow_step<BLOCK>(ps, partials, nparts);
   extern __shared__ __align__(16) unsigned char smem[];
-  PowAvEpi epi{u, ps->inv_norm};
+  PowAvEpi epi{u};
   Gather<double, 1> g{{w}};
   run_sched<double, 1, BLOCK, E>(S, rp, col, val, g, epi, smem);
 }
@@ -479,18 +504,19 @@ struct PowEpi {
   double* split_q;
   __device__ __forceinline__ double load(int j) const { return w[j]; }
   __device__ __forceinline__ void apply(int j, double old, double s) {
-    w[j] = s;
-    lam += (old * inv) * s;
-    nw2 += s * s;
+    const double wn = s * inv;
+    w[j] = wn;
+    lam += (old * inv) * wn;
+    nw2 += wn * wn;
   }
   __device__ __forceinline__ void row(int j, const double (&s)[1], int group) {
     if (group < 0) {
       apply(j, load(j), s[0]);
     } else {
-      const double v = w[j] * inv;
-      w[j] = s[0];
-      split_q[2 * group] = v * s[0];
-      split_q[2 * group + 1] = s[0] * s[0];
+      const double v = w[j] * inv, wn = s[0] * inv;
+      w[j] = wn;
+      split_q[2 * group] = v * wn;
+      split_q[2 * group + 1] = wn * wn;
     }
   }
 };
@@ -498,54 +524,32 @@ struct PowEpi {
 template <int BLOCK, int E>
 __global__ void __launch_bounds__(BLOCK) k_pow_ATu(SchedView S, const int32_t* rp, const int32_t* col,
                                                   const double* val, const double* u, double* w,
-                                                  double* partials, PowerState* ps, int ngroups) {
+                                                  double* partials, const PowerState* ps) {
   pdl_enter();
   if (ps->stopped) return;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[2 * (BLOCK / 32)];
-  __shared__ int is_last;
-  double* split_q = partials + 2 * (size_t)gridDim.x;
-  PowEpi epi{w, ps->inv_norm, 0.0, 0.0, split_q};
+  PowEpi epi{w, ps->inv_norm, 0.0, 0.0, partials + 2 * (size_t)gridDim.x};
   Gather<double, 1> g{{u}};
   run_sched<double, 1, BLOCK, E>(S, rp, col, val, g, epi, smem);
   double vv[2] = {epi.lam, epi.nw2};
   block_sum_scatter<BLOCK, 2>(vv, red, partials + 2 * (size_t)blockIdx.x);
-  if (threadIdx.x == 0) {
-    __threadfence();
-    is_last = (atomicAdd(&ps->ticket, 1) == (int)gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  __shared__ double tot[2];
-  parts_sum<BLOCK, 2>(partials, (int)gridDim.x + ngroups, nullptr, 0, tot, red);
-  if (threadIdx.x != 0) return;
-  const double lam = tot[0], nw2 = tot[1];
-  ps->ticket = 0;
-  ps->k += 1;
-  ps->lam = lam;
-  const double nw = sqrt(nw2);
-  if (nw == 0.0) {
-    ps->stopped = 1;
-    ps->inv_norm = 0.0;
-    return;
-  }
-  ps->inv_norm = 1.0 / nw;
-  if (ps->k > 1 && fabs(lam - ps->lam_prev) <= ps->rel_tol * lam) ps->stopped = 1;
-  ps->lam_prev = lam;
-  if (ps->k >= ps->max_iter) ps->stopped = 1;
 }
 
 void launch_pow_Av(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
-                   const double* w, double* u, PowerState* ps, const Launch& L, cudaStream_t s) {
+                   const double* w, double* u, PowerState* ps, const double* partials, int nparts,
+                   const Launch& L, cudaStream_t s) {
   PDHG_DISPATCH_FIXED(S.e, launch_pdl(k_pow_Av<kBlock, E_>, L.grid, kBlock, L.smem, s, S, rp, col, val, w,
-                                      u, (const PowerState*)ps));
+                                      u, ps, partials, nparts));
 }
 void launch_pow_ATu(const SchedView& S, const int32_t* rp, const int32_t* col, const double* val,
-                    const double* u, double* w, double* partials, PowerState* ps, const Launch& L,
+                    const double* u, double* w, double* partials, const PowerState* ps, const Launch& L,
                     cudaStream_t s) {
   PDHG_DISPATCH_FIXED(S.e, launch_pdl(k_pow_ATu<kBlock, E_>, L.grid, kBlock, L.smem, s, S, rp, col, val, u,
-                                      w, partials, ps, (int)S.ngroups));
+                                      w, partials, ps));
+}
+void launch_pow_end(PowerState* ps, const double* partials, int nparts, cudaStream_t s) {
+  k_pow_end<<<1, 256, 0, s>>>(ps, partials, nparts);
 }
 template <int E>
 static const void* pow_kernel(bool at) {

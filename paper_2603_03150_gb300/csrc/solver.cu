@@ -1001,8 +1001,10 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
                     ctx->l_a64.smem};
     const Launch lt{std::max(1, std::min(T8.ntiles, ctx->nsm * pow_occupancy(true, T8.e, ctx->l_t64.smem))),
                     ctx->l_t64.smem};
+    const int nparts = lt.grid + T8.ngroups;
     for (int it = 0; it < ctx->opt.power_max_iter; ++it) {
-      launch_pow_Av(A8, ctx->a_rp, ctx->a_col, ctx->a_val64, w, u, ctx->ps, la, ctx->stream);
+      launch_pow_Av(A8, ctx->a_rp, ctx->a_col, ctx->a_val64, w, u, ctx->ps, ctx->partials,
+                    it ? nparts : 0, la, ctx->stream);
       launch_pow_ATu(T8, ctx->t_rp, ctx->t_col, ctx->t_val64, u, w, ctx->partials, ctx->ps, lt,
                      ctx->stream);
       ctx->launches += 2;
@@ -1013,6 +1015,8 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
         if (hp.stopped) break;
       }
     }
+    launch_pow_end(ctx->ps, ctx->partials, nparts, ctx->stream);
+    ctx->launches += 1;
     CK(cudaGetLastError());
   }
   stage("power iteration");
