@@ -116,12 +116,12 @@ void launch_convert_d2f(const double* src, float* dst, int64_t len, cudaStream_t
 void launch_convert_f2d(const float* src, double* dst, int64_t len, cudaStream_t s);
 
 // ---- setup (setup_kernels.cu) -------------------------------------------
-void launch_validate(int m, int n, const int32_t* rp, const int32_t* col, const double* val,
+void launch_validate(int m, int n, int64_t nnz, const int32_t* rp, const int32_t* col, const double* val,
                      const double* b, const double* c, int32_t* flags, cudaStream_t s);
 void launch_col_hist(int64_t nnz, const int32_t* col, int32_t* cnt, cudaStream_t s);
 // exclusive scan of cnt[len] into out[len+1]; tmp holds >= len/1024 + 2 ints
 void launch_scan(const int32_t* cnt, int32_t* out, int len, int32_t* tmp, cudaStream_t s);
-void launch_scatter(int m, const int32_t* rp, const int32_t* col, const double* val,
+void launch_scatter(int m, int64_t nnz, const int32_t* rp, const int32_t* col, const double* val,
                     int32_t* cursor, int32_t* col_t, double* val_t, cudaStream_t s);
 void launch_segsort(int nseg, const int32_t* seg_ptr, int32_t* keys, double* vals,
                     const int32_t* long_ids, int n_long, int32_t* tmp_k, double* tmp_v,
@@ -148,7 +148,7 @@ void launch_row_stat(int nrows, const int32_t* rp, const int32_t* col, const dou
 void launch_recip(const double* in, double* out, int64_t len, cudaStream_t s);
 void launch_fill(double* d, double v, int64_t len, cudaStream_t s);
 // A~_ij = (D_r[i] A_ij) D_c[j]; transposed = 1 when the rows are columns of A
-void launch_scale_vals(int nrows, const int32_t* rp, const int32_t* col, const double* val,
+void launch_scale_vals(int nrows, int64_t nnz, const int32_t* rp, const int32_t* col, const double* val,
                        const double* D_r, const double* D_c, int transposed, double* out64,
                        float* out32, cudaStream_t s);
 void launch_scale_vec(int len, const double* d, const double* v, double* out64, float* out32,

@@ -578,18 +578,12 @@ namespace {
 // cnt[p*R + i] = nonzeros of row i in panel p, src[.] = the first of them
 __global__ void k_pl_count(int R, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                            int P, int32_t* cnt, int32_t* src) {
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int i = warp; i < R; i += nw) {
-    const int s = rp[i], e = rp[i + 1];
-    for (int k = s + lane; k < e; k += 32) {
-      const int p = col[k] / P;
-      const int64_t f = (int64_t)p * R + i;
-      atomicAdd(cnt + f, 1);
-      if (k == s || col[k - 1] / P != p) src[f] = k;
-    }
-  }
+  each_nonzero(R, rp, [&](int k, int i) {
+    const int p = col[k] / P;
+    const int64_t f = (int64_t)p * R + i;
+    atomicAdd(cnt + f, 1);
+    if (k == rp[i] || col[k - 1] / P != p) src[f] = k;
+  });
 }
 
 __global__ void k_pl_flag(int64_t len, const int32_t* __restrict__ cnt, int32_t* flag) {
@@ -826,7 +820,7 @@ pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out) {
   auto count = [&](int P_, int np_) -> pdhg_status {
     const int64_t len_ = (int64_t)np_ * R;
     PL_CK(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * len_, s));
-    k_pl_count<<<grid_for((int64_t)R * 32), 256, 0, s>>>(R, rp, col, P_, cnt.p, src.p);
+    k_pl_count<<<grid_for(ctx->nnz / 8), 256, 0, s>>>(R, rp, col, P_, cnt.p, src.p);
     k_pl_flag<<<grid_for(len_), 256, 0, s>>>(len_, cnt.p, flag.p);
     launch_scan(flag.p, psidx.p, (int)len_, scan_tmp.p, s);
     k_pl_panel_first<<<(np_ + 256) / 256, 256, 0, s>>>(np_, R, psidx.p, pfirst.p);

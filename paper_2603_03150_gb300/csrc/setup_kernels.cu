@@ -21,19 +21,13 @@ static int grid_cap(int64_t work, int per_block = 256, int cap = 8192) {
 // ---------------------------------------------------------------------------
 __global__ void k_validate(int m, int n, const int32_t* rp, const int32_t* col, const double* val,
                            const double* b, const double* c, int32_t* flags) {
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
   int f = 0;
-  for (int i = warp; i < m; i += nw) {
-    const int s = rp[i], e = rp[i + 1];
-    for (int k = s + lane; k < e; k += 32) {
-      const int cj = col[k];
-      if (cj < 0 || cj >= n) f |= 1;
-      if (k > s && col[k - 1] >= cj) f |= 2;
-      if (!isfinite(val[k])) f |= 4;
-    }
-  }
+  each_nonzero(m, rp, [&](int k, int i) {
+    const int cj = col[k];
+    if (cj < 0 || cj >= n) f |= 1;
+    if (k > rp[i] && col[k - 1] >= cj) f |= 2;
+    if (!isfinite(val[k])) f |= 4;
+  });
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
   for (int i = tid; i < m; i += nt)
     if (!isfinite(b[i])) f |= 8;
@@ -42,9 +36,9 @@ __global__ void k_validate(int m, int n, const int32_t* rp, const int32_t* col, 
   if (f) atomicOr(flags, f);
 }
 
-void launch_validate(int m, int n, const int32_t* rp, const int32_t* col, const double* val,
+void launch_validate(int m, int n, int64_t nnz, const int32_t* rp, const int32_t* col, const double* val,
                      const double* b, const double* c, int32_t* flags, cudaStream_t s) {
-  k_validate<<<grid_cap((int64_t)m * 32), 256, 0, s>>>(m, n, rp, col, val, b, c, flags);
+  k_validate<<<grid_cap(std::max<int64_t>({nnz / 8, m, n})), 256, 0, s>>>(m, n, rp, col, val, b, c, flags);
 }
 
 // ---------------------------------------------------------------------------
@@ -152,19 +146,15 @@ void launch_scan(const int32_t* cnt, int32_t* out, int len, int32_t* tmp, cudaSt
 
 __global__ void k_scatter(int m, const int32_t* rp, const int32_t* col, const double* val,
                           int32_t* cursor, int32_t* col_t, double* val_t) {
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int i = warp; i < m; i += nw)
-    for (int k = rp[i] + lane; k < rp[i + 1]; k += 32) {
-      const int pos = atomicAdd(cursor + col[k], 1);
-      col_t[pos] = i;
-      val_t[pos] = val[k];
-    }
+  each_nonzero(m, rp, [&](int k, int i) {
+    const int pos = atomicAdd(cursor + col[k], 1);
+    col_t[pos] = i;
+    val_t[pos] = val[k];
+  });
 }
-void launch_scatter(int m, const int32_t* rp, const int32_t* col, const double* val,
+void launch_scatter(int m, int64_t nnz, const int32_t* rp, const int32_t* col, const double* val,
                     int32_t* cursor, int32_t* col_t, double* val_t, cudaStream_t s) {
-  k_scatter<<<grid_cap((int64_t)m * 32), 256, 0, s>>>(m, rp, col, val, cursor, col_t, val_t);
+  k_scatter<<<grid_cap(nnz / 8), 256, 0, s>>>(m, rp, col, val, cursor, col_t, val_t);
 }
 
 // segments of <= 32 entries: one thread, insertion sort in place
@@ -377,23 +367,18 @@ void launch_fill(double* d, double v, int64_t len, cudaStream_t s) {
 __global__ void k_scale_vals(int nrows, const int32_t* rp, const int32_t* col, const double* val,
                              const double* d_row, const double* d_col, int transposed,
                              double* out64, float* out32) {
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int i = warp; i < nrows; i += nw)
-    for (int k = rp[i] + lane; k < rp[i + 1]; k += 32) {
-      const double dr = transposed ? d_row[col[k]] : d_row[i];
-      const double dc = transposed ? d_col[i] : d_col[col[k]];
-      const double v = (dr * val[k]) * dc;
-      out64[k] = v;
-      if (out32) out32[k] = (float)v;
-    }
+  each_nonzero(nrows, rp, [&](int k, int i) {
+    const double dr = transposed ? d_row[col[k]] : d_row[i];
+    const double dc = transposed ? d_col[i] : d_col[col[k]];
+    const double v = (dr * val[k]) * dc;
+    out64[k] = v;
+    if (out32) out32[k] = (float)v;
+  });
 }
-void launch_scale_vals(int nrows, const int32_t* rp, const int32_t* col, const double* val,
+void launch_scale_vals(int nrows, int64_t nnz, const int32_t* rp, const int32_t* col, const double* val,
                        const double* D_r, const double* D_c, int transposed, double* out64,
                        float* out32, cudaStream_t s) {
-  k_scale_vals<<<grid_cap((int64_t)nrows * 32), 256, 0, s>>>(nrows, rp, col, val, D_r, D_c,
-                                                            transposed, out64, out32);
+  k_scale_vals<<<grid_cap(nnz / 8), 256, 0, s>>>(nrows, rp, col, val, D_r, D_c, transposed, out64, out32);
 }
 
 __global__ void k_scale_vec(int len, const double* d, const double* v, double* out64, float* out32) {

@@ -812,7 +812,7 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
   CKS(dalloc(ctx, &tmp, (size_t)n / 1024 + 8));
   // validation on device
   CK(cudaMemsetAsync(flags, 0, sizeof(int32_t), ctx->stream));
-  launch_validate(m, n, ctx->a_rp, ctx->a_col, ctx->a_val_orig, ctx->b, ctx->c, flags, ctx->stream);
+  launch_validate(m, n, nnz, ctx->a_rp, ctx->a_col, ctx->a_val_orig, ctx->b, ctx->c, flags, ctx->stream);
   ctx->launches += 1;
   int32_t hflags = 0;
   CK(cudaMemcpyAsync(&hflags, flags, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
@@ -830,7 +830,7 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
   launch_col_hist(nnz, ctx->a_col, cnt, ctx->stream);
   launch_scan(cnt, ctx->t_rp, n, tmp, ctx->stream);
   CK(cudaMemcpyAsync(cnt, ctx->t_rp, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream));
-  launch_scatter(m, ctx->a_rp, ctx->a_col, ctx->a_val_orig, cnt, ctx->t_col, ctx->t_val_orig,
+  launch_scatter(m, nnz, ctx->a_rp, ctx->a_col, ctx->a_val_orig, cnt, ctx->t_col, ctx->t_val_orig,
                  ctx->stream);
   ctx->launches += 1 + (n > 0 ? 3 : 0) + 1;  // histogram, scan, scatter
   ctx->h_t_rp.resize((size_t)n + 1);
@@ -905,9 +905,9 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
                     plan_t, ctx->stream);
   }
   sub("  scaling rounds");
-  launch_scale_vals(m, ctx->a_rp, ctx->a_col, ctx->a_val_orig, ctx->D_r, ctx->D_c, 0,
+  launch_scale_vals(m, nnz, ctx->a_rp, ctx->a_col, ctx->a_val_orig, ctx->D_r, ctx->D_c, 0,
                     ctx->a_val64, ctx->a_val32, ctx->stream);
-  launch_scale_vals(n, ctx->t_rp, ctx->t_col, ctx->t_val_orig, ctx->D_r, ctx->D_c, 1,
+  launch_scale_vals(n, nnz, ctx->t_rp, ctx->t_col, ctx->t_val_orig, ctx->D_r, ctx->D_c, 1,
                     ctx->t_val64, ctx->t_val32, ctx->stream);
   launch_scale_vec(m, ctx->D_r, ctx->b, ctx->b_t64, ctx->b_t32, ctx->stream);
   launch_scale_vec(n, ctx->D_c, ctx->c, ctx->c_t64, ctx->c_t32, ctx->stream);
