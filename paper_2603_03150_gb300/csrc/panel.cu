@@ -19,6 +19,7 @@
 // barrier follows the panel load, so 32 warps per SM run independently.
 #include <algorithm>
 #include <cstdio>
+#include <initializer_list>
 #include <vector>
 
 #include "context.h"
@@ -753,13 +754,31 @@ int grid_for(int64_t work, int per = 256, int cap = 16384) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, cap));
 }
 
-template <typename T>
-struct Tmp {  // device scratch freed with the object
-  T* p = nullptr;
-  ~Tmp() {
-    if (p) cudaFree(p);
+// Device scratch of several arrays, one allocation, freed with the object (an
+// allocation and its release took about 0.1 ms, and the release waits for the
+// GPU: 15 of them per matrix were 1.5 ms of a set-up).
+struct Scratch {
+  void* base = nullptr;
+  ~Scratch() {
+    if (base) cudaFree(base);
   }
-  cudaError_t alloc(size_t n) { return cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)); }
+  struct Part {
+    int32_t** p;
+    size_t n;
+  };
+  cudaError_t alloc(std::initializer_list<Part> parts) {
+    auto room = [](size_t n) { return (std::max<size_t>(n, 1) * sizeof(int32_t) + 255) & ~size_t(255); };
+    size_t total = 0;
+    for (const Part& q : parts) total += room(q.n);
+    cudaError_t e = cudaMalloc(&base, total);
+    if (e != cudaSuccess) return e;
+    char* at = static_cast<char*>(base);
+    for (const Part& q : parts) {
+      *q.p = reinterpret_cast<int32_t*>(at);
+      at += room(q.n);
+    }
+    return cudaSuccess;
+  }
 };
 
 }  // namespace
@@ -809,23 +828,20 @@ pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out) {
   const int pstride = (R + 3) & ~3;
 
   // pseudo-rows: counts per (panel, row), their prefix, the first of each panel
-  Tmp<int32_t> cnt, src, flag, psidx, scan_tmp, pfirst;
-  PL_CK(cnt.alloc(len));
-  PL_CK(src.alloc(len));
-  PL_CK(flag.alloc(len));
-  PL_CK(psidx.alloc(len + 1));
-  PL_CK(scan_tmp.alloc(len / 1024 + 2 + 1024));
-  PL_CK(pfirst.alloc(np + 1));
+  Scratch pseudo, segments, per_tile;
+  int32_t *cnt, *src, *flag, *psidx, *scan_tmp, *pfirst;
+  PL_CK(pseudo.alloc({{&cnt, (size_t)len}, {&src, (size_t)len}, {&flag, (size_t)len}, {&psidx, (size_t)len + 1},
+                      {&scan_tmp, (size_t)len / 1024 + 2 + 1024}, {&pfirst, (size_t)np + 1}}));
   std::vector<int32_t> h_pfirst;
   auto count = [&](int P_, int np_) -> pdhg_status {
     const int64_t len_ = (int64_t)np_ * R;
-    PL_CK(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * len_, s));
-    k_pl_count<<<grid_for(ctx->nnz / 8), 256, 0, s>>>(R, rp, col, P_, cnt.p, src.p);
-    k_pl_flag<<<grid_for(len_), 256, 0, s>>>(len_, cnt.p, flag.p);
-    launch_scan(flag.p, psidx.p, (int)len_, scan_tmp.p, s);
-    k_pl_panel_first<<<(np_ + 256) / 256, 256, 0, s>>>(np_, R, psidx.p, pfirst.p);
+    PL_CK(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * len_, s));
+    k_pl_count<<<grid_for(ctx->nnz / 8), 256, 0, s>>>(R, rp, col, P_, cnt, src);
+    k_pl_flag<<<grid_for(len_), 256, 0, s>>>(len_, cnt, flag);
+    launch_scan(flag, psidx, (int)len_, scan_tmp, s);
+    k_pl_panel_first<<<(np_ + 256) / 256, 256, 0, s>>>(np_, R, psidx, pfirst);
     h_pfirst.assign(np_ + 1, 0);
-    PL_CK(cudaMemcpyAsync(h_pfirst.data(), pfirst.p, sizeof(int32_t) * (np_ + 1),
+    PL_CK(cudaMemcpyAsync(h_pfirst.data(), pfirst, sizeof(int32_t) * (np_ + 1),
                           cudaMemcpyDeviceToHost, s));
     PL_CK(cudaStreamSynchronize(s));
     ctx->launches += 6;
@@ -846,12 +862,6 @@ pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out) {
   }
   const int nps = h_pfirst[np];
   CKS(dalloc(ctx, &out->psrow, (size_t)nps + 16));  // spare: prefetches round up to 16 bytes
-  Tmp<int32_t> pslen, pssrc;
-  PL_CK(pslen.alloc(nps));
-  PL_CK(pssrc.alloc(nps));
-  k_pl_compact<<<grid_for(len), 256, 0, s>>>(len, R, cnt.p, src.p, psidx.p, out->psrow, pslen.p,
-                                             pssrc.p);
-
   // segments of at most kPackSeg pseudo-rows within a panel, packed in parallel
   constexpr int kSeg = kPackSeg;
   std::vector<int2> h_segs;
@@ -862,38 +872,36 @@ pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out) {
       h_seg_panel.push_back(p);
     }
   const int nseg = (int)h_segs.size();
-  Tmp<int2> segs;
-  Tmp<int32_t> seg_panel, tcount, toff;
-  PL_CK(segs.alloc(nseg));
-  PL_CK(seg_panel.alloc(nseg));
-  PL_CK(tcount.alloc(nseg));
-  PL_CK(toff.alloc(nseg + 1));
+  int32_t *segs_words, *seg_panel, *tcount, *toff, *pssrc, *pslen = flag;  // (the flags have been summed)
+  PL_CK(segments.alloc({{&segs_words, 2 * (size_t)nseg}, {&seg_panel, (size_t)nseg}, {&tcount, (size_t)nseg},
+                        {&toff, (size_t)nseg + 1}, {&pssrc, (size_t)nps}}));
+  int2* segs = reinterpret_cast<int2*>(segs_words);
+  k_pl_compact<<<grid_for(len), 256, 0, s>>>(len, R, cnt, src, psidx, out->psrow, pslen,
+                                             pssrc);
   if (nseg > 0) {
-    PL_CK(cudaMemcpyAsync(segs.p, h_segs.data(), sizeof(int2) * nseg, cudaMemcpyHostToDevice, s));
-    PL_CK(cudaMemcpyAsync(seg_panel.p, h_seg_panel.data(), sizeof(int32_t) * nseg,
+    PL_CK(cudaMemcpyAsync(segs, h_segs.data(), sizeof(int2) * nseg, cudaMemcpyHostToDevice, s));
+    PL_CK(cudaMemcpyAsync(seg_panel, h_seg_panel.data(), sizeof(int32_t) * nseg,
                           cudaMemcpyHostToDevice, s));
-    k_pl_pack<false><<<(nseg + kPackWarps - 1) / kPackWarps, kPackWarps * 32, 0, s>>>(nseg, segs.p, seg_panel.p, pslen.p,
-                                                         nullptr, pscap, tcount.p, nullptr, nullptr,
+    k_pl_pack<false><<<(nseg + kPackWarps - 1) / kPackWarps, kPackWarps * 32, 0, s>>>(nseg, segs, seg_panel, pslen,
+                                                         nullptr, pscap, tcount, nullptr, nullptr,
                                                          nullptr);
   }
-  launch_scan(tcount.p, toff.p, nseg, scan_tmp.p, s);
+  launch_scan(tcount, toff, nseg, scan_tmp, s);
   std::vector<int32_t> h_toff(nseg + 1);
-  PL_CK(cudaMemcpyAsync(h_toff.data(), toff.p, sizeof(int32_t) * (nseg + 1),
+  PL_CK(cudaMemcpyAsync(h_toff.data(), toff, sizeof(int32_t) * (nseg + 1),
                         cudaMemcpyDeviceToHost, s));
   PL_CK(cudaStreamSynchronize(s));
   const int nt = h_toff[nseg];
   CKS(dalloc(ctx, &out->tiles, (size_t)nt));
-  Tmp<int32_t> tlen, tpanel, nzoff;
-  PL_CK(tlen.alloc(nt));
-  PL_CK(tpanel.alloc(nt));
-  PL_CK(nzoff.alloc(nt + 1));
+  int32_t *tlen, *tpanel, *nzoff;
+  PL_CK(per_tile.alloc({{&tlen, (size_t)nt}, {&tpanel, (size_t)nt}, {&nzoff, (size_t)nt + 1}}));
   if (nseg > 0)
-    k_pl_pack<true><<<(nseg + kPackWarps - 1) / kPackWarps, kPackWarps * 32, 0, s>>>(nseg, segs.p, seg_panel.p, pslen.p, toff.p,
-                                                        pscap, nullptr, out->tiles, tlen.p, tpanel.p);
-  launch_scan(tlen.p, nzoff.p, nt, scan_tmp.p, s);
-  if (nt > 0) k_pl_tile_begin<<<(nt + 255) / 256, 256, 0, s>>>(nt, nzoff.p, out->tiles);
+    k_pl_pack<true><<<(nseg + kPackWarps - 1) / kPackWarps, kPackWarps * 32, 0, s>>>(nseg, segs, seg_panel, pslen, toff,
+                                                        pscap, nullptr, out->tiles, tlen, tpanel);
+  launch_scan(tlen, nzoff, nt, scan_tmp, s);
+  if (nt > 0) k_pl_tile_begin<<<(nt + 255) / 256, 256, 0, s>>>(nt, nzoff, out->tiles);
   std::vector<int32_t> h_nzoff(nt + 1);
-  PL_CK(cudaMemcpyAsync(h_nzoff.data(), nzoff.p, sizeof(int32_t) * (nt + 1),
+  PL_CK(cudaMemcpyAsync(h_nzoff.data(), nzoff, sizeof(int32_t) * (nt + 1),
                         cudaMemcpyDeviceToHost, s));
   PL_CK(cudaStreamSynchronize(s));
   const int64_t nzp = h_nzoff[nt];
@@ -903,7 +911,7 @@ pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out) {
   CKS(dalloc(ctx, &out->col, (size_t)nzp + 32));
   CKS(dalloc(ctx, &out->wd, (size_t)nzp / 8 + 16));
   if (nt > 0)
-    k_pl_fill<<<grid_for((int64_t)nt * 32), 256, 0, s>>>(nt, out->tiles, tpanel.p, pslen.p, pssrc.p,
+    k_pl_fill<<<grid_for((int64_t)nt * 32), 256, 0, s>>>(nt, out->tiles, tpanel, pslen, pssrc,
                                                         col, val, P, out->val, out->col, out->wd);
   ctx->launches += 1;
 

@@ -533,8 +533,8 @@ static pdhg_status tune_schedules(pdhg_ctx* ctx) {
         d = fixed;
         if (e == kSliced && mx) d.view.slice_val = d.v32;
       } else {
-        std::future<HostSched>& pre = ctx->presched[which][e == 16 ? 0 : 1];
-        HostSched h = (cand.second == 0 && (e == 16 || e == 32) && pre.valid())
+        std::future<HostSched>& pre = ctx->presched[which][e == 16 ? 0 : e == 32 ? 1 : 2];
+        HostSched h = (cand.second == 0 && e >= 8 && pre.valid())
                           ? pre.get()
                           : build_sched(rp.data(), nrows, e, nullptr, 1, cand.second);
         CKS(upload_sched(ctx, h, &d, on_a ? ctx->a_rp : ctx->t_rp));
@@ -970,17 +970,17 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
   CKS(fixed_schedules(ctx));
   stage("float64 schedules");
 
-  // the tuner's E = 16 and E = 32 schedules are host work: build them on a
-  // host thread while the GPU runs the power iteration
+  // the tuner's E = 16 and E = 32 schedules, and E = 8 beside slices, are host
+  // work: build them on a host thread while the GPU runs the power iteration
   if (ctx->opt.autotune && ctx->opt.tile_nnz == 0 && !ctx->resident) {
     for (int which = 0; which < 2; ++which)
-      for (int q = 0; q < 2; ++q) {
+      for (int q = 0; q < 3; ++q) {
         const int32_t* rp = which == 0 ? ctx->h_a_rp.data() : ctx->h_t_rp.data();
         const int nrows = which == 0 ? m : n;
-        if ((int64_t)rp[nrows] < (int64_t)kLongWindowRows * nrows ||
-            (which == 0 ? ctx->sa8 : ctx->st8).view.e == kSliced)
+        const bool slices = (which == 0 ? ctx->sa8 : ctx->st8).view.e == kSliced;
+        if (q == 2 ? !(slices && ctx->mixed) : slices || (int64_t)rp[nrows] < (int64_t)kLongWindowRows * nrows)
           continue;  // not tried
-        const int e = q == 0 ? 16 : 32;
+        const int e = q == 0 ? 16 : q == 1 ? 32 : 8;
         ctx->presched[which][q] = std::async(std::launch::async, [rp, nrows, e] {
           return build_sched(rp, nrows, e, nullptr, 1, 0);
         });
