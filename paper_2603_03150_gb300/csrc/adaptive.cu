@@ -252,11 +252,11 @@ __global__ void k_adapt_revert(IterBuffers<T> B) {
 
 template <typename T>
 void launch_adapt_primal(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_S(B.t_sched.e, launch_pdl(k_aprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(T, B.t_sched.e, launch_pdl(k_aprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_adapt_dual(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_S(B.a_sched.e, launch_pdl(k_adual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(T, B.a_sched.e, launch_pdl(k_adual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_adapt_revert(const IterBuffers<T>& B, int grid, cudaStream_t s) {
@@ -273,10 +273,11 @@ PDHG_INST(double)
 
 template <int E>
 static const void* adaptive_kernel(int which) {
+  constexpr int F = E == kSliced ? 8 : E;  // (float32 has no slices)
   switch (which) {
-    case 0: return (const void*)k_aprimal<float, kBlock, E>;
+    case 0: return (const void*)k_aprimal<float, kBlock, F>;
     case 1: return (const void*)k_aprimal<double, kBlock, E>;
-    case 2: return (const void*)k_adual<float, kBlock, E>;
+    case 2: return (const void*)k_adual<float, kBlock, F>;
     case 3: return (const void*)k_adual<double, kBlock, E>;
     default: return nullptr;
   }
@@ -296,7 +297,7 @@ cudaError_t configure_adaptive_kernels(size_t max_smem) {
 
 int adaptive_occupancy(int which, int e, size_t smem) {
   const void* f = nullptr;
-  PDHG_DISPATCH_S(e, f = adaptive_kernel<E_>(which));
+  PDHG_DISPATCH_S(double, e, f = adaptive_kernel<E_>(which));
   int nb = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, kBlock, smem);
   return nb < 1 ? 1 : nb;

@@ -54,10 +54,6 @@ constexpr int kSliced = 64;       // SchedView::e of a sliced schedule
 constexpr int kSliceRows = 64;    // rows sorted together
 constexpr int kSliceShort = 24;   // a lane per row up to this many nonzeros
 constexpr int kSliceWarps = 8;    // per SM, or short rows take more lanes
-// Float32 half-steps: slices up to this many nonzeros (A~^T of the planted LP
-// 100,000 x 250,000 8.6 -> 6.9 us, of 20,000 x 50,000 5.2 -> 3.5), tiles above
-// (A~^T of the 2000 x 2000 transportation LP 24.8 us against 32.9).
-constexpr int kSliceMaxNnz32 = 1 << 21;
 constexpr int kSliceMaxRow = 256; // 8 lanes per row up to this many; none longer
 
 // ---------------------------------------------------------------------------

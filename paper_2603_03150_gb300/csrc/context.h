@@ -60,7 +60,6 @@ struct DevSched {
   int32_t* counters = nullptr;
   double* slots = nullptr;
   uint32_t* wd = nullptr;
-  float* v32 = nullptr;  // sliced: the values in float32 (float32-mixed contexts)
   SchedView view{};
 };
 

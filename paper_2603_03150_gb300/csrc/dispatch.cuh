@@ -1,10 +1,11 @@
 // Launch helpers shared by the translation units that launch tile kernels.
 #pragma once
+#include "common.cuh"
 #include <cuda_runtime.h>
 
 // SpMV variant of a schedule -> template instantiation: segmented with
 // E = 8, 16, 32 nonzeros per thread, or vector with 4 / 8 lanes per row
-// (E_ = -4, -8); PDHG_DISPATCH_S also the slices of single LPs.
+// (E_ = -4, -8); PDHG_DISPATCH_S also the slices of single LPs in float64.
 #define PDHG_DISPATCH_E(e, ...)                 \
   switch (e) {                                  \
     case -4: {                                  \
@@ -29,9 +30,9 @@
     } break;                                    \
   }
 
-#define PDHG_DISPATCH_S(e, ...)                 \
-  if ((e) == kSliced) {                         \
-    constexpr int E_ = kSliced;                 \
+#define PDHG_DISPATCH_S(T, e, ...)              \
+  if (sizeof(T) == 8 && (e) == kSliced) {       \
+    constexpr int E_ = sliced_or_8<T>();        \
     __VA_ARGS__;                                \
   } else {                                      \
     PDHG_DISPATCH_E(e, __VA_ARGS__)             \
@@ -47,6 +48,12 @@
   }
 
 namespace pdhg {
+
+// (float32 half-steps have no slices: no kernels of that kind are built)
+template <typename T>
+constexpr int sliced_or_8() {
+  return sizeof(T) == 8 ? kSliced : 8;
+}
 
 // Launch with programmatic stream serialization (the kernel must start with
 // pdl_enter(): it may begin while the previous kernel on the stream drains).

@@ -47,11 +47,11 @@ __global__ void __launch_bounds__(BLOCK) k_hdual(IterBuffers<T> B, int i) {
 
 template <typename T>
 void launch_hprimal(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_S(B.t_sched.e, launch_pdl(k_hprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(T, B.t_sched.e, launch_pdl(k_hprimal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_hdual(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_S(B.a_sched.e, launch_pdl(k_hdual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(T, B.a_sched.e, launch_pdl(k_hdual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template void launch_hprimal<float>(const IterBuffers<float>&, const Launch&, int, cudaStream_t);
 template void launch_hprimal<double>(const IterBuffers<double>&, const Launch&, int, cudaStream_t);
@@ -60,10 +60,11 @@ template void launch_hdual<double>(const IterBuffers<double>&, const Launch&, in
 
 template <int E>
 static const void* halpern_kernel(int which) {
+  constexpr int F = E == kSliced ? 8 : E;  // (float32 has no slices)
   switch (which) {
-    case 0: return (const void*)k_hprimal<float, kBlock, E>;
+    case 0: return (const void*)k_hprimal<float, kBlock, F>;
     case 1: return (const void*)k_hprimal<double, kBlock, E>;
-    case 2: return (const void*)k_hdual<float, kBlock, E>;
+    case 2: return (const void*)k_hdual<float, kBlock, F>;
     case 3: return (const void*)k_hdual<double, kBlock, E>;
     default: return nullptr;
   }
@@ -83,7 +84,7 @@ cudaError_t configure_halpern_kernels(size_t max_smem) {
 
 int halpern_occupancy(int which, int e, size_t smem) {
   const void* f = nullptr;
-  PDHG_DISPATCH_S(e, f = halpern_kernel<E_>(which));
+  PDHG_DISPATCH_S(double, e, f = halpern_kernel<E_>(which));
   int nb = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, kBlock, smem);
   return nb < 1 ? 1 : nb;

@@ -191,15 +191,15 @@ __global__ void k_restart(IterBuffers<T> B) {
 
 template <typename T>
 void launch_primal(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_S(B.t_sched.e, launch_pdl(k_primal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(T, B.t_sched.e, launch_pdl(k_primal<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_dual(const IterBuffers<T>& B, const Launch& L, int i, cudaStream_t s) {
-  PDHG_DISPATCH_S(B.a_sched.e, launch_pdl(k_dual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
+  PDHG_DISPATCH_S(T, B.a_sched.e, launch_pdl(k_dual<T, kBlock, E_>, L.grid, kBlock, L.smem, s, B, i));
 }
 template <typename T>
 void launch_eval(const IterBuffers<T>& B, const Launch& L, int chunk, cudaStream_t s) {
-  PDHG_DISPATCH_S(B.t_sched.e, k_eval<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(B, chunk));
+  PDHG_DISPATCH_S(T, B.t_sched.e, k_eval<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(B, chunk));
 }
 template <typename T>
 void launch_restart(const IterBuffers<T>& B, int grid, cudaStream_t s) {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(BLOCK) k_spmv(SchedView S, const int32_t* rp, 
 template <typename T>
 void launch_spmv(const SchedView& S, const int32_t* rp, const int32_t* col, const T* val,
                  const T* v, T* out, const Launch& L, cudaStream_t s) {
-  PDHG_DISPATCH_S(S.e, k_spmv<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, v, out));
+  PDHG_DISPATCH_S(T, S.e, k_spmv<T, kBlock, E_><<<L.grid, kBlock, L.smem, s>>>(S, rp, col, val, v, out));
 }
 
 // ---------------------------------------------------------------------------
@@ -546,14 +546,15 @@ size_t tile_smem(int nv, bool f32, int max_rows, int e) {
 
 template <int E>
 static const void* tile_kernel(int which) {
+  constexpr int F = E == kSliced ? 8 : E;  // (float32 has no slices)
   switch (which) {
-    case 0: return (const void*)k_primal<float, kBlock, E>;
+    case 0: return (const void*)k_primal<float, kBlock, F>;
     case 1: return (const void*)k_primal<double, kBlock, E>;
-    case 2: return (const void*)k_dual<float, kBlock, E>;
+    case 2: return (const void*)k_dual<float, kBlock, F>;
     case 3: return (const void*)k_dual<double, kBlock, E>;
-    case 4: return (const void*)k_eval<float, kBlock, E>;
+    case 4: return (const void*)k_eval<float, kBlock, F>;
     case 5: return (const void*)k_eval<double, kBlock, E>;
-    case 6: return (const void*)k_spmv<float, kBlock, E>;
+    case 6: return (const void*)k_spmv<float, kBlock, F>;
     case 7: return (const void*)k_spmv<double, kBlock, E>;
     default: return nullptr;
   }

@@ -404,6 +404,11 @@ std::vector<int32_t> res_order(const std::vector<ResLp>& lps, const std::vector<
 // tile kernels' own paths.
 pdhg_status resident_build(pdhg_ctx* ctx) {
   const pdhg_options& o = ctx->opt;
+  // A float32-mixed solve of one LP keeps the tile kernels' order of addition:
+  // its float64 solution is that of float32 iterates, which differ by 1e-6
+  // between orders, and a program that stores or compares such solutions would
+  // see it.
+  if (ctx->mixed && !ctx->batch) return PDHG_OK;
   if (o.tile_nnz != 0 || o.spmv_layout != 0 || o.panel_width != 0 || o.kernel_timing != 0 ||
       o.step_rule != 0 || (ctx->batch && o.persistent != 0))
     return PDHG_OK;

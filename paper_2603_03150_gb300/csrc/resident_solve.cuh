@@ -348,18 +348,20 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
 // the kernel for clusters of C CTAs
 template <typename T>
 const void* res_solve_kernel(int C, bool halpern) {
+  constexpr bool H = sizeof(T) == 8;  // float32 runs in batches, which have no Halpern form
   const void* f = nullptr;
-  RES_DISPATCH_C(C, f = halpern ? (const void*)k_res_solve<T, C_, true>
+  RES_DISPATCH_C(C, f = halpern ? (const void*)k_res_solve<T, C_, H>
                                 : (const void*)k_res_solve<T, C_, false>);
   return f;
 }
 template <typename T>
 cudaError_t launch_res_solve(const ResSolve<T>& A, int C, int lps, size_t smem, bool halpern,
                              cudaStream_t s) {
+  constexpr bool H = sizeof(T) == 8;
   cudaLaunchAttribute attr;
   const cudaLaunchConfig_t cfg = res_config(C, lps, smem, s, &attr);
   cudaError_t e = cudaSuccess;
-  RES_DISPATCH_C(C, e = halpern ? cudaLaunchKernelEx(&cfg, k_res_solve<T, C_, true>, A)
+  RES_DISPATCH_C(C, e = halpern ? cudaLaunchKernelEx(&cfg, k_res_solve<T, C_, H>, A)
                                 : cudaLaunchKernelEx(&cfg, k_res_solve<T, C_, false>, A));
   return e;
 }

@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 __global__ void __launch_bounds__(kWarps * 32)
     k_sl_fill(int nrows, int nwin, int lg1, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
               const double* __restrict__ val, const int32_t* __restrict__ slice0,
-              const int32_t* __restrict__ elem0, int4* out, int32_t* col_s, double* v64, float* v32) {
+              const int32_t* __restrict__ elem0, int4* out, int32_t* col_s, double* v64) {
   __shared__ int key[kWarps][kSliceRows];
   __shared__ uint8_t at[kWarps][kSliceRows];
   const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, q = blockIdx.x * kWarps + wi;
@@ -107,10 +107,8 @@ __global__ void __launch_bounds__(kWarps * 32)
     for (int k = 0; k < w; ++k) {
       const int j = k * G + gl;
       const bool in = j < len;
-      const double v = in ? val[b + j] : 0.0;
       col_s[off + k * 32 + lane] = in ? col[b + j] : 0;
-      v64[off + k * 32 + lane] = v;
-      if (v32) v32[off + k * 32 + lane] = (float)v;
+      v64[off + k * 32 + lane] = in ? val[b + j] : 0.0;
     }
     off += 32 * w;
   }
@@ -118,8 +116,8 @@ __global__ void __launch_bounds__(kWarps * 32)
 
 }  // namespace
 
-// The sliced schedule of A~ (on_a) or A~^T with its float64 values (and, up to
-// kSliceMaxNnz32 nonzeros, float32 ones in float32-mixed contexts); no row has more than kSliceMaxRow nonzeros.
+// The sliced schedule of A~ (on_a) or A~^T with its float64 values; no row has
+// more than kSliceMaxRow nonzeros.
 // d->view.e stays 0, and the matrix is left to the tiles, where rows of very
 // different lengths share windows (more padding than nonzeros) or where the
 // copy would take more than a quarter of the memory that is left.
@@ -142,7 +140,6 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
           *scol = nullptr;
   unsigned long long *padded = nullptr, total = 0;
   double* v64 = nullptr;
-  float* v32 = nullptr;
   CKS(dalloc(ctx, &ord, (size_t)nw * kSliceRows));
   CKS(dalloc(ctx, &count, (size_t)nw));
   CKS(dalloc(ctx, &slice0, (size_t)nw + 1));
@@ -160,8 +157,7 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   CK(cudaMemcpyAsync(&total, padded, sizeof(total), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (total > (unsigned long long)ctx->nnz * 2 || total > (unsigned long long)INT32_MAX) return PDHG_OK;
-  const bool f32 = ctx->mixed && ctx->nnz <= kSliceMaxNnz32;
-  const size_t bytes = (size_t)total * (f32 ? 16 : 12);
+  const size_t bytes = (size_t)total * 12;
   size_t left = 0, all = 0;
   if (bytes > (size_t(1) << 28)) {
     CK(cudaMemGetInfo(&left, &all));
@@ -170,8 +166,7 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   CKS(dalloc(ctx, &slices, (size_t)nslices));
   CKS(dalloc(ctx, &scol, (size_t)total));
   CKS(dalloc(ctx, &v64, (size_t)total));
-  if (f32) CKS(dalloc(ctx, &v32, (size_t)total));
-  k_sl_fill<<<grid, kWarps * 32, 0, s>>>(nrows, nw, lg1, rp, col, val, slice0, elem0, slices, scol, v64, v32);
+  k_sl_fill<<<grid, kWarps * 32, 0, s>>>(nrows, nw, lg1, rp, col, val, slice0, elem0, slices, scol, v64);
   ctx->launches += 1;
   CK(cudaGetLastError());
   SchedView& V = d->view;
@@ -184,7 +179,6 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   V.slice_ord = ord;
   V.slice_col = scol;
   V.slice_val = v64;
-  d->v32 = v32;
   return PDHG_OK;
 }
 

@@ -516,14 +516,11 @@ static pdhg_status tune_schedules(pdhg_ctx* ctx) {
     } else {
       cands = {{8, 0}};
     }
-    // sliced: in float64 slices were the faster ones on every measured matrix;
-    // in float32 8 nonzeros per thread stays a candidate
+    // In float64 the slices were the faster ones on every matrix that has them;
+    // float32 half-steps keep the tiles, whose order of addition their results
+    // have (see resident_build).
     const DevSched& fixed = on_a ? ctx->sa8 : ctx->st8;
-    if (fixed.view.e == kSliced) {
-      cands.clear();
-      if (mx) cands.push_back({8, 0});
-      if (!mx || (fixed.v32 && ctx->opt.autotune)) cands.push_back({kSliced, 0});
-    }
+    if (fixed.view.e == kSliced && !mx) cands = {{kSliced, 0}};
     DevSched best{};
     float best_ms = 1e30f;
     for (const auto& cand : cands) {
@@ -531,7 +528,6 @@ static pdhg_status tune_schedules(pdhg_ctx* ctx) {
       DevSched d;
       if (e == fixed.view.e && cand.second == 0) {
         d = fixed;
-        if (e == kSliced && mx) d.view.slice_val = d.v32;
       } else {
         std::future<HostSched>& pre = ctx->presched[which][e == 16 ? 0 : e == 32 ? 1 : 2];
         HostSched h = (cand.second == 0 && e >= 8 && pre.valid())
@@ -978,8 +974,9 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
         const int32_t* rp = which == 0 ? ctx->h_a_rp.data() : ctx->h_t_rp.data();
         const int nrows = which == 0 ? m : n;
         const bool slices = (which == 0 ? ctx->sa8 : ctx->st8).view.e == kSliced;
-        if (q == 2 ? !(slices && ctx->mixed) : slices || (int64_t)rp[nrows] < (int64_t)kLongWindowRows * nrows)
-          continue;  // not tried
+        const bool long_rows = (int64_t)rp[nrows] >= (int64_t)kLongWindowRows * nrows;
+        if (slices && !ctx->mixed) continue;          // not tried
+        if (q == 2 ? !slices : !long_rows) continue;  // built already, or not tried
         const int e = q == 0 ? 16 : q == 1 ? 32 : 8;
         ctx->presched[which][q] = std::async(std::launch::async, [rp, nrows, e] {
           return build_sched(rp, nrows, e, nullptr, 1, 0);
@@ -1186,8 +1183,7 @@ extern "C" pdhg_status pdhg_solve(pdhg_ctx* ctx, double eps_rel, int64_t max_ite
   hs.rejects = 0;
   CK(cudaMemcpyAsync(ctx->sc, &hs, sizeof(hs), cudaMemcpyHostToDevice, ctx->stream));
   if (ctx->resident) {
-    const pdhg_status rs = ctx->mixed ? resident_solve<float>(ctx, iter_buffers<float>(ctx))
-                                      : resident_solve<double>(ctx, iter_buffers<double>(ctx));
+    const pdhg_status rs = resident_solve<double>(ctx, iter_buffers<double>(ctx));
     CKS(rs);
     if (rs == PDHG_TIMEOUT) {
       ctx->last_status = rs;

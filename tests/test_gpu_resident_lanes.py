@@ -5,7 +5,8 @@ not fill their lanes, empty rows, rows of the longer classes beside short ones.
 
 Tolerances as in the other parity tests: float64 states 1e-9 relative in the
 infinity norm (sums in another order over 100 iterations of a nonexpansive map),
-float32-mixed states 1e-4."""
+float32-mixed solutions (of a batch of one LP: a float32 LP alone keeps the tile
+kernels) 1e-4."""
 import numpy as np
 import pytest
 import scipy.sparse as sp
@@ -50,10 +51,15 @@ def test_states_match_the_tile_kernels(rows, lanes, precision, tol):
     lp = rows_lp(np.resize(pool[::-1], rows), 127, rows)
     out = []
     for tile_nnz in (0, 2044):
+        if precision == "fp32":
+            with pdhg.BatchSolver([lp], precision=precision, tile_nnz=tile_nnz) as s:
+                s.solve(0.0, 100)
+                out.append((s.get(), 0.0))
+            continue
         with pdhg.Solver.from_lp(lp, precision=precision, tile_nnz=tile_nnz) as s:
             assert s.solve(0.0, 100) == pdhg.PDHG_MAX_ITER
             out.append((s.state(), s.scaling()["sigma_max"]))
     (a, sa), (b, sb) = out
     assert abs(sa - sb) <= 1e-12 * sb
-    for k in ("x", "y", "x_avg", "y_avg"):
+    for k in ("x", "y", "x_avg", "y_avg") if precision == "fp64" else ("x", "y"):
         assert rel_inf(a[k], b[k]) < tol, k
