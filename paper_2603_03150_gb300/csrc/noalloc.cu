@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "pdhg.h"
+#include "resident.cuh"
 
 namespace pdhg {
 void set_error(const char* fmt, ...);
@@ -42,28 +43,52 @@ __device__ __forceinline__ double na_block_sum(int base, int end, const double* 
   return o[0];
 }
 
-// n <= kNaPerBlock: all of it in one block, one launch (500 entries, call after
-// call: 10.2 us where three launches took 14.3)
-__global__ void __launch_bounds__(kNaThreads)
+// n <= kNaSmall: one launch, a cluster of 8 blocks whose sums of x^T z go
+// through distributed shared memory.  Three launches took 14.5 us call after
+// call at any of these sizes and one block of 256 threads 10.4 / 14.6 / 24.3 at
+// 500 / 1000 / 2000 entries (an entry's quotients keep an SM's float64 pipe for
+// 18 clocks); the cluster takes 8.3 up to 2048 entries and 10.4 up to 4096, the two
+// launches above 12.5.
+constexpr int kNaCluster = 8, kNaSmall = 4096;
+__global__ void __cluster_dims__(kNaCluster, 1, 1) __launch_bounds__(kNaThreads)
     k_na_small(int n, const double* __restrict__ x, const double* __restrict__ z, double mu_min,
-               double delta, double alpha, double* scratch, double* mu_out,
-               double* __restrict__ x_out, double* __restrict__ z_out) {
-  __shared__ double red[kNaThreads / 32];
-  __shared__ double mu_s;
-  const double s = na_block_sum(0, n, x, z, red);
+               double delta, double alpha, double* mu_out, double* __restrict__ x_out,
+               double* __restrict__ z_out) {
+  constexpr int K = kNaSmall / (kNaCluster * kNaThreads);
+  __shared__ double part[kNaCluster], red[kNaThreads / 32], mu_s;
+  const pdhg::ResCluster<kNaCluster> cl(part);
+  const int first = cl.rank * kNaThreads + threadIdx.x;
+  double xs[K], zs[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int j = first + k * kNaCluster * kNaThreads;
+    xs[k] = j < n ? x[j] : 0.0;
+    zs[k] = j < n ? z[j] : 0.0;
+  }
+  cl.sync();  // every block runs: its shared memory may be written
+  double acc[1] = {0.0}, sum[1];
+#pragma unroll
+  for (int k = 0; k < K; ++k) acc[0] += xs[k] * zs[k];
+  pdhg::block_sum<kNaThreads, 1>(acc, sum, red);
+  if (threadIdx.x == 0) cl.push((uint32_t)cl.rank * 8u, sum[0]);
+  cl.sync();
   if (threadIdx.x == 0) {
+    const double s = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
     mu_s = fmax(s / (double)n, mu_min);
-    scratch[kNaMaxBlocks] = mu_s;
-    if (mu_out) *mu_out = mu_s;
+    if (mu_out && cl.rank == 0) *mu_out = mu_s;
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < n; j += kNaThreads) {
-    double xp = x[j], zp = z[j];
-    pdhg::centered_pair(mu_s, delta, alpha, xp, zp);
-    x_out[j] = xp;
-    z_out[j] = zp;
+#pragma unroll 1
+  for (int k = 0; k < K; ++k) {
+    const int j = first + k * kNaCluster * kNaThreads;
+    if (j >= n) break;
+    pdhg::centered_pair(mu_s, delta, alpha, xs[0], zs[0]);
+    x_out[j] = xs[0];
+    z_out[j] = zs[0];
+    xs[0] = xs[K - 1], zs[0] = zs[K - 1];
   }
 }
+static_assert(kNaSmall == 2 * kNaCluster * kNaThreads, "an entry or two per thread");
 
 // partial sums of x^T z; the block that finishes last adds them in a fixed
 // order and writes mu (one thread adding them took 68 clocks for each)
@@ -155,9 +180,9 @@ extern "C" pdhg_status pdhg_centered_point_noalloc(int32_t n, const double* x, c
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int nblocks = (int)((n + kNaPerBlock - 1) / kNaPerBlock);
-  if (nblocks == 1) {
-    k_na_small<<<1, kNaThreads, 0, s>>>(n, x, z, mu_min, delta_max, alpha_min, scratch, mu_target,
-                                        x_out, z_out);
+  if (n <= kNaSmall) {
+    k_na_small<<<kNaCluster, kNaThreads, 0, s>>>(n, x, z, mu_min, delta_max, alpha_min, mu_target, x_out,
+                                                 z_out);
   } else {
     k_na_partial<<<nblocks, kNaThreads, 0, s>>>(n, x, z, mu_min, scratch, mu_target);
     int grid = (n + 255) / 256;

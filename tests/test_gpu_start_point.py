@@ -1,5 +1,5 @@
-"""The no-allocation start point at the edges of its two forms (one block up to
-2048 entries, partial sums by many blocks above) and on special values, against
+"""The no-allocation start point at the edges of its two forms (a cluster of
+blocks up to 4096 entries, partial sums by many blocks above) and on special values, against
 the oracle.  Tolerance: the sums of up to 70,000 positive products agree to
 1e-12, so mu and the moved entries to 1e-11 relative."""
 import numpy as np
