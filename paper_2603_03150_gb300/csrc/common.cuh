@@ -54,7 +54,8 @@ constexpr int kSliced = 64;       // SchedView::e of a sliced schedule
 constexpr int kSliceRows = 64;    // rows sorted together
 constexpr int kSliceShort = 24;   // a lane per row up to this many nonzeros
 constexpr int kSliceWarps = 8;    // per SM, or short rows take more lanes
-constexpr int kSliceMaxRow = 256; // 8 lanes per row up to this many; none longer
+constexpr int kSliceMid = 128;    // 8 lanes per row up to this many, a warp above
+constexpr int kSliceMaxSteps = 255;
 
 // ---------------------------------------------------------------------------
 // Column-panel layout of one matrix (float32 iterations).  The columns are cut

@@ -247,7 +247,8 @@ pdhg_status polling_resources(pdhg_ctx* ctx);
 // panels do not apply (float64, batches, or dense partial sums above about
 // twice the nonzeros); the device layout
 bool panel_shape(const pdhg_ctx* ctx, bool on_a, int* P, int* npanels, int pscap = 256);
-// the sliced schedule of A~ or A~^T (slices.cu): no row above kSliceMaxRow
+// whether a matrix is to be sliced, and its sliced schedule (slices.cu)
+bool slices_pay(const pdhg_ctx* ctx, bool on_a);
 pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d);
 pdhg_status build_panel_layout(pdhg_ctx* ctx, bool on_a, DevPanel* out);
 // batched solve from iteration k0 to max_iter in one cooperative launch

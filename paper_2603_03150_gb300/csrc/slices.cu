@@ -14,15 +14,17 @@ constexpr int kWarps = 8;
 static_assert(kSliceRows == 64, "a lane takes two rows of a window");
 
 struct Cut {  // of one window: rows of each class, and where its slices start
-  int n8, n1, lg1;  // rows with 8 lanes, rows with 2^lg1 lanes
+  int n32, n8, n1, lg1;  // rows with 32, 8 and 2^lg1 lanes
   __device__ __forceinline__ int s8() const { return (n8 + 3) / 4; }
-  __device__ __forceinline__ int slices() const { return s8() + ((n1 << lg1) + 31) / 32; }
+  __device__ __forceinline__ int slices() const { return n32 + s8() + ((n1 << lg1) + 31) / 32; }
   // lanes per row (log2), first position and rows of slice s
   __device__ __forceinline__ void slice(int s, int& lg, int& p0, int& rows) const {
-    if (s < s8())
-      lg = 3, p0 = 4 * s, rows = min(4, n8 - p0);
+    if (s < n32)
+      lg = 5, p0 = s, rows = 1;
+    else if (s < n32 + s8())
+      lg = 3, p0 = n32 + 4 * (s - n32), rows = min(4, n32 + n8 - p0);
     else
-      lg = lg1, p0 = n8 + (32 >> lg1) * (s - s8()), rows = min(32 >> lg1, n8 + n1 - p0);
+      lg = lg1, p0 = n32 + n8 + (32 >> lg1) * (s - n32 - s8()), rows = min(32 >> lg1, n32 + n8 + n1 - p0);
   }
 };
 
@@ -46,15 +48,16 @@ __device__ __forceinline__ Cut sort_window(int nrows, int q, const int32_t* __re
       for (int k = 0; k < 2; ++k)
         rank[k] += other > len[k] || (other == len[k] && j < lane + 32 * k);
     }
-  int n8 = 0;
+  int n32 = 0, n8 = 0;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     key[rank[h]] = len[h];
     at[rank[h]] = (uint8_t)(lane + 32 * h);
-    n8 += __popc(__ballot_sync(0xffffffffu, len[h] > kSliceShort << lg1));
+    n32 += __popc(__ballot_sync(0xffffffffu, len[h] > kSliceMid));
+    n8 += __popc(__ballot_sync(0xffffffffu, len[h] > kSliceShort << lg1 && len[h] <= kSliceMid));
   }
   __syncwarp();
-  return Cut{n8, nr - n8, lg1};
+  return Cut{n32, n8, nr - n32 - n8, lg1};
 }
 
 __global__ void __launch_bounds__(kWarps * 32)
@@ -65,7 +68,7 @@ __global__ void __launch_bounds__(kWarps * 32)
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, q = blockIdx.x * kWarps + w;
   if (q >= nwin) return;  // warp-uniform
   const Cut c = sort_window(nrows, q, rp, lg1, key[w], at[w]);
-  for (int p = lane; p < c.n8 + c.n1; p += 32) ord[(size_t)q * kSliceRows + p] = at[w][p];
+  for (int p = lane; p < c.n32 + c.n8 + c.n1; p += 32) ord[(size_t)q * kSliceRows + p] = at[w][p];
   int e = 0;
   for (int s = lane; s < c.slices(); s += 32) {
     int lg, p0, rows;
@@ -116,8 +119,32 @@ __global__ void __launch_bounds__(kWarps * 32)
 
 }  // namespace
 
-// The sliced schedule of A~ (on_a) or A~^T with its float64 values; no row has
-// more than kSliceMaxRow nonzeros.
+// log2 of the lanes of a short row: 1, or 2 or 4 lanes where that leaves the SMs
+// fewer than kSliceWarps warps
+static int short_lanes(const pdhg_ctx* ctx, bool on_a) {
+  const int64_t rows = on_a ? ctx->m : ctx->n;
+  int lg = 0;
+  while (lg < 2 && (rows << lg) < (int64_t)32 * kSliceWarps * ctx->nsm && ctx->nnz >= rows << (lg + 2)) ++lg;
+  return lg;
+}
+
+// The rule for slices in place of tiles: from 2^16 nonzeros on where the LP is
+// not solved on chip and no tile capacity is forced, and where the chain of steps
+// of a row that has a warp to itself is short beside the whole.  A step of a lone warp takes about
+// 0.2 us and a million nonzeros 3.7 us in slices and 7 in tiles.  Float64 A~ of
+// transportation LPs (rows as long as the other side), tiles / slices, us:
+// 2000 x 2000 (62 steps, 8 million) 61 / 42, 1200 x 1900 39 / 22, 700 x 900 13.9 /
+// 10.9, 400 x 400 (13 steps) 7.1 / 5.8; 301 x 707 (22 steps, 0.4 million) 7.7 /
+// 7.6; and left to the tiles 1000 x 300 (31 steps, 0.6 million) 7.9 / 11.1,
+// 200 x 2000 10.8 / 16.1, 1900 x 40 6.4 / 13.5.
+bool slices_pay(const pdhg_ctx* ctx, bool on_a) {
+  if (ctx->batch || ctx->resident || ctx->opt.tile_nnz != 0 || ctx->nnz < (1 << 16)) return false;
+  const int longest = on_a ? ctx->longest_a : ctx->longest_t, steps = (longest + 31) / 32;
+  return longest <= kSliceMid || (steps <= kSliceMaxSteps && steps <= 14 + (int)(ctx->nnz >> 16));
+}
+
+// The sliced schedule of A~ (on_a) or A~^T with its float64 values; no slice
+// has more than kSliceMaxSteps steps (slices_pay).
 // d->view.e stays 0, and the matrix is left to the tiles, where rows of very
 // different lengths share windows (more padding than nonzeros) or where the
 // copy would take more than a quarter of the memory that is left.
@@ -128,12 +155,7 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   const double* val = on_a ? ctx->a_val64 : ctx->t_val64;
   cudaStream_t s = ctx->stream;
   const int nw = (nrows + kSliceRows - 1) / kSliceRows, grid = (nw + kWarps - 1) / kWarps;
-  // short rows: a lane each, or 2 or 4 where that leaves the SMs fewer than
-  // kSliceWarps warps
-  int lg1 = 0;
-  while (lg1 < 2 && ((int64_t)nrows << lg1) < (int64_t)32 * kSliceWarps * ctx->nsm &&
-         ctx->nnz >= ((int64_t)nrows << (lg1 + 2)))
-    ++lg1;
+  const int lg1 = short_lanes(ctx, on_a);
   int4* slices = nullptr;
   uint8_t* ord = nullptr;
   int32_t *elems = nullptr, *elem0 = nullptr, *count = nullptr, *slice0 = nullptr, *tmp = nullptr,
@@ -171,7 +193,7 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   CK(cudaGetLastError());
   SchedView& V = d->view;
   V.ntiles = (nslices + kBlock / 32 - 1) / (kBlock / 32);
-  V.tile_nnz = kSliceMaxRow;
+  V.tile_nnz = 32 * kSliceMaxSteps;
   V.max_rows = kSliceRows;
   V.e = kSliced;
   V.nslices = nslices;

@@ -195,13 +195,6 @@ Launch pdhg::make_launch(pdhg_ctx* ctx, int occ_kind, int e, size_t smem, int nt
 }
 
 
-// A matrix may be sliced (spmv_slice.cuh) from 2^16 nonzeros on where the LP is
-// not solved on chip, no row is long and no tile capacity is forced.
-static bool sliced(const pdhg_ctx* ctx, bool on_a) {
-  return !ctx->batch && !ctx->resident && ctx->opt.tile_nnz == 0 && ctx->nnz >= (1 << 16) &&
-         (on_a ? ctx->longest_a : ctx->longest_t) <= kSliceMaxRow;
-}
-
 // Float64 schedules (report, Algorithm 1, power iteration) and reduction
 // scratch sized for any iteration schedule the tuner may pick.
 static pdhg_status fixed_schedules(pdhg_ctx* ctx) {
@@ -216,7 +209,7 @@ static pdhg_status fixed_schedules(pdhg_ctx* ctx) {
     const std::vector<int32_t>& rp = on_a ? ctx->h_a_rp : ctx->h_t_rp;
     const int nrows = on_a ? ctx->m : ctx->n;
     DevSched* d = on_a ? &ctx->sa8 : &ctx->st8;
-    if (sliced(ctx, on_a)) CKS(build_slices(ctx, on_a, d));
+    if (slices_pay(ctx, on_a)) CKS(build_slices(ctx, on_a, d));
     if (d->view.e != kSliced)
       CKS(upload_sched(ctx, build_sched(rp.data(), nrows, kFixedE), d, on_a ? ctx->a_rp : ctx->t_rp));
     if ((on_a ? ctx->longest_a : ctx->longest_t) > cap_min)

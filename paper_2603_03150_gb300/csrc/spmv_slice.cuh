@@ -1,12 +1,13 @@
 // Sliced SpMV core: the row-sorted counterpart of run_tiles (spmv_tile.cuh) for
-// large matrices without long rows, with the same epilogues.
+// large matrices whose longest row is short beside the whole (slices_pay in
+// slices.cu), with the same epilogues.
 //
 // Windows of kSliceRows rows are sorted by length (longest first, equal lengths
 // in row order); rows of up to kSliceShort nonzeros go 32 to a slice (a lane
-// each), longer ones 4 to a slice (8 lanes each).  Step k of a slice is 32
-// consecutive values and columns.  A warp takes a slice: a row costs one
-// multiply-add per nonzero (and three additions of a shuffle sum in the longer
-// class) where run_tiles adds a segmented scan of 5 additions for 8 nonzeros,
+// each; 2 or 4 on small matrices), those of up to kSliceMid 4 to a slice (8 lanes
+// each), longer ones one to a slice.  Step k of a slice is 32 consecutive values
+// and columns.  A warp takes a slice: a row costs one multiply-add per nonzero
+// (and the additions of a shuffle sum in the longer classes) where run_tiles adds a segmented scan of 5 additions for 8 nonzeros,
 // and there is no block barrier and no staging: the lane that holds a row's sum
 // runs its epilogue, whose operands it has loaded before the sum.
 //
@@ -17,9 +18,9 @@
 // (12.5) 15.8 -> 11.4, A~^T of the power-law LP 43.8 -> 36.6, A~^T of the
 // transportation LP (2) 70.6 -> 60.4.  Windows: the lanes' accesses stay within
 // a window, so wider ones sort better but scatter more: A~^T of the power-law
-// LP 36.6 / 39.2 / 42.2 us at 64 / 128 / 256 rows.  Matrices with longer rows
-// keep the tiles (power-law A~: slices of 32 lanes for rows up to 1024 and chunks
-// above, 49 us against 43.5).
+// LP 36.6 / 39.2 / 42.2 us at 64 / 128 / 256 rows.  Cutting longer rows into
+// chunks did not pay: power-law A~ (rows up to 20,000) 49 us against the tiles'
+// 43.5.
 #pragma once
 #include "spmv_tile.cuh"
 

@@ -1,8 +1,8 @@
-"""Large matrices without long rows in slices (a warp per slice of up to 32 rows
-sorted in windows of 64) against the tile kernels, which a forced tile capacity
-asks for: rows at the edges of the classes (24, 48 or 96 nonzeros with 1, 2 or 4
-lanes per short row, 256 the longest), empty rows, last windows of 1 row, tails
-of 0 to 3 steps; and matrices that keep the tiles.
+"""Large matrices in slices (a warp per slice of up to 32 rows sorted in windows
+of 64) against the tile kernels, which a forced tile capacity asks for: rows at
+the edges of the classes (24, 48 or 96 nonzeros with 1, 2 or 4 lanes per short
+row, 128 with 8 lanes, a warp above), empty rows, last windows of 1 row, tails of
+0 to 3 steps; and matrices that keep the tiles.
 
 Tolerances as in the other parity tests: float64 states 1e-9 relative in the
 infinity norm (the sums run in another order, about 1e-15 per product, over 100
@@ -53,8 +53,8 @@ def rows_lp(lengths, n, seed):
 def lengths(m, seed):
     """Runs of 32 equal lengths from the edges of every class, long ones rare."""
     rng = np.random.default_rng(seed)
-    pool = [0, 1, 2, 3, 4, 5, 7, 8, 23, 24, 25, 47, 48, 49, 95, 96, 97, 255, 256]
-    p = np.array([1.0] * 16 + [0.5, 0.2, 0.2])
+    pool = [0, 1, 2, 3, 4, 5, 7, 8, 23, 24, 25, 47, 48, 49, 95, 96, 97, 127, 128, 129, 255, 256, 257, 600]
+    p = np.array([1.0] * 16 + [0.5] + [0.2] * 6 + [0.05])
     return np.repeat(rng.choice(pool, size=m // 32 + 1, p=p / p.sum()), 32)[:m]
 
 
@@ -63,6 +63,7 @@ MAKERS = {  # 4, 2 and 1 lanes per short row of A; A^T's rows follow
     "lanes_2": lambda: rows_lp(lengths(20033, 2), 30011, 2),
     "lanes_1": lambda: rows_lp(lengths(44993, 3), 60013, 3),
     "planted": lambda: lpgen.planted_lp(33_001, 82_507, seed=5),
+    "transport": lambda: lpgen.transportation_lp(417, 431),  # 14 steps a row
 }
 
 
@@ -85,8 +86,8 @@ def test_states_match_the_tile_kernels(name, method):
 
 
 @pytest.mark.parametrize("name,rows", [
-    ("too_long", np.r_[257, np.full(21000, 17)]),
-    ("too_ragged", np.where(np.arange(40000) % 64 == 0, 250, 4)),  # padded above 2 x
+    ("too_long", np.r_[3000, np.full(21000, 17)]),  # 94 steps, 0.36 million nonzeros
+    ("too_ragged", np.where(np.arange(96000) % 64 == 0, 24, 1)),  # padded above 2 x
 ])
 def test_matrices_that_keep_the_tiles(name, rows):
     lp = rows_lp(rows, 30011, 4)
