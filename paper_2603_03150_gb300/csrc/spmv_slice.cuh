@@ -7,16 +7,17 @@
 // each; 2 or 4 on small matrices), those of up to kSliceMid 4 to a slice (8 lanes
 // each), longer ones one to a slice.  Step k of a slice is 32 consecutive values
 // and columns.  A warp takes a slice: a row costs one multiply-add per nonzero
-// (and the additions of a shuffle sum in the longer classes) where run_tiles adds a segmented scan of 5 additions for 8 nonzeros,
-// and there is no block barrier and no staging: the lane that holds a row's sum
-// runs its epilogue, whose operands it has loaded before the sum.
+// (and the additions of a shuffle sum in the longer classes) where run_tiles adds
+// a segmented scan of 5 additions for 8 nonzeros, and there is no block barrier
+// and no staging: the lane that holds a row's sum runs its epilogue, whose
+// operands it has loaded before the sum.
 //
 // What bounds it is latency (ncu, A~^T of the power-law LP, float64: long
 // scoreboard 31 of 39 cycles per issued instruction, float64 pipe 30%).  Per
 // half-step kernel, tiles of 8 nonzeros per thread against slices, float64: A~^T
 // (5 nonzeros a row) of the planted LP 100,000 x 250,000 16.5 -> 9.7 us, its A~
-// (12.5) 15.8 -> 11.4, A~^T of the power-law LP 43.8 -> 36.6, A~^T of the
-// transportation LP (2) 70.6 -> 60.4.  Windows: the lanes' accesses stay within
+// (12.5) 15.8 -> 11.4, A~^T of the power-law LP 43.8 -> 35.4, A~^T of the
+// transportation LP 2000 x 2000 (2) 77 -> 52.  Windows: the lanes' accesses stay within
 // a window, so wider ones sort better but scatter more: A~^T of the power-law
 // LP 36.6 / 39.2 / 42.2 us at 64 / 128 / 256 rows.  Cutting longer rows into
 // chunks did not pay: power-law A~ (rows up to 20,000) 49 us against the tiles'
@@ -29,7 +30,6 @@ namespace pdhg {
 __host__ __device__ constexpr int slice_steps(int w) { return w & 0xff; }
 __host__ __device__ constexpr int slice_lg(int w) { return (w >> 8) & 15; }
 __host__ __device__ constexpr int slice_nrows(int w) { return (w >> 12) & 63; }
-__host__ __device__ constexpr int slice_first(int w) { return w >> 18; }
 
 // Sums of a slice: lane l gets the row l >> lg.  Four steps at a time with the
 // next four's values and columns in flight; the last w mod 4 are loaded and
