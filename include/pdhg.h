@@ -125,8 +125,10 @@ typedef struct pdhg_options {
   double pid_kp;           /* proportional gain (default 0.99)                  */
   double pid_ki;           /* integral gain (default 0.01)                      */
   double pid_kd;           /* derivative gain (default 0)                       */
-  int32_t persistent;      /* batched contexts: 0 (default): each F-iteration
-                              chunk is a CUDA graph of per-half-step launches;
+  int32_t persistent;      /* batched contexts: 0 (default): LPs that fit on
+                              chip by a thread-block cluster each, else each
+                              F-iteration chunk as a CUDA graph of
+                              per-half-step launches;
                               1: the whole solve is one cooperative launch
                               (every block resident), the phases separated by
                               grid-wide barriers whose waits are bounded; it
@@ -134,7 +136,8 @@ typedef struct pdhg_options {
                               (full tiles) whatever the tuner picked           */
   int32_t wait_limit_ms;   /* bound of one device-side wait (default 1000): a
                               grid barrier of the persistent batched solve,
-                              or the bulk copy of a column panel of the
+                              another CTA's vector in an on-chip solve, or the
+                              bulk copy of a column panel of the
                               gathered vector; a wait past it ends the solve
                               with PDHG_TIMEOUT                               */
   int32_t wait_test;       /* 1: every grid barrier waits for one arrival more
@@ -301,10 +304,9 @@ pdhg_status pdhg_get_kernel_timing_parts(pdhg_ctx* ctx, double* ms, int64_t* sam
  * stream on its current iterate.  With options.step_rule = 1 the half-steps
  * are the adaptive step's own: the primal also saves the accepted state
  * and writes the attempt's x beside it, the dual also forms A~ times the
- * move and applies the acceptance test, followed by the kernel that undoes a
- * rejected attempt (timed with the dual).  Launches are back to back as in a solve
+ * move and applies the acceptance test.  Launches are back to back as in a solve
  * (programmatic dependent launch), with no event between them.  A context
- * whose LP is solved on chip (constant step, tile_nnz = 0, spmv_layout = 0,
+ * whose LP is solved on chip (float64, constant step, tile_nnz = 0, spmv_layout = 0,
  * kernel_timing = 0, vectors that fit in a cluster's shared memory) has no
  * half-step kernels of its own: the tile kernels are timed.  The solver
  * state is saved to a temporary device buffer first and restored after, so
@@ -314,7 +316,8 @@ pdhg_status pdhg_time_kernels(pdhg_ctx* ctx, int32_t reps, double* ms);
 /* Tile schedule picked for A (dual kernel) and A^T (primal kernel): nonzeros
  * per tile (at most), threads per block, tiles, and the SpMV variant (8, 16,
  * 32: segmented with that many nonzeros per thread; -4, -8: vector with that
- * many lanes per row).  Any pointer may be NULL.  */
+ * many lanes per row; 64: row-sorted slices, a warp each, of which a tile is a
+ * block's worth).  Any pointer may be NULL.  */
 pdhg_status pdhg_get_schedule(pdhg_ctx* ctx, int32_t* a_tile_nnz, int32_t* a_block,
                               int32_t* a_tiles, int32_t* at_tile_nnz, int32_t* at_block,
                               int32_t* at_tiles, int32_t* a_variant, int32_t* at_variant);
