@@ -29,8 +29,8 @@ constexpr int kResThreads = 512, kResWarps = kResThreads / 32;
 constexpr int kResShort = 24;   // a lane per row up to this many nonzeros
 constexpr int kResMid = 256;    // 8 lanes per row up to this many, a warp above
 constexpr int kResMaxC = 16;    // CTAs of a cluster (16 needs the non-portable size)
-// What is solved on chip, and by how many CTAs (us per iteration, one LP, GB300;
-// tile kernels: 10 at 200 x 500, 11.4 at 2000 x 5000):
+// What is solved on chip, and by how many CTAs (us per iteration, one LP, GB300,
+// one lane per short row; tile kernels: 10 at 200 x 500, 11.4 at 2000 x 5000):
 //   float64, clusters of 1 / 4 / 16: 60 x 150 2.4 / 2.6 / 2.7, 200 x 500 3.4 /
 //   2.5 / 2.7, 2000 x 5000 23.7 / 7.1 / 3.7; float32: 1.1 / 1.3 / 1.5, 1.4 / 1.4
 //   / 1.5, 9.8 / 3.1 / 2.3.
