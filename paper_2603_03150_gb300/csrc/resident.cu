@@ -219,7 +219,8 @@ __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
     X[lp.n] = 0.0;
     Y[lp.m] = 0.0;
   }
-  ResExchange<C> ex(cl, L, smem, A.wait_ns, (uint32_t)lp.n * 8u, (uint32_t)lp.m * 8u, 2, 2);
+  ResExchange<C> ex(cl, L, smem, A.wait_ns, (uint32_t)lp.n * 8u, (uint32_t)lp.m * 8u, 2, 2,
+                    res_idle(Ma, Mt));
   double lam = 0.0, lam_prev = 0.0, inv = A.max_iter > 0 ? 1.0 : 0.0;
   int k = 0;  // steps whose w has been computed
   cl.sync();
@@ -504,6 +505,14 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
     resident_free(ctx);
     return PDHG_OK;
   }
+  // A CTA without a slice of either matrix would have no warp that is held to the
+  // others' phases.  (A CTA's share of the work is at least kResMinOps
+  // operations, so every CTA of a cluster has slices.)
+  for (const ResLp& p : lps)
+    if (std::max(p.a_slices, p.t_slices) < p.C) {
+      resident_free(ctx);
+      return PDHG_OK;
+    }
   int64_t ea = 0, et = 0;
   for (int l = 0; l < count; ++l) {
     lps[l].a_el = ea;

@@ -17,8 +17,19 @@
 // Slice s belongs to CTA s mod C of the cluster and warp (s / C) mod kResWarps
 // of it: always the same lane works on a row, so the row's own operands need
 // no barrier.  Every CTA holds the whole gathered vectors; a new entry is
-// written to all C copies through distributed shared memory, and one cluster
-// barrier separates the half-steps.
+// written to all C copies through distributed shared memory.
+//
+// Who waits.  A half-step ends for a warp when its CTA's transaction barrier has
+// counted the whole vector.  The wait names a phase by its parity alone, so a
+// warp must have seen a phase before the next one completes.  Two things hold a
+// warp to that: it has rows (the vector after next cannot be complete without
+// them, and it computes them behind the wait), or it is warp 0, whose thread
+// arms the barrier's next phase.  A warp without a slice of either matrix has
+// neither: the LP 200 x 500 leaves 12 of a CTA's 16 warps in that state, and one
+// that was a whole iteration late would have taken a phase that is over for one
+// that never ends.  It reads no vector, so it does not wait for them: the block
+// barriers that all warps meet (every 64 iterations and at an evaluation in the
+// solve, in every sum of the power iteration and the conjugate gradients) hold it.
 #pragma once
 #include "common.cuh"
 #include "kernels.h"
@@ -192,7 +203,8 @@ struct ResCluster {
   }
   // waits until the vector counted by barrier `bar` has arrived (phase parity)
   // and lets thread 0 expect the next one; false (for the whole warp) once a
-  // lane's wait ran past limit_ns
+  // lane's wait ran past limit_ns.  Only for warps that cannot miss a phase (see
+  // the head of this file).
   __device__ __forceinline__ bool arrived(uint32_t bar, uint32_t parity, uint32_t bytes,
                                           unsigned long long limit_ns) const {
     const uint32_t mb = base + bar;
@@ -314,7 +326,7 @@ __device__ __forceinline__ void res_dot(const ResSlice& s, const TV* __restrict_
 // One matrix of an LP as a CTA sees it; f(slice, row of this lane or -1) for
 // the CTA's slices of this warp (row -1: a lane without a row of its own).
 // The first slice's descriptor stays in registers, the next one's is loaded
-// ahead.
+// ahead.  empty(): the warp has no slice.
 struct ResMat {
   const ResSlice* sl;
   const uint16_t* col;
@@ -324,6 +336,7 @@ struct ResMat {
       : sl(sl_), col(col_), slices(n), s0(rank + (int)(threadIdx.x >> 5) * C) {
     first = s0 < n ? __ldg(reinterpret_cast<const int4*>(sl + s0)) : make_int4(0, 0, 0, 0);
   }
+  __device__ __forceinline__ bool empty() const { return s0 >= slices; }
   template <int C, class F>
   __device__ __forceinline__ void each(F&& f) const {
     const int lane = threadIdx.x & 31;
@@ -336,6 +349,11 @@ struct ResMat {
     }
   }
 };
+
+// a warp that no vector has to arrive for (see the head of this file)
+__device__ __forceinline__ bool res_idle(const ResMat& a, const ResMat& b) {
+  return threadIdx.x >= 32 && a.empty() && b.empty();
+}
 
 // Sums of NQ quantities over the cluster, the same bits on every CTA: the
 // block's sums to every CTA's record of this rank, a cluster barrier, then the
@@ -366,9 +384,10 @@ __device__ __forceinline__ bool res_reduce(const ResCluster<C>& cl, const ResSme
 // Exchanges of an iteration that needs sums besides the two vectors (the power
 // iteration, the conjugate gradients): barrier 0 counts X, 1 Y, 2 and 3 the
 // records of two sums.  Each barrier goes through one phase per iteration.  A
-// CTA may be one exchange ahead of another, never two: each exchange waits for
-// every CTA's part, so a record is read everywhere before its slot is written
-// again.
+// CTA may be one exchange ahead of another, never two: each sum waits for every
+// CTA's part, so a record is read everywhere before its slot is written again.
+// All warps wait for the sums (each ends with a block barrier, and its next
+// phase needs records sent behind it); idle ones do not wait for X and Y.
 template <int C>
 struct ResExchange {
   const ResCluster<C>& cl;
@@ -377,12 +396,13 @@ struct ResExchange {
   unsigned long long wait_ns;
   uint32_t bytes_x, bytes_y;
   int nq0, nq1;        // quantities of the two sums
+  bool idle;           // this warp (res_idle)
   uint32_t phase = 0;
   bool lost = false;  // a wait ran out (uniform in a warp)
   __device__ __forceinline__ ResExchange(const ResCluster<C>& c, const ResSmem& l, unsigned char* s,
                                          unsigned long long limit, uint32_t bx, uint32_t by,
-                                         int q0, int q1)
-      : cl(c), L(l), smem(s), wait_ns(limit), bytes_x(bx), bytes_y(by), nq0(q0), nq1(q1) {
+                                         int q0, int q1, bool idle_)
+      : cl(c), L(l), smem(s), wait_ns(limit), bytes_x(bx), bytes_y(by), nq0(q0), nq1(q1), idle(idle_) {
     if (C > 1 && threadIdx.x == 0)
       for (int b = 0; b < 4; ++b) {
         mbar_init(cl.base + L.bar + 8u * b);
@@ -397,7 +417,7 @@ struct ResExchange {
   __device__ __forceinline__ void wait(int b) {
     if constexpr (C == 1)
       __syncthreads();
-    else if (!lost)
+    else if (!lost && !(idle && b < 2))
       lost = !cl.arrived(L.bar + 8u * b, phase, expect(b), wait_ns);
   }
   // NQ sums over the cluster, the same bits in every thread; slot 0 or 1, each

@@ -110,7 +110,8 @@ __global__ void __launch_bounds__(kResThreads) k_res_cg(ResCg A) {
   const double *tv = A.t_val + lp.t_el, *av = A.a_val + lp.a_el;
   const uint16_t* on = A.ord_n + lp.n_off;
   const int32_t* bcol = A.bcol + lp.n_off;
-  ResExchange<C> ex(cl, L, smem, A.wait_ns, (uint32_t)lp.n * 8u, (uint32_t)lp.m * 8u, 2, 1);
+  ResExchange<C> ex(cl, L, smem, A.wait_ns, (uint32_t)lp.n * 8u, (uint32_t)lp.m * 8u, 2, 1,
+                    res_idle(Ma, Mt));
   if (tid == 0) {
     X[lp.n] = 0.0;
     Y[lp.m] = 0.0;

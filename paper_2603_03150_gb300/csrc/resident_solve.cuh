@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
   const uint32_t bar_x = L.bar, bar_y = L.bar + 8u;
   const uint32_t bytes_x = (uint32_t)(lp.n * sizeof(T)), bytes_y = (uint32_t)(lp.m * sizeof(T));
   uint32_t phase = 0;  // the parity of both barriers' current phase
+  const bool idle = C > 1 && res_idle(Ma, Mt);
   if (C > 1 && tid == 0) {
     mbar_init(cl.base + bar_x);
     mbar_init(cl.base + bar_y);
@@ -110,10 +111,16 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
     const int len = (int)(next - k0);
     const T tau = (T)sc.tau, sigma = (T)sc.sigma;
     for (int i = 0; i < len; ++i) {
-      if ((i & 63) == 0) {  // the next 64 weights (one float64 division each)
-        if (tid < 64) {
-          const long long tt = tt0 + i + tid;
-          tab[tid] = hal ? halpern_weight(tt + 1, T(0)) : avg_weight(tt + 1, T(0));
+      if ((i & 63) == 0) {
+        // The next 64 weights (a float64 division each), by warp 0: it has seen
+        // the last Y complete, so every warp with rows has taken its last weight;
+        // a warp without rows may be here while the others still read the table.
+        if (tid < 32) {
+#pragma unroll
+          for (int e = tid; e < 64; e += 32) {
+            const long long tt = tt0 + i + e;
+            tab[e] = hal ? halpern_weight(tt + 1, T(0)) : avg_weight(tt + 1, T(0));
+          }
         }
         lost = __syncthreads_or(lost);
         if (lost) break;
@@ -138,7 +145,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
         }
       });
       if constexpr (C == 1) cl.sync();
-      else if (!lost) lost = !cl.arrived(bar_x, phase, bytes_x, A.wait_ns);
+      else if (!lost && !idle) lost = !cl.arrived(bar_x, phase, bytes_x, A.wait_ns);
       Ma.template each<C>([&](const ResSlice& s, int row) {
         const T* const buf[1] = {X};
         T h1[1] = {T(0)};
@@ -161,7 +168,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
         }
       });
       if constexpr (C == 1) cl.sync();
-      else if (!lost) lost = !cl.arrived(bar_y, phase, bytes_y, A.wait_ns);
+      else if (!lost && !idle) lost = !cl.arrived(bar_y, phase, bytes_y, A.wait_ns);
       phase ^= 1u;
     }
     // a wait that ran out: tell every CTA (each comes to the next cluster
