@@ -141,9 +141,11 @@ typedef struct pdhg_options {
                               gathered vector; a wait past it ends the solve
                               with PDHG_TIMEOUT                               */
   int32_t wait_test;       /* 1: every grid barrier waits for one arrival more
-                              than the grid has, and every column-panel load
-                              for 16 bytes more than its copies deliver, so
-                              the bounded waits run out (tests the
+                              than the grid has, every column-panel load for 16
+                              bytes more than its copies deliver, and every
+                              exchange between the CTAs of an LP solved on chip
+                              by more than one for 8 bytes more than they send,
+                              so the bounded waits run out (tests the
                               PDHG_TIMEOUT path; default 0)                   */
   int32_t step_rule;       /* 0 (default): constant step eta = eta_safety /
                               sigma_max; 1: PDLP's adaptive step (Applegate et

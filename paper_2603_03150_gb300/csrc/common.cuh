@@ -498,6 +498,10 @@ __device__ __forceinline__ void mbar_arrive_expect(uint32_t mb, uint32_t bytes) 
                "r"(bytes)
                : "memory");
 }
+// counts `bytes` as arrived without any
+__device__ __forceinline__ void mbar_complete_tx(uint32_t mb, uint32_t bytes) {
+  asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(bytes) : "memory");
+}
 // global [src, src + bytes) -> shared dst (both 16-byte aligned, bytes a
 // multiple of 16), completing on the barrier mb
 __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uint32_t bytes,

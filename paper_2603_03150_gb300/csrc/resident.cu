@@ -198,6 +198,7 @@ struct ResPower {
   int max_iter;
   double rel_tol;
   unsigned long long wait_ns;
+  uint32_t tx_extra;
   int32_t* err;  // 1 once a wait between CTAs ran out
 };
 template <int C>
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
     Y[lp.m] = 0.0;
   }
   ResExchange<C> ex(cl, L, smem, A.wait_ns, (uint32_t)lp.n * 8u, (uint32_t)lp.m * 8u, 2, 2,
-                    res_idle(Ma, Mt));
+                    A.tx_extra, res_idle(Ma, Mt));
   double lam = 0.0, lam_prev = 0.0, inv = A.max_iter > 0 ? 1.0 : 0.0;
   int k = 0;  // steps whose w has been computed
   cl.sync();
@@ -268,8 +269,10 @@ __global__ void __launch_bounds__(kResThreads) k_res_power(ResPower A) {
     ex.wait(0);
     ex.next();
   }
-  if (__syncthreads_or(ex.lost) && tid == 0) atomicExch(A.err, 1);
-  cl.sync();  // no CTA leaves while another may still write to it
+  if (ex.finish()) {
+    if (tid == 0) atomicExch(A.err, 1);
+    return;
+  }
   if (cl.rank == 0 && tid == 0) {
     PowerState p{};
     p.lam = lam;
@@ -545,7 +548,7 @@ pdhg_status resident_power(pdhg_ctx* ctx) {
   ResData* d = res_of(ctx);
   ResPower A{d->lp,    nullptr,  d->a_sl, d->t_sl, d->a_col, d->t_col,
              d->a_val, d->t_val, ctx->ps, ctx->opt.power_max_iter, ctx->opt.power_rel_tol,
-             (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull, d->active + 1};
+             (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull, res_tx_extra(ctx), d->active + 1};
   CKS(res_groups(ctx, d->groups, d->side, [&](const ResGroup& g, cudaStream_t s) {
     A.list = d->list + g.first;
     cudaLaunchAttribute attr;
@@ -588,6 +591,7 @@ static pdhg_status res_solve(pdhg_ctx* ctx, const IterBuffers<T>& B, int32_t* ac
   A.active = active;
   A.slice_ns = 100000000ull;
   A.wait_ns = (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull;
+  A.tx_extra = res_tx_extra(ctx);
   A.err = d->active + 1;
   return res_groups(ctx, d->groups, d->side, [&](const ResGroup& g, cudaStream_t s) {
     A.list = d->list + g.first;

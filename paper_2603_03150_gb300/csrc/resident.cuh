@@ -106,7 +106,7 @@ __host__ __device__ inline ResSmem res_smem(int m, int n, int own_m, int own_n, 
     return at;
   };
   r.sc = take(sizeof(Scalars));
-  r.rec = take(kResMaxC * 18 * 8);   // one record per CTA: 16 sums, 1 flag
+  r.rec = take(kResMaxC * 18 * 8);   // one record per CTA: 16 sums, 2 flags
   r.red = take(nvm ? 16 * kResWarps * 8 : (2 * kResThreads + 8) * 8);  // (no vectors of rows: ResExchange)
   r.tab = take(64 * 8);              // averaging weights of 64 iterations
   r.bar = take(32);                  // transaction barriers: X, Y and two sums
@@ -225,6 +225,23 @@ struct ResCluster {
     const bool ok = __all_sync(0xffffffffu, done != 0);
     if (threadIdx.x == 0 && ok) mbar_arrive_expect(mb, bytes);
     return ok;
+  }
+  // Thread 0, on its way out after a wait that ran out: waits until everything
+  // that was sent to this CTA over barrier `bar` has arrived.  A CTA must not
+  // exit while a store is on its way to it, and neither a cluster barrier nor a
+  // delay tells that none is.  The barrier counts bytes: thread 0 has let it
+  // expect `armed` so far (the last phase, of the given parity, is the one that
+  // is open), and all CTAs together have sent `sent`.  What was expected and
+  // not sent is counted as arrived; what was sent beyond it (a CTA may be one
+  // exchange ahead) is a phase of its own.  Bounded by limit_ns a phase.
+  __device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, long long sent, long long armed,
+                                        unsigned long long limit_ns) const {
+    const uint32_t mb = base + bar;
+    if (sent < armed) mbar_complete_tx(mb, (uint32_t)(armed - sent));
+    if (mbar_wait(mb, parity, limit_ns) && sent > armed) {
+      mbar_arrive_expect(mb, (uint32_t)(sent - armed));
+      mbar_wait(mb, parity ^ 1u, limit_ns);
+    }
   }
 };
 
@@ -390,19 +407,24 @@ __device__ __forceinline__ bool res_reduce(const ResCluster<C>& cl, const ResSme
 // phase needs records sent behind it); idle ones do not wait for X and Y.
 template <int C>
 struct ResExchange {
+  static constexpr int kFlags = 4 * kResMaxC, kCounts = 5 * kResMaxC;  // in the records, behind the sums
   const ResCluster<C>& cl;
   const ResSmem& L;
   unsigned char* smem;
   unsigned long long wait_ns;
   uint32_t bytes_x, bytes_y;
   int nq0, nq1;        // quantities of the two sums
+  uint32_t extra;      // bytes every phase expects and nobody sends (wait_test)
   bool idle;           // this warp (res_idle)
   uint32_t phase = 0;
-  bool lost = false;  // a wait ran out (uniform in a warp)
+  bool lost = false;  // a wait ran out (uniform in a warp, which sends nothing more)
+  uint32_t sent[4] = {}, seen[4] = {};  // per barrier: values sent, phases seen complete
   __device__ __forceinline__ ResExchange(const ResCluster<C>& c, const ResSmem& l, unsigned char* s,
                                          unsigned long long limit, uint32_t bx, uint32_t by,
-                                         int q0, int q1, bool idle_)
-      : cl(c), L(l), smem(s), wait_ns(limit), bytes_x(bx), bytes_y(by), nq0(q0), nq1(q1), idle(idle_) {
+                                         int q0, int q1, uint32_t extra_, bool idle_)
+      : cl(c), L(l), smem(s), wait_ns(limit), bytes_x(bx), bytes_y(by), nq0(q0), nq1(q1), extra(extra_),
+        idle(idle_) {
+    if (C > 1 && threadIdx.x < kResMaxC) reinterpret_cast<double*>(smem + L.rec)[kFlags + threadIdx.x] = 0.0;
     if (C > 1 && threadIdx.x == 0)
       for (int b = 0; b < 4; ++b) {
         mbar_init(cl.base + L.bar + 8u * b);
@@ -410,15 +432,38 @@ struct ResExchange {
       }
   }
   __device__ __forceinline__ uint32_t expect(int b) const {
-    return b == 0 ? bytes_x : b == 1 ? bytes_y : (uint32_t)(C * 8 * (b == 2 ? nq0 : nq1));
+    return extra + (b == 0 ? bytes_x : b == 1 ? bytes_y : (uint32_t)(C * 8 * (b == 2 ? nq0 : nq1)));
   }
-  __device__ __forceinline__ void send_x(int p, double v) const { cl.send(L.X + 8u * p, L.bar, v); }
-  __device__ __forceinline__ void send_y(int p, double v) const { cl.send(L.Y + 8u * p, L.bar + 8u, v); }
+  __device__ __forceinline__ void send_x(int p, double v) {
+    if (lost) return;
+    cl.send(L.X + 8u * p, L.bar, v);
+    sent[0] += 1;
+  }
+  __device__ __forceinline__ void send_y(int p, double v) {
+    if (lost) return;
+    cl.send(L.Y + 8u * p, L.bar + 8u, v);
+    sent[1] += 1;
+  }
+  // this rank's record of quantity q, by a whole warp: lane r's to rank r
+  __device__ __forceinline__ void send_record(int slot, int q, double v) {
+    if (lost) return;
+    if ((threadIdx.x & 31) < C)
+      cl.send_to(threadIdx.x & 31, L.rec + (uint32_t)(slot * 2 * kResMaxC + q * kResMaxC + cl.rank) * 8u,
+                 L.bar + 16u + 8u * slot, v);
+    sent[2] += slot == 0;
+    sent[3] += slot != 0;
+  }
+  __device__ __forceinline__ void wait(int b, uint32_t parity) {
+    if (lost || (idle && b < 2)) return;
+    lost = !cl.arrived(L.bar + 8u * b, parity, expect(b), wait_ns);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) seen[e] += !lost && e == b;
+  }
   __device__ __forceinline__ void wait(int b) {
     if constexpr (C == 1)
       __syncthreads();
-    else if (!lost && !(idle && b < 2))
-      lost = !cl.arrived(L.bar + 8u * b, phase, expect(b), wait_ns);
+    else
+      wait(b, phase);
   }
   // NQ sums over the cluster, the same bits in every thread; slot 0 or 1, each
   // once per iteration.  The threads' shares go through shared memory to one
@@ -439,9 +484,7 @@ struct ResExchange {
     __syncthreads();
     if (warp < NQ) {
       double t = block_share(red + warp * kResThreads + lane);
-      const uint32_t bar = L.bar + 16u + 8u * slot;
-      if (lane < C)
-        cl.send_to(lane, L.rec + (uint32_t)(slot * 2 * kResMaxC + warp * kResMaxC + cl.rank) * 8u, bar, t);
+      send_record(slot, warp, t);
       if (C > 1) {
         // the records of every CTA, in a tree
         wait(2 + slot);
@@ -481,17 +524,14 @@ struct ResExchange {
     for (int e = 0; e < NQ; ++e) red[e * kResThreads + threadIdx.x] = v[e];
     __syncthreads();
     if (q < 0) return;
-    const double t = block_share(red + q * kResThreads + lane);
-    if (lane < C)
-      cl.send_to(lane, L.rec + (uint32_t)(slot * 2 * kResMaxC + q * kResMaxC + cl.rank) * 8u,
-                 L.bar + 16u + 8u * slot, t);
+    send_record(slot, q, block_share(red + q * kResThreads + lane));
   }
   template <int NQ, class F>
   __device__ __forceinline__ bool sum_end(int slot, uint32_t parity, double (&res)[NQ][2], F&& fin) {
     const int lane = threadIdx.x & 31, q = (int)(threadIdx.x >> 5) - (kResWarps - NQ);
     double* out = reinterpret_cast<double*>(smem + L.red) + 2 * kResThreads;
     const double* rec = reinterpret_cast<const double*>(smem + L.rec) + slot * 2 * kResMaxC;
-    if (C > 1 && !lost) lost = !cl.arrived(L.bar + 16u + 8u * slot, parity, expect(2 + slot), wait_ns);
+    if (C > 1) wait(2 + slot, parity);
     if (q >= 0) {
       double r = lane < C ? rec[q * kResMaxC + lane] : 0.0;
 #pragma unroll
@@ -530,6 +570,37 @@ struct ResExchange {
   __device__ __forceinline__ bool ends(bool stop) const { return __syncthreads_or(stop || lost); }
   // ends an iteration that used every barrier once
   __device__ __forceinline__ void next() { phase ^= 1u; }
+  // Ends the kernel's exchanges (all threads of all CTAs): whether a wait ran out
+  // in any CTA of the cluster.  Without one, everything sent has arrived, since
+  // every CTA has waited for it.  With one, the CTAs tell each other how much
+  // they have sent, and each waits for what is still on its way to it.
+  __device__ __forceinline__ bool finish() {
+    if constexpr (C == 1) return false;
+    const double* rec = reinterpret_cast<const double*>(smem + L.rec);
+    if (__syncthreads_or(lost) && threadIdx.x == 0) cl.push(L.rec + (uint32_t)(kFlags + cl.rank) * 8u, 1.0);
+    cl.sync();
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < C; ++q) any |= rec[kFlags + q] != 0.0;
+    if (!any) return false;
+    double v[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b)  // (a record is sent to each CTA by a lane of its own)
+      v[b] = b < 2 || (threadIdx.x & 31) == 0 ? (double)sent[b] : 0.0;
+    double* red = reinterpret_cast<double*>(smem + L.red);
+    double* mine = red + 2 * kResThreads;
+    block_sum_scatter<kResThreads, 4>(v, red, mine);
+    if (threadIdx.x < 4) cl.push(L.rec + (uint32_t)(kCounts + 4 * cl.rank + threadIdx.x) * 8u, mine[threadIdx.x]);
+    cl.sync();
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        double all = 0.0;
+        for (int q = 0; q < C; ++q) all += rec[kCounts + 4 * q + b];
+        cl.drain(L.bar + 8u * b, seen[b] & 1u, 8ll * (long long)all, (1ll + seen[b]) * expect(b), wait_ns);
+      }
+    return true;
+  }
 };
 
 #define RES_DISPATCH_C(c, ...)  \
@@ -615,6 +686,7 @@ struct ResSolve {
   int32_t* active;        // LPs not finished
   unsigned long long slice_ns;
   unsigned long long wait_ns;  // bound of a wait for another CTA's vector
+  uint32_t tx_extra;           // bytes each such wait expects and nobody sends (wait_test)
   int32_t* err;                // 1 once such a wait ran out
 };
 

@@ -83,6 +83,7 @@ struct ResCg {
   double tol2;
   int max_iter;
   unsigned long long wait_ns;
+  uint32_t tx_extra;
   int32_t* err;
 };
 
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_cg(ResCg A) {
   const uint16_t* on = A.ord_n + lp.n_off;
   const int32_t* bcol = A.bcol + lp.n_off;
   ResExchange<C> ex(cl, L, smem, A.wait_ns, (uint32_t)lp.n * 8u, (uint32_t)lp.m * 8u, 2, 1,
-                    res_idle(Ma, Mt));
+                    A.tx_extra, res_idle(Ma, Mt));
   if (tid == 0) {
     X[lp.n] = 0.0;
     Y[lp.m] = 0.0;
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_cg(ResCg A) {
       ex.next();
     }
   }
-  if (ex.ends(false)) {
+  if (ex.finish()) {
     if (tid == 0) atomicExch(A.err, 1);
   } else {
     Mt.template each<C>([&](const ResSlice& s, int row) {
@@ -216,7 +217,6 @@ __global__ void __launch_bounds__(kResThreads) k_res_cg(ResCg A) {
     });
     if (cl.rank == 0 && tid == 0) A.iters[l] = it;
   }
-  cl.sync();  // no CTA leaves while another may still write to it
 }
 
 const void* cg_kernel(int C) {
@@ -391,7 +391,7 @@ pdhg_status resident_cg(pdhg_ctx* ctx, ResCgData* d, bool original, const double
   }
   ResCg A{d->lp,   nullptr, d->a_sl,      d->t_sl,      d->a_col, d->t_col, d->ord_n,
           d->val[o][0], d->val[o][1], d->bcol, rhs, w, d->iters, tol * tol, max_iter,
-          (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull, d->flags + 1};
+          (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull, res_tx_extra(ctx), d->flags + 1};
   CKS(res_groups(ctx, d->groups, d->side, [&](const ResGroup& g, cudaStream_t q) {
     A.list = d->list + g.first;
     cudaLaunchAttribute attr;

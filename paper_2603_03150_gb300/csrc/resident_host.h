@@ -56,6 +56,9 @@ pdhg_status res_groups(pdhg_ctx* ctx, const std::vector<ResGroup>& groups, const
   return PDHG_OK;
 }
 
+// bytes beyond those sent that a wait between CTAs expects
+inline uint32_t res_tx_extra(const pdhg_ctx* ctx) { return ctx->opt.wait_test ? 8u : 0u; }
+
 std::vector<int> res_clusters(const pdhg_ctx* ctx, const std::vector<double>& ops, double min_ops,
                               const std::function<bool(int, int)>& fits);
 std::vector<int32_t> res_order(const std::vector<ResLp>& lps, const std::vector<double>& ops);

@@ -56,7 +56,8 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
   const uint16_t* om = A.ord_m + lp.m_off;
   // X and Y of an iteration travel by transaction-counted stores
   const uint32_t bar_x = L.bar, bar_y = L.bar + 8u;
-  const uint32_t bytes_x = (uint32_t)(lp.n * sizeof(T)), bytes_y = (uint32_t)(lp.m * sizeof(T));
+  const uint32_t bytes_x = (uint32_t)(lp.n * sizeof(T)) + A.tx_extra,
+                 bytes_y = (uint32_t)(lp.m * sizeof(T)) + A.tx_extra;
   uint32_t phase = 0;  // the parity of both barriers' current phase
   const bool idle = C > 1 && res_idle(Ma, Mt);
   if (C > 1 && tid == 0) {
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
     mbar_arrive_expect(cl.base + bar_y, bytes_y);
   }
   if (tid < kResMaxC) reinterpret_cast<double*>(smem + L.rec)[tid * 18 + 17] = 0.0;
-  bool lost = false;  // a wait ran out
+  bool lost = false;  // a wait ran out (uniform in a warp, which sends nothing more)
   auto push_x = [&](int p, T v) { cl.push(L.X + (uint32_t)p * (uint32_t)sizeof(T), v); };
   auto push_y = [&](int p, T v) { cl.push(L.Y + (uint32_t)p * (uint32_t)sizeof(T), v); };
   cl.sync();  // every CTA of the cluster has started (its shared memory may be written)
@@ -110,6 +111,8 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
     const long long next = min((k0 / F + 1) * F, sc.max_iter);
     const int len = (int)(next - k0);
     const T tau = (T)sc.tau, sigma = (T)sc.sigma;
+    const uint32_t phase0 = phase;
+    int sent = 0, seen = 0;  // half-steps of this chunk that the warp has computed, seen arrive
     for (int i = 0; i < len; ++i) {
       if ((i & 63) == 0) {
         // The next 64 weights (a float64 division each), by warp 0: it has seen
@@ -127,7 +130,7 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
       }
       const T w = tab[i & 63];
       const bool first = tt0 + i == 0;
-      Mt.template each<C>([&](const ResSlice& s, int row) {
+      if (C == 1 || !lost) Mt.template each<C>([&](const ResSlice& s, int row) {
         const T* const buf[1] = {Y};
         const int p = s.p0 + row, k = s.loc + row;
         T d[1] = {row >= 0 ? cc[k] : T(0)};  // c~ - A~^T y, the sum starting at c~
@@ -144,9 +147,11 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
           xa[k] = first ? xn : a + (xn - a) * w;
         }
       });
+      sent += !lost;
       if constexpr (C == 1) cl.sync();
       else if (!lost && !idle) lost = !cl.arrived(bar_x, phase, bytes_x, A.wait_ns);
-      Ma.template each<C>([&](const ResSlice& s, int row) {
+      seen += !lost;
+      if (C == 1 || !lost) Ma.template each<C>([&](const ResSlice& s, int row) {
         const T* const buf[1] = {X};
         T h1[1] = {T(0)};
         res_dot<1, false>(s, av, Ma.col, buf, h1);
@@ -167,8 +172,10 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
           axa[k] = first ? h : b + (h - b) * w;
         }
       });
+      sent += !lost;
       if constexpr (C == 1) cl.sync();
       else if (!lost && !idle) lost = !cl.arrived(bar_y, phase, bytes_y, A.wait_ns);
+      seen += !lost;
       phase ^= 1u;
     }
     // a wait that ran out: tell every CTA (each comes to the next cluster
@@ -189,10 +196,19 @@ __global__ void __launch_bounds__(kResThreads) k_res_solve(ResSolve<T> A) {
       bool any = false;
 #pragma unroll
       for (int q = 0; q < C; ++q) any |= reinterpret_cast<const double*>(smem + L.rec)[q * 18 + 17] != 0.0;
-      if (any) {  // the whole cluster leaves together, its last stores given time to land
+      if (any) {  // the whole cluster leaves, each CTA when what was sent to it has arrived
         if (tid == 0) atomicExch(A.err, 1);
-        __nanosleep(100000);
-        cl.sync();
+        double n[2] = {0.0, 0.0};
+        Mt.template each<C>([&](const ResSlice&, int row) { n[0] += row >= 0; });
+        Ma.template each<C>([&](const ResSlice&, int row) { n[1] += row >= 0; });
+        n[0] *= (sent + 1) / 2;
+        n[1] *= sent / 2;
+        res_reduce<2>(cl, L, smem, n, tot);
+        if (tid == 0) {
+          const int x = (seen + 1) / 2, y = seen / 2;
+          cl.drain(bar_x, phase0 ^ (x & 1), (long long)tot[0] * sizeof(T), (1ll + x) * bytes_x, A.wait_ns);
+          cl.drain(bar_y, phase0 ^ (y & 1), (long long)tot[1] * sizeof(T), (1ll + y) * bytes_y, A.wait_ns);
+        }
         return;
       }
     }

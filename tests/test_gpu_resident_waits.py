@@ -64,3 +64,78 @@ def test_power_iteration_many_times(name):
         with pdhg.Solver.from_lp(lp, power_rel_tol=0.0, power_max_iter=2000) as s:
             sigma.add(s.scaling()["sigma_max"])
     assert len(sigma) == 1
+
+
+def gives_up(create, call=None):
+    """create() or call(solver) ends with an error status; the GPU stays usable."""
+    if call is None:
+        with pytest.raises(pdhg.PDHGError):
+            create()
+    else:
+        with create() as s:
+            for _ in range(2):
+                call(s)
+    lp = lpgen.planted_lp(200, 500, seed=1)
+    with pdhg.Solver.from_lp(lp) as s:
+        assert s.solve(1e-4, 20_000) == pdhg.PDHG_CONVERGED
+
+
+# clusters of 2, 4, 8 and 16 CTAs, and of CTAs without rows of a matrix
+CLUSTERS = {f"planted_{m}": (lambda m=m: lpgen.planted_lp(m, 5 * m // 2, seed=m)) for m in (100, 200, 400, 900)}
+CLUSTERS.update({k: v for k, v in MAKERS.items() if k != "idle_warps"})
+
+
+@pytest.mark.parametrize("method", ["averaged", "halpern"])
+@pytest.mark.parametrize("name", list(CLUSTERS))
+def test_solve_whose_wait_runs_out(name, method):
+    """options.wait_test makes each exchange expect 8 bytes that nobody sends
+    (without a power iteration, which would give up first)."""
+    lp = CLUSTERS[name]()
+
+    def call(s):
+        assert s.solve(1e-4, 1000) == pdhg.PDHG_TIMEOUT
+
+    gives_up(lambda: pdhg.Solver.from_lp(lp, method=method, power_max_iter=0, wait_test=True, wait_limit_ms=5), call)
+
+
+def test_batch_whose_waits_run_out():
+    """LPs of every cluster size, one of a single CTA (which has no exchanges)."""
+    lps = [lpgen.planted_lp(m, 5 * m // 2, seed=m) for m in (12, 200, 400, 800, 1600)]
+
+    def call(s):
+        assert s.solve(1e-4, 1000) == pdhg.PDHG_TIMEOUT
+        assert list(s.lp_status) == [pdhg.PDHG_TIMEOUT] * len(lps)
+
+    for precision in ("fp64", "fp32"):
+        gives_up(lambda: pdhg.BatchSolver(lps, precision=precision, power_max_iter=0, wait_test=1, wait_limit_ms=5), call)
+
+
+@pytest.mark.parametrize("name", list(CLUSTERS))
+def test_power_iteration_whose_wait_runs_out(name):
+    lp = CLUSTERS[name]()
+    gives_up(lambda: pdhg.Solver.from_lp(lp, wait_test=True, wait_limit_ms=5))
+
+
+def one_cta_lp(m=20, n=400, per_col=2):
+    """Solved by one CTA, which has no exchanges; with every column active its
+    conjugate gradients have enough work for two.  All data positive and c = 0:
+    every entry of x moves off zero and none has a z."""
+    rng = np.random.default_rng(7)
+    rows = np.concatenate([rng.choice(m, size=per_col, replace=False) for _ in range(n)])
+    A = sp.csr_matrix((rng.uniform(0.5, 1.5, n * per_col), (rows, np.repeat(np.arange(n), per_col))), shape=(m, n))
+    A.sort_indices()
+    return lpgen.LP(m, n, A.indptr.astype(np.int32), A.indices.astype(np.int32), A.data, A @ np.ones(n), np.zeros(n))
+
+
+def test_polish_whose_wait_runs_out():
+    lp = one_cta_lp()
+
+    def call(s):
+        s.solve(0.0, 64)
+        with pytest.raises(pdhg.PDHGError):
+            s.polish()
+
+    gives_up(lambda: pdhg.BatchSolver([lp], wait_test=1, wait_limit_ms=5), call)
+    with pdhg.BatchSolver([lp]) as s:
+        s.solve(0.0, 64)
+        assert s.polish()["active"][0] == lp.n
