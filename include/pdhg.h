@@ -136,10 +136,12 @@ typedef struct pdhg_options {
                               (full tiles) whatever the tuner picked           */
   int32_t wait_limit_ms;   /* bound of one device-side wait (default 1000): a
                               grid barrier of the persistent batched solve,
-                              another CTA's vector in an on-chip solve, or the
-                              bulk copy of a column panel of the
-                              gathered vector; a wait past it ends the solve
-                              with PDHG_TIMEOUT                               */
+                              another CTA's vector or sum of an LP on chip (the
+                              power iteration of create, the solve, the
+                              conjugate gradients of polish and adjoint), or
+                              the bulk copy of a column panel of the gathered
+                              vector; a wait past it ends the call with
+                              PDHG_TIMEOUT                                    */
   int32_t wait_test;       /* 1: every grid barrier waits for one arrival more
                               than the grid has, every column-panel load for 16
                               bytes more than its copies deliver, and every
@@ -173,7 +175,9 @@ void pdhg_default_options(pdhg_options* opt);
  *  opt        NULL for defaults
  * On device: builds A^T (stable by row), scales (Ruiz + Pock-Chambolle),
  * estimates sigma_max(A~) by power iteration, sets omega_0 = ||c~||/||b~||,
- * and starts from x = 0, y = 0.  Invalid CSR -> PDHG_INVALID_ARG.  */
+ * and starts from x = 0, y = 0.  Invalid CSR -> PDHG_INVALID_ARG; a wait of the
+ * power iteration past options.wait_limit_ms -> PDHG_TIMEOUT.  *out is NULL
+ * unless PDHG_OK is returned.  */
 pdhg_status pdhg_create(pdhg_ctx** out, int32_t m, int32_t n, const int32_t* row_ptr,
                         const int32_t* col, const double* val, const double* b,
                         const double* c, const pdhg_options* opt);
@@ -344,7 +348,8 @@ pdhg_status pdhg_get_layout(pdhg_ctx* ctx, int64_t* panels, int64_t* panel_width
  *             increasing within a row, in [0, n_l)
  *  val        float64[sum nnz];  b float64[sum m];  c float64[sum n]
  * Pointers are host or device as for pdhg_create (options.io_on_device).
- * Totals of rows, columns and nonzeros must fit in int32.  */
+ * Totals of rows, columns and nonzeros must fit in int32.  *out is NULL unless
+ * PDHG_OK is returned (errors as for pdhg_create).  */
 pdhg_status pdhg_batch_create(pdhg_ctx** out, int32_t count, const int32_t* m, const int32_t* n,
                               const int32_t* row_ptr, const int32_t* col, const double* val,
                               const double* b, const double* c, const pdhg_options* opt);
@@ -365,7 +370,8 @@ pdhg_status pdhg_batch_set_rhs(pdhg_ctx* ctx, const double* b, const double* c);
  * max_iter.  lp_status (HOST int32[count] or NULL) receives each LP's
  * status; the return value is the largest of them (PDHG_CONVERGED only if
  * all converged).  With options.persistent = 1 the solve is one cooperative
- * launch; if one of its grid barriers waits past options.wait_limit_ms every
+ * launch.  If one of its grid barriers, or with LPs on chip a wait between CTAs,
+ * waits past options.wait_limit_ms, every
  * block returns and the call returns PDHG_TIMEOUT (every lp_status too): the
  * iterates are then not meaningful, the context stays usable (destroy it, or
  * restore a state before solving again).  */
@@ -395,7 +401,10 @@ pdhg_status pdhg_batch_warmstart_point(pdhg_ctx* ctx, double mu_min, double delt
  * iterate, stopping at relative residual cg_tol or cg_max_iter steps).
  *  x            float64[sum n] polished x in the original models (or NULL)
  *  lp_active    HOST int32[count]: |B| per LP (or NULL)
- *  lp_cg_iters  HOST int32[count]: CG steps per LP (or NULL)  */
+ *  lp_cg_iters  HOST int32[count]: CG steps per LP (or NULL)
+ * A wait between CTAs past options.wait_limit_ms -> PDHG_TIMEOUT, here and in
+ * pdhg_batch_adjoint: no result is written (lp_active aside), and the call may be
+ * made again.  */
 pdhg_status pdhg_batch_polish(pdhg_ctx* ctx, double cg_tol, int32_t cg_max_iter, double* x,
                               int32_t* lp_active, int32_t* lp_cg_iters);
 

@@ -445,7 +445,7 @@ extern "C" pdhg_status pdhg_batch_polish(pdhg_ctx* ctx, double cg_tol, int32_t c
   std::vector<int32_t> iters;
   if (d->chip) CKS(resident_cg_layout(ctx, d->chip, d->mask, act.data()));
   if (resident_cg_ready(d->chip))
-    CKS(resident_cg(ctx, d->chip, false, d->rhs, d->w, cg_tol, cg_max_iter, &iters));
+    CKT(resident_cg(ctx, d->chip, false, d->rhs, d->w, cg_tol, cg_max_iter, &iters));
   else
     CKS(run_cg(ctx, d, cg_tol, cg_max_iter, &iters, ctx->a_val64, ctx->t_val64));
   if (lp_cg_iters)
@@ -487,7 +487,7 @@ extern "C" pdhg_status pdhg_batch_adjoint(pdhg_ctx* ctx, const double* grad_x, d
   ctx->launches += 2;
   std::vector<int32_t> iters;
   if (resident_cg_ready(d->chip))
-    CKS(resident_cg(ctx, d->chip, true, d->rhs, d->w, cg_tol, cg_max_iter, &iters));
+    CKT(resident_cg(ctx, d->chip, true, d->rhs, d->w, cg_tol, cg_max_iter, &iters));
   else
     CKS(run_cg(ctx, d, cg_tol, cg_max_iter, &iters, ctx->a_val_orig, ctx->t_val_orig));
   if (lp_cg_iters)

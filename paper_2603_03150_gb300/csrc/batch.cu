@@ -1311,7 +1311,7 @@ static pdhg_status batch_create_impl(pdhg_ctx* ctx, const int32_t* m, const int3
   stage("on-chip layout");
   // a3 per LP: power iteration
   if (ctx->resident) {
-    CKS(resident_power(ctx));
+    CKT(resident_power(ctx));
   } else {
     double *v = ctx->xs64, *u = ctx->ys64, *w = ctx->out_n2;
     int32_t* ticket = ctx->active + 2;
@@ -1400,7 +1400,7 @@ extern "C" pdhg_status pdhg_batch_create(pdhg_ctx** out, int32_t count, const in
   ctx->mixed = ctx->opt.precision == PDHG_FP32_MIXED;
   ctx->log_cap = 1;
   pdhg_status st = batch_create_impl(ctx, m, n, row_ptr, col, val, b, c);
-  if (st < 0) {
+  if (st != PDHG_OK) {
     const std::string msg = pdhg_last_error();
     pdhg_destroy(ctx);
     set_error("%s", msg.c_str());

@@ -33,6 +33,13 @@ void clear_error();
     if (s_ < 0) return s_;                 \
   } while (0)
 
+// where PDHG_TIMEOUT (positive, as the outcomes of a solve are) ends the call too
+#define CKT(expr)                          \
+  do {                                     \
+    pdhg_status s_ = (expr);               \
+    if (s_ != PDHG_OK) return s_;          \
+  } while (0)
+
 
 namespace pdhg {
 
@@ -260,7 +267,7 @@ pdhg_status batch_persistent_solve(pdhg_ctx* ctx, long long k0, long long max_it
 // ctx->ps and resident_solve runs every LP from its stored state to its end.
 pdhg_status resident_build(pdhg_ctx* ctx);
 void resident_free(pdhg_ctx* ctx);
-pdhg_status resident_power(pdhg_ctx* ctx);
+pdhg_status resident_power(pdhg_ctx* ctx);  // PDHG_TIMEOUT: a wait between CTAs ran out, as below
 template <typename T>
 pdhg_status resident_solve(pdhg_ctx* ctx, const IterBuffers<T>& B);
 // conjugate gradients of the adjoint on chip (resident_cg.cu): the layout of an

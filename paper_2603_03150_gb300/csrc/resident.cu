@@ -562,7 +562,7 @@ pdhg_status resident_power(pdhg_ctx* ctx) {
   CK(cudaStreamSynchronize(ctx->stream));
   if (err) {
     set_error("power iteration: a CTA waited longer than options.wait_limit_ms for another's vector");
-    return PDHG_CUDA_ERROR;
+    return PDHG_TIMEOUT;
   }
   return PDHG_OK;
 }

@@ -392,6 +392,7 @@ pdhg_status resident_cg(pdhg_ctx* ctx, ResCgData* d, bool original, const double
   ResCg A{d->lp,   nullptr, d->a_sl,      d->t_sl,      d->a_col, d->t_col, d->ord_n,
           d->val[o][0], d->val[o][1], d->bcol, rhs, w, d->iters, tol * tol, max_iter,
           (unsigned long long)ctx->opt.wait_limit_ms * 1000000ull, res_tx_extra(ctx), d->flags + 1};
+  CK(cudaMemsetAsync(d->flags + 1, 0, sizeof(int32_t), s));
   CKS(res_groups(ctx, d->groups, d->side, [&](const ResGroup& g, cudaStream_t q) {
     A.list = d->list + g.first;
     cudaLaunchAttribute attr;
@@ -407,7 +408,7 @@ pdhg_status resident_cg(pdhg_ctx* ctx, ResCgData* d, bool original, const double
   CK(cudaStreamSynchronize(s));
   if (err) {
     set_error("conjugate gradients: a CTA waited longer than options.wait_limit_ms for another's vector");
-    return PDHG_CUDA_ERROR;
+    return PDHG_TIMEOUT;
   }
   return PDHG_OK;
 }

@@ -997,7 +997,7 @@ static pdhg_status create_impl(pdhg_ctx* ctx, const int32_t* row_ptr, const int3
 
   // a3: power iteration on A~^T A~ (float64)
   if (ctx->resident) {
-    CKS(resident_power(ctx));
+    CKT(resident_power(ctx));
   } else {
     double *w = ctx->xs64, *u = ctx->ys64;
     launch_pow_init(n, w, ctx->ps, ctx->opt.power_max_iter, ctx->opt.power_rel_tol, ctx->stream);
@@ -1128,7 +1128,7 @@ extern "C" pdhg_status pdhg_create(pdhg_ctx** out, int32_t m, int32_t n, const i
     // an all-zero A is legal only with nnz = 0; checked after row_ptr is read
   }
   st = create_impl(ctx, row_ptr, col, val, b, c);
-  if (st < 0) {
+  if (st != PDHG_OK) {
     const std::string msg = g_last_error;
     pdhg_destroy(ctx);
     g_last_error = msg;

@@ -543,7 +543,7 @@ class BatchSolver(Solver):
         act = np.zeros(self.count, dtype=np.int32)
         it = np.zeros(self.count, dtype=np.int32)
         _check(self._L.pdhg_batch_polish(self._ctx, cg_tol, cg_max_iter, _ptr(x), _ptr(act),
-                                         _ptr(it)))
+                                         _ptr(it)), allow_positive=False)
         return dict(x=x, active=act, cg_iters=it)
 
     def adjoint(self, grad_x, cg_tol: float = 1e-12, cg_max_iter: int = 5000, out=None):
@@ -553,5 +553,5 @@ class BatchSolver(Solver):
         if not self.device_io and not _is_torch(grad_x):
             grad_x = np.ascontiguousarray(grad_x, dtype=np.float64)
         _check(self._L.pdhg_batch_adjoint(self._ctx, _ptr(grad_x), _ptr(gb), _ptr(gc), cg_tol,
-                                          cg_max_iter, _ptr(it)))
+                                          cg_max_iter, _ptr(it)), allow_positive=False)
         return dict(grad_b=gb, grad_c=gc, cg_iters=it)

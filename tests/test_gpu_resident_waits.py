@@ -67,10 +67,11 @@ def test_power_iteration_many_times(name):
 
 
 def gives_up(create, call=None):
-    """create() or call(solver) ends with an error status; the GPU stays usable."""
+    """create() or call(solver) ends with PDHG_TIMEOUT; the GPU stays usable."""
     if call is None:
-        with pytest.raises(pdhg.PDHGError):
+        with pytest.raises(pdhg.PDHGError) as e:
             create()
+        assert e.value.status == pdhg.PDHG_TIMEOUT
     else:
         with create() as s:
             for _ in range(2):
@@ -132,8 +133,9 @@ def test_polish_whose_wait_runs_out():
 
     def call(s):
         s.solve(0.0, 64)
-        with pytest.raises(pdhg.PDHGError):
+        with pytest.raises(pdhg.PDHGError) as e:
             s.polish()
+        assert e.value.status == pdhg.PDHG_TIMEOUT
 
     gives_up(lambda: pdhg.BatchSolver([lp], wait_test=1, wait_limit_ms=5), call)
     with pdhg.BatchSolver([lp]) as s:
