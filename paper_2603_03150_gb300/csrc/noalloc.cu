@@ -5,8 +5,7 @@
 // Some callers cannot call cudaMalloc: an interior-point solver that owns a
 // fixed device memory pool and must not grow it, or a host thread that must
 // not take the device allocator's locks.  For them the scratch this
-// computation needs -- one partial sum of x^T z per block and mu_target --
-// lives in a file-scope __device__ array that every GPU which loads this
+// computation needs -- one partial sum of x^T z per block -- lives in a file-scope __device__ array that every GPU which loads this
 // library holds until the process exits.
 #include <mutex>
 
@@ -23,14 +22,17 @@ namespace {
 constexpr int kNaThreads = 256;
 constexpr int kNaPerBlock = 2048;   // entries of x^T z reduced by one block
 constexpr int kNaMaxBlocks = 4096;  // partial-sum slots
+// Blocks of the second pass, two per SM of a GB300: an entry's quotients bound it
+// (about 24 operations of the float64 pipe, which 16 warps per SM keep busy), and
+// every block adds the partial sums again (300,000 / 1,000,000 / 8,388,608
+// entries: 304 blocks 26.6 / 69.7 / 519 us, 608 26.7 / 71.7 / 521, 1216 28.7 /
+// 76.2 / 522).
+constexpr int kNaApplyBlocks = 304;
 constexpr long long kNaMaxN = (long long)kNaPerBlock * kNaMaxBlocks;  // 8,388,608
 
-// [0, kNaMaxBlocks): per-block partial sums of x^T z; [kNaMaxBlocks]: mu_target.
-// Every call writes each slot it reads before reading it, so nothing has to
+// Per-block partial sums of x^T z.  Every call writes each slot it reads before reading it, so nothing has to
 // be cleared between calls.  32 KB per device.
-static __device__ __align__(256) double g_na_scratch[kNaMaxBlocks + 2];
-// blocks of a call's reduction that have finished; the last one sets it back
-static __device__ int g_na_ticket;
+static __device__ __align__(256) double g_na_scratch[kNaMaxBlocks];
 
 // sum of x z over [base, end) by one block, in thread 0
 __device__ __forceinline__ double na_block_sum(int base, int end, const double* __restrict__ x,
@@ -48,7 +50,7 @@ __device__ __forceinline__ double na_block_sum(int base, int end, const double* 
 // call at any of these sizes and one block of 256 threads 10.4 / 14.6 / 24.3 at
 // 500 / 1000 / 2000 entries (an entry's quotients keep an SM's float64 pipe for
 // 18 clocks); the cluster takes 8.3 up to 2048 entries and 10.4 up to 4096, the two
-// launches above 12.5.
+// launches above 10.3 at 4097.
 constexpr int kNaCluster = 8, kNaSmall = 4096;
 __global__ void __cluster_dims__(kNaCluster, 1, 1) __launch_bounds__(kNaThreads)
     k_na_small(int n, const double* __restrict__ x, const double* __restrict__ z, double mu_min,
@@ -90,37 +92,43 @@ __global__ void __cluster_dims__(kNaCluster, 1, 1) __launch_bounds__(kNaThreads)
 }
 static_assert(kNaSmall == 2 * kNaCluster * kNaThreads, "an entry or two per thread");
 
-// partial sums of x^T z; the block that finishes last adds them in a fixed
-// order and writes mu (one thread adding them took 68 clocks for each)
+// partial sums of x^T z
 __global__ void __launch_bounds__(kNaThreads)
-    k_na_partial(int n, const double* __restrict__ x, const double* __restrict__ z, double mu_min,
-                 double* scratch, double* mu_out) {
-  __shared__ double red[kNaThreads / 32], tot[1];
-  __shared__ int is_last;
+    k_na_partial(int n, const double* __restrict__ x, const double* __restrict__ z, double* scratch) {
+  __shared__ double red[kNaThreads / 32];
   const int base = blockIdx.x * kNaPerBlock;
   const double s = na_block_sum(base, min(n, base + kNaPerBlock), x, z, red);
-  if (threadIdx.x == 0) {
-    scratch[blockIdx.x] = s;
-    __threadfence();
-    is_last = atomicAdd(&g_na_ticket, 1) == (int)gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  pdhg::parts_sum<kNaThreads, 1>(scratch, (int)gridDim.x, nullptr, 0, tot, red);
-  if (threadIdx.x == 0) {
-    const double mu = fmax(tot[0] / (double)n, mu_min);
-    scratch[kNaMaxBlocks] = mu;
-    if (mu_out) *mu_out = mu;
-    g_na_ticket = 0;
-  }
+  if (threadIdx.x == 0) scratch[blockIdx.x] = s;
 }
 
-// Algorithm 1's per-entry update (Section 3.1)
-__global__ void k_na_apply(int n, const double* __restrict__ x, const double* __restrict__ z,
-                           const double* scratch, double delta, double alpha,
-                           double* __restrict__ x_out, double* __restrict__ z_out) {
-  const double mu = scratch[kNaMaxBlocks];
+// mu, which the first warp of every block adds from the partial sums (one order
+// in all of them), and Algorithm 1's per-entry update (Section 3.1).  Nothing of a
+// call outlives it: a count of finished blocks, which would let the last one of
+// k_na_partial add the sums, would be wrong for good after two calls that overlap
+// (and took longer: 4097 / 50,000 / 300,000 entries 12.3 / 14.4 / 27.7 us against
+// 10.3 / 12.3 / 26.6).
+__global__ void __launch_bounds__(kNaThreads)
+    k_na_apply(int n, const double* __restrict__ x, const double* __restrict__ z,
+               const double* scratch, int nparts, double mu_min, double delta, double alpha,
+               double* mu_out, double* __restrict__ x_out, double* __restrict__ z_out) {
+  __shared__ double mu_s;
+  if (threadIdx.x < 32) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int p = threadIdx.x; p < nparts; p += 128)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (p + 32 * e < nparts) s[e] += __ldcg(scratch + p + 32 * e);
+    double t = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    t = fmax(t / (double)n, mu_min);
+    if (threadIdx.x == 0) {
+      mu_s = t;
+      if (mu_out && blockIdx.x == 0) *mu_out = t;
+    }
+  }
+  __syncthreads();
+  const double mu = mu_s;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
     double xp = x[j], zp = z[j];
     pdhg::centered_pair(mu, delta, alpha, xp, zp);
@@ -184,10 +192,11 @@ extern "C" pdhg_status pdhg_centered_point_noalloc(int32_t n, const double* x, c
     k_na_small<<<kNaCluster, kNaThreads, 0, s>>>(n, x, z, mu_min, delta_max, alpha_min, mu_target, x_out,
                                                  z_out);
   } else {
-    k_na_partial<<<nblocks, kNaThreads, 0, s>>>(n, x, z, mu_min, scratch, mu_target);
-    int grid = (n + 255) / 256;
-    if (grid > 4096) grid = 4096;
-    k_na_apply<<<grid, 256, 0, s>>>(n, x, z, scratch, delta_max, alpha_min, x_out, z_out);
+    k_na_partial<<<nblocks, kNaThreads, 0, s>>>(n, x, z, scratch);
+    int grid = (n + kNaThreads - 1) / kNaThreads;
+    if (grid > kNaApplyBlocks) grid = kNaApplyBlocks;
+    k_na_apply<<<grid, kNaThreads, 0, s>>>(n, x, z, scratch, nblocks, mu_min, delta_max, alpha_min, mu_target,
+                                           x_out, z_out);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) {
