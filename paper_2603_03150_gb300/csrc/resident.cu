@@ -130,44 +130,47 @@ static __global__ void __launch_bounds__(256) k_res_sort(ResBuild B) {
   }
 }
 
-static __global__ void __launch_bounds__(256) k_res_fill(ResFill F) {
-  const int l = blockIdx.y >> 1, side = blockIdx.y & 1, lane = threadIdx.x & 31;
-  const ResLp lp = F.lp[l];
-  const int64_t off = side ? lp.n_off : lp.m_off, coff = side ? lp.m_off : lp.n_off;
-  const int32_t* rp = (side ? F.t_rp : F.a_rp) + off;
-  const int32_t* col = side ? F.t_col : F.a_col;
-  const double* val = side ? F.t_val : F.a_val;
-  const int32_t* src = side ? F.t_src : F.a_src;
-  const uint16_t* ord = (side ? F.ord_n : F.ord_m) + off;
-  const uint16_t* pos = (side ? F.pos_m : F.pos_n) + coff;
-  const ResSlice* sl = (side ? F.t_sl : F.a_sl) + off;
-  const int64_t el = side ? lp.t_el : lp.a_el;
-  uint16_t* oc = side ? F.t_c : F.a_c;
-  double* ov = side ? F.t_v : F.a_v;
-  float* of = side ? F.t_f : F.a_f;
-  const uint16_t dummy = (uint16_t)(side ? lp.m : lp.n);
-  const int S = side ? lp.t_slices : lp.a_slices;
-  for (int s = blockIdx.x * 8 + (threadIdx.x >> 5); s < S; s += gridDim.x * 8) {
-    const ResSlice d = sl[s];
-    const int lg = res_lg(d.wgr), G = 1 << lg, row = lane >> lg, gl = lane & (G - 1);
-    int b = 0, len = 0;
-    if (row < res_rows(d.wgr)) {
-      const int i = ord[d.p0 + row];
-      b = rp[i];
-      len = rp[i + 1] - b;
-    }
-    for (int k = 0; k < res_steps(d.wgr); ++k) {
-      const int j = k * G + gl;
-      uint16_t c = dummy;
-      double v = 0.0;
-      if (j < len) {
-        v = val[src ? src[b + j] : b + j];
-        if (oc) c = pos[col[b + j] - coff];
+static __global__ void __launch_bounds__(256) k_res_fill(ResFill F, int count) {
+  const int lane = threadIdx.x & 31;
+  for (int q = blockIdx.y; q < 2 * count; q += gridDim.y) {  // (a grid has at most 65535 in y)
+    const int l = q >> 1, side = q & 1;
+    const ResLp lp = F.lp[l];
+    const int64_t off = side ? lp.n_off : lp.m_off, coff = side ? lp.m_off : lp.n_off;
+    const int32_t* rp = (side ? F.t_rp : F.a_rp) + off;
+    const int32_t* col = side ? F.t_col : F.a_col;
+    const double* val = side ? F.t_val : F.a_val;
+    const int32_t* src = side ? F.t_src : F.a_src;
+    const uint16_t* ord = (side ? F.ord_n : F.ord_m) + off;
+    const uint16_t* pos = (side ? F.pos_m : F.pos_n) + coff;
+    const ResSlice* sl = (side ? F.t_sl : F.a_sl) + off;
+    const int64_t el = side ? lp.t_el : lp.a_el;
+    uint16_t* oc = side ? F.t_c : F.a_c;
+    double* ov = side ? F.t_v : F.a_v;
+    float* of = side ? F.t_f : F.a_f;
+    const uint16_t dummy = (uint16_t)(side ? lp.m : lp.n);
+    const int S = side ? lp.t_slices : lp.a_slices;
+    for (int s = blockIdx.x * 8 + (threadIdx.x >> 5); s < S; s += gridDim.x * 8) {
+      const ResSlice d = sl[s];
+      const int lg = res_lg(d.wgr), G = 1 << lg, row = lane >> lg, gl = lane & (G - 1);
+      int b = 0, len = 0;
+      if (row < res_rows(d.wgr)) {
+        const int i = ord[d.p0 + row];
+        b = rp[i];
+        len = rp[i + 1] - b;
       }
-      const int64_t at = el + d.off + k * 32 + lane;
-      if (oc) oc[at] = c;
-      ov[at] = v;
-      if (of) of[at] = (float)v;
+      for (int k = 0; k < res_steps(d.wgr); ++k) {
+        const int j = k * G + gl;
+        uint16_t c = dummy;
+        double v = 0.0;
+        if (j < len) {
+          v = val[src ? src[b + j] : b + j];
+          if (oc) c = pos[col[b + j] - coff];
+        }
+        const int64_t at = el + d.off + k * 32 + lane;
+        if (oc) oc[at] = c;
+        ov[at] = v;
+        if (of) of[at] = (float)v;
+      }
     }
   }
 }
@@ -176,7 +179,7 @@ void launch_res_sort(const ResBuild& B, int count, cudaStream_t s) {
   k_res_sort<<<2 * count, 256, 0, s>>>(B);
 }
 void launch_res_fill(const ResFill& F, int count, int max_slices, cudaStream_t s) {
-  k_res_fill<<<dim3(std::min((max_slices + 7) / 8, 64), 2 * count), 256, 0, s>>>(F);
+  k_res_fill<<<dim3(std::min((max_slices + 7) / 8, 64), std::min(2 * count, 65535)), 256, 0, s>>>(F, count);
 }
 
 // ---------------------------------------------------------------------------

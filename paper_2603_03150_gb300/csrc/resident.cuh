@@ -655,7 +655,7 @@ struct ResBuild {
   int32_t* longest;             // the longest row of any matrix
 };
 
-// values and columns of the slices: a warp per slice, grid (x, 2 LPs);
+// values and columns of the slices: a warp per slice, the matrices in y;
 // entries past a row's end: value 0 and the column of the slot that holds 0
 struct ResFill {
   const ResLp* lp;
