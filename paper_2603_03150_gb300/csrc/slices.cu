@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 }
 
 __global__ void __launch_bounds__(kWarps * 32)
-    k_sl_fill(int nrows, int nwin, int lg1, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
+    k_sl_fill(int nrows, int ncols, int nwin, int lg1, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
               const double* __restrict__ val, const int32_t* __restrict__ slice0,
               const int32_t* __restrict__ elem0, int4* out, int32_t* col_s, double* v64) {
   __shared__ int key[kWarps][kSliceRows];
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kWarps * 32)
     for (int k = 0; k < w; ++k) {
       const int j = k * G + gl;
       const bool in = j < len;
-      col_s[off + k * 32 + lane] = in ? col[b + j] : 0;
+      col_s[off + k * 32 + lane] = in ? col[b + j] : ncols;
       v64[off + k * 32 + lane] = in ? val[b + j] : 0.0;
     }
     off += 32 * w;
@@ -150,7 +150,7 @@ bool slices_pay(const pdhg_ctx* ctx, bool on_a) {
 // copy would take more than a quarter of the memory that is left.
 pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   *d = DevSched{};
-  const int nrows = on_a ? ctx->m : ctx->n;
+  const int nrows = on_a ? ctx->m : ctx->n, ncols = on_a ? ctx->n : ctx->m;
   const int32_t *rp = on_a ? ctx->a_rp : ctx->t_rp, *col = on_a ? ctx->a_col : ctx->t_col;
   const double* val = on_a ? ctx->a_val64 : ctx->t_val64;
   cudaStream_t s = ctx->stream;
@@ -188,7 +188,7 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   CKS(dalloc(ctx, &slices, (size_t)nslices));
   CKS(dalloc(ctx, &scol, (size_t)total));
   CKS(dalloc(ctx, &v64, (size_t)total));
-  k_sl_fill<<<grid, kWarps * 32, 0, s>>>(nrows, nw, lg1, rp, col, val, slice0, elem0, slices, scol, v64);
+  k_sl_fill<<<grid, kWarps * 32, 0, s>>>(nrows, ncols, nw, lg1, rp, col, val, slice0, elem0, slices, scol, v64);
   ctx->launches += 1;
   CK(cudaGetLastError());
   SchedView& V = d->view;

@@ -750,16 +750,18 @@ pdhg_status pdhg::alloc_arrays(pdhg_ctx* ctx) {
   const size_t es = elem(ctx);
   void** vecs_n[] = {&ctx->x, &ctx->x_avg, &ctx->x_last};
   void** vecs_m[] = {&ctx->y, &ctx->y_avg, &ctx->y_last, &ctx->Ax, &ctx->Ax_avg, &ctx->Ax_last};
-  for (void** p : vecs_n) want((char**)p, es * n);
-  for (void** p : vecs_m) want((char**)p, es * m);
+  // (every vector that a product gathers has a 0 behind its last entry: that is
+  // what the slices' padding reads, see spmv_slice.cuh)
+  for (void** p : vecs_n) want((char**)p, es * (n + 1));
+  for (void** p : vecs_m) want((char**)p, es * (m + 1));
   if (ctx->opt.step_rule == 1 && !ctx->batch) {
     want((char**)&ctx->x_avg_prev, es * n);
-    want((char**)&ctx->adapt_xx, es * 2 * (size_t)n);
-    for (void** p : {&ctx->y_prev, &ctx->y_avg_prev, &ctx->Ax_prev, &ctx->Ax_avg_prev})
-      want((char**)p, es * m);
+    want((char**)&ctx->adapt_xx, es * 2 * ((size_t)n + 1));
+    want((char**)&ctx->y_prev, es * (m + 1));
+    for (void** p : {&ctx->y_avg_prev, &ctx->Ax_prev, &ctx->Ax_avg_prev}) want((char**)p, es * m);
   }
-  want(&ctx->xs64, n);
-  want(&ctx->ys64, m);
+  want(&ctx->xs64, (size_t)n + 1);
+  want(&ctx->ys64, (size_t)m + 1);
   want(&ctx->out_n1, n);
   want(&ctx->out_n2, n);
   want(&ctx->out_m1, m);
@@ -775,7 +777,12 @@ pdhg_status pdhg::alloc_arrays(pdhg_ctx* ctx) {
     *q.p = at;
     at += q.bytes;
   }
-  if (ctx->adapt_xx) CK(cudaMemsetAsync(ctx->adapt_xx, 0, es * 2 * (size_t)n, ctx->stream));
+  CK(cudaMemsetAsync(ctx->xs64 + n, 0, sizeof(double), ctx->stream));
+  CK(cudaMemsetAsync(ctx->ys64 + m, 0, sizeof(double), ctx->stream));
+  if (ctx->adapt_xx) {
+    CK(cudaMemsetAsync(ctx->adapt_xx, 0, es * 2 * ((size_t)n + 1), ctx->stream));
+    CK(cudaMemsetAsync((char*)ctx->y_prev + es * m, 0, es, ctx->stream));
+  }
   return PDHG_OK;
 }
 
@@ -925,8 +932,8 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
   CK(cudaGetLastError());
 
   // zero state (also what the autotuner multiplies)
-  for (void** p : vecs_n) CK(cudaMemsetAsync(*p, 0, es * n, ctx->stream));
-  for (void** p : vecs_m) CK(cudaMemsetAsync(*p, 0, es * m, ctx->stream));
+  for (void** p : vecs_n) CK(cudaMemsetAsync(*p, 0, es * (n + 1), ctx->stream));
+  for (void** p : vecs_m) CK(cudaMemsetAsync(*p, 0, es * (m + 1), ctx->stream));
 
   return PDHG_OK;
 }

@@ -6,7 +6,9 @@
 // in row order); rows of up to kSliceShort nonzeros go 32 to a slice (a lane
 // each; 2 or 4 on small matrices), those of up to kSliceMid 4 to a slice (8 lanes
 // each), longer ones one to a slice.  Step k of a slice is 32 consecutive values
-// and columns.  A warp takes a slice: a row costs one multiply-add per nonzero
+// and columns; past a row's end the value is 0 and the column the one behind the
+// last, where every gathered vector holds a 0 (a column that the row does not hold
+// could hold an infinity or a NaN, which a value of 0 would carry into the sum).  A warp takes a slice: a row costs one multiply-add per nonzero
 // (and the additions of a shuffle sum in the longer classes) where run_tiles adds
 // a segmented scan of 5 additions for 8 nonzeros, and there is no block barrier
 // and no staging: the lane that holds a row's sum runs its epilogue, whose

@@ -105,3 +105,35 @@ def test_float32_half_steps_keep_the_order_of_the_tiles():
             out.append(s.state())
     for k in ("x", "y", "x_avg", "y_avg"):
         np.testing.assert_array_equal(out[0][k], out[1][k], err_msg=k)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("method", ["averaged", "halpern", "adaptive"])
+@pytest.mark.parametrize("name", ["lanes_4", "lanes_1", "planted"])
+def test_a_non_finite_entry_reaches_its_own_rows_only(name, method, bad):
+    """Entry 0 of y (then of x) infinite or NaN: the products, the next iterate
+    and the returned solution are non-finite where the tile kernels' are, and
+    the rest agrees to 1e-9 as above."""
+    lp = MAKERS[name]()
+    kw = {"step_rule": "adaptive"} if method == "adaptive" else {"method": method}
+    with pdhg.Solver.from_lp(lp, **kw) as s, pdhg.Solver.from_lp(lp, tile_nnz=2044, **kw) as t:
+        assert s.schedule()["a_variant"] == s.schedule()["at_variant"] == SLICED
+        s.solve(0.0, 8)
+        good = s.state()
+        for field in ("y", "x"):
+            out = []
+            for q in (s, t):
+                st = {k: np.array(v) if isinstance(v, np.ndarray) else v for k, v in good.items()}
+                st[field][0] = bad
+                st = {k: v for k, v in st.items() if not k.startswith("Ax")}  # products from the state
+                q.set_state(st)
+                before = {k: v for k, v in q.state().items() if k.startswith("Ax")}
+                g = q.get()
+                q.solve(0.0, 9)
+                out.append({**before, **{"get_" + k: g[k] for k in "xyz"}, **{k: q.state()[k] for k in ("x", "y")}})
+            for k in out[0]:
+                a, b = out[0][k], out[1][k]
+                fin = np.isfinite(b)
+                np.testing.assert_array_equal(np.isfinite(a), fin, err_msg=f"{field} {k}")
+                assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(a[~fin] > 0, b[~fin] > 0), k
+                assert fin.mean() > 0.5 and rel_inf(a[fin], b[fin]) < 1e-9, (field, k)
