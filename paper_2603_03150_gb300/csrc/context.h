@@ -204,6 +204,26 @@ struct StageClock {
   }
 };
 
+// make(), which builds a layout that the context can do without: where it does not
+// find room for it (PDHG_OOM), what it has allocated is given back and drop() is
+// to leave the context as it was.
+template <class F, class G>
+pdhg_status if_room(pdhg_ctx* ctx, F&& make, G&& drop) {
+  const size_t kept = ctx->allocs.size(), left = ctx->slab_left;
+  char* const slab = ctx->slab;
+  const pdhg_status st = make();
+  if (st != PDHG_OOM) return st;
+  cudaGetLastError();
+  CK(cudaStreamSynchronize(ctx->stream));
+  for (size_t i = kept; i < ctx->allocs.size(); ++i) cudaFree(ctx->allocs[i]);
+  ctx->allocs.resize(kept);
+  ctx->slab = slab;
+  ctx->slab_left = left;
+  pdhg::set_error("%s", "");
+  drop();
+  return PDHG_OK;
+}
+
 // Device memory freed with the context.  Arrays of up to 128 KB share blocks of
 // 1 MB: a small LP's set-up made some 80 allocations of its own and its release
 // as many: creating and closing an LP of 200 x 500 1.59 -> 1.37 ms.

@@ -407,9 +407,9 @@ std::vector<int32_t> res_order(const std::vector<ResLp>& lps, const std::vector<
 }
 
 // Chooses the cluster size of every LP and builds the layout; leaves
-// ctx->resident NULL where the LPs do not fit on chip or options ask for the
-// tile kernels' own paths.
-pdhg_status resident_build(pdhg_ctx* ctx) {
+// ctx->resident NULL where the LPs do not fit on chip, options ask for the tile
+// kernels' own paths or there is no memory for it.
+static pdhg_status res_build(pdhg_ctx* ctx) {
   const pdhg_options& o = ctx->opt;
   // A float32-mixed solve of one LP keeps the tile kernels' order of addition:
   // its float64 solution is that of float32 iterates, which differ by 1e-6
@@ -545,6 +545,10 @@ pdhg_status resident_build(pdhg_ctx* ctx) {
   CK(d->side.make((int)d->groups.size()));
   CK(cudaStreamSynchronize(ctx->stream));  // the host vectors go out of scope
   return PDHG_OK;
+}
+
+pdhg_status resident_build(pdhg_ctx* ctx) {
+  return if_room(ctx, [&] { return res_build(ctx); }, [&] { resident_free(ctx); });
 }
 
 pdhg_status resident_power(pdhg_ctx* ctx) {

@@ -259,8 +259,9 @@ void resident_cg_free(ResCgData* d) {
 }
 bool resident_cg_ready(const ResCgData* d) { return d && d->ready; }
 
-// B = the columns with mask != 0, active[l] of them in LP l
-pdhg_status resident_cg_layout(pdhg_ctx* ctx, ResCgData* d, const double* mask, const int32_t* active) {
+// B = the columns with mask != 0, active[l] of them in LP l; not ready where the
+// LPs are not solved on chip or there is no memory for the layout
+static pdhg_status cg_layout(pdhg_ctx* ctx, ResCgData* d, const double* mask, const int32_t* active) {
   d->ready = d->original = false;
   if (!ctx->resident) return PDHG_OK;
   const int count = ctx->count, m = ctx->m, n = ctx->n;
@@ -370,6 +371,15 @@ pdhg_status resident_cg_layout(pdhg_ctx* ctx, ResCgData* d, const double* mask, 
   CK(cudaStreamSynchronize(s));
   d->ready = true;
   return PDHG_OK;
+}
+
+pdhg_status resident_cg_layout(pdhg_ctx* ctx, ResCgData* d, const double* mask, const int32_t* active) {
+  const bool had = d->lp != nullptr;  // (the arrays are kept between layouts)
+  return if_room(ctx, [&] { return cg_layout(ctx, d, mask, active); },
+                 [&] {
+                   d->ready = false;
+                   if (!had) d->lp = nullptr;
+                 });
 }
 
 // w (start in, solution out) of M_B^T M_B w = rhs per LP, M the scaled matrix

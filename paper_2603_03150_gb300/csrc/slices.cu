@@ -148,7 +148,7 @@ bool slices_pay(const pdhg_ctx* ctx, bool on_a) {
 // d->view.e stays 0, and the matrix is left to the tiles, where rows of very
 // different lengths share windows (more padding than nonzeros) or where the
 // copy would take more than a quarter of the memory that is left.
-pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
+static pdhg_status make_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   *d = DevSched{};
   const int nrows = on_a ? ctx->m : ctx->n, ncols = on_a ? ctx->n : ctx->m;
   const int32_t *rp = on_a ? ctx->a_rp : ctx->t_rp, *col = on_a ? ctx->a_col : ctx->t_col;
@@ -202,6 +202,10 @@ pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
   V.slice_col = scol;
   V.slice_val = v64;
   return PDHG_OK;
+}
+
+pdhg_status build_slices(pdhg_ctx* ctx, bool on_a, DevSched* d) {
+  return if_room(ctx, [&] { return make_slices(ctx, on_a, d); }, [&] { *d = DevSched{}; });
 }
 
 }  // namespace pdhg
