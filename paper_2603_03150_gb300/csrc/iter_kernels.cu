@@ -528,10 +528,10 @@ PDHG_INST(double)
 #undef PDHG_INST
 
 // shared memory of the tile kernels (NV vectors, precision, rows per tile,
-// schedule variant: e < 0 is the vector kernel, which stages its sums as the
-// slices do)
+// schedule variant: e < 0 is the vector kernel; the slices use none)
 size_t tile_smem(int nv, bool f32, int max_rows, int e) {
-  if (e < 0 || e == kSliced) {
+  if (e == kSliced) return 0;
+  if (e < 0) {
     if (nv == 1)
       return f32 ? tile_vec_smem_bytes<float, 1, kBlock>(max_rows)
                  : tile_vec_smem_bytes<double, 1, kBlock>(max_rows);

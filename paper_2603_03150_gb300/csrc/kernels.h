@@ -138,6 +138,7 @@ struct RowStatPlan {
   int long_len = 1 << 30;
   const int32_t* long_ids = nullptr;
   int nlong = 0;
+  int nsm = 1;
 };
 // One Ruiz / Pock-Chambolle round for the rows of D_self M D_other: d_new =
 // d_self / statistic, mode 0: sqrt(max |.|), mode 1: sqrt(sum |.|); zero -> 1.

@@ -335,7 +335,7 @@ void launch_row_stat(int nrows, const int32_t* rp, const int32_t* col, const dou
   // has 32 warps, fewer rows a warp on smaller matrices (200 rows: 5.6 us in
   // one pass against 19 in 16)
   const int rpw = 32 / plan.lanes;
-  const int passes = std::max(1, std::min(plan.lanes, nrows / (rpw * 152 * 32)));
+  const int passes = std::max(1, std::min(plan.lanes, nrows / (rpw * plan.nsm * 32)));
   const int g = plan.nlong + grid_cap((int64_t)nrows * 32 / (passes * rpw));
 #define PDHG_ROW_STAT(G)                                                                              \
   if (mode)                                                                                           \

@@ -882,6 +882,7 @@ pdhg_status pdhg::prepare_matrix(pdhg_ctx* ctx) {
       const double mean = nrows > 0 ? (double)rp[nrows] / nrows : 0.0;
       pl->lanes = mean <= 6 ? 4 : mean <= 12 ? 8 : mean <= 24 ? 16 : 32;
       pl->long_len = kLongRow;
+      pl->nsm = ctx->nsm;
       int32_t most = 0;
       const int32_t* r = rp.data();
       for (int i = 0; i < nrows; ++i) most = std::max(most, r[i + 1] - r[i]);
