@@ -166,6 +166,13 @@ typedef struct pdhg_options {
 void pdhg_default_options(pdhg_options* opt);
 
 /* Create a solver context for one LP (Section 2 standard form).
+ * An LP of up to 320,000 nonzeros whose vectors fit in the shared memory of a
+ * cluster is solved on chip (one launch for many iterations) in float64 with the
+ * constant step and tile_nnz, spmv_layout, panel_width and kernel_timing 0; a
+ * batch (pdhg_batch_create) in either precision, if all of its LPs are such.  A
+ * float32-mixed LP by itself is not, so that its iterates keep the order of
+ * addition of the tile kernels: at that size float64, or a batch of one, is
+ * several times faster per iteration (200 x 500: 2.2 us, 1.5 us, against 10).
  *  m, n       rows and columns of A (m >= 1, n >= 1)
  *  row_ptr    int32[m+1], row_ptr[0] = 0, non-decreasing, nnz = row_ptr[m]
  *             <= 2^31 - 2^16 (int32 tile indexing)
@@ -313,7 +320,7 @@ pdhg_status pdhg_get_kernel_timing_parts(pdhg_ctx* ctx, double* ms, int64_t* sam
  * move and applies the acceptance test.  Launches are back to back as in a solve
  * (programmatic dependent launch), with no event between them.  A context
  * whose LP is solved on chip (float64, constant step, tile_nnz = 0, spmv_layout = 0,
- * kernel_timing = 0, vectors that fit in a cluster's shared memory) has no
+ * panel_width = 0, kernel_timing = 0, vectors that fit in a cluster's shared memory) has no
  * half-step kernels of its own: the tile kernels are timed.  The solver
  * state is saved to a temporary device buffer first and restored after, so
  * a solve continues as if the call had not happened.  Single-LP contexts.  */

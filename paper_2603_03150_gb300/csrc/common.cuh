@@ -294,8 +294,11 @@ __device__ __forceinline__ double min_pos(double v, double w) {
   return is_nan_bits(b) || (a < b && !is_nan_bits(a)) ? v : w;
 }
 
-// x / d from inv = 1 / d: the product corrected by its residual (3 float64
-// operations; a division takes about 10)
+// x / d from inv, 1 / d correctly rounded: the product corrected by its residual (3
+// float64 operations; a division takes about 10).  The result is the correctly
+// rounded quotient where nothing underflows: none of 620 million pairs differed
+// from x / d (random ones and mantissas near the ends), nor any pair of mantissas
+// of 6 to 13 bits in arithmetic of that precision.
 __device__ __forceinline__ double div_by(double x, double d, double inv) {
   const double q = x * inv;
   const bool finite = ((unsigned long long)__double_as_longlong(q) << 1) < 0xffe0000000000000ull;
@@ -545,9 +548,8 @@ __device__ __forceinline__ double halpern_weight(long long n, double) {
 // A step's two scalars for a whole block.  A float64 division by every thread
 // (about 12 operations of 16 clocks per warp on GB300's float64 pipe) is work of
 // the pipe that bounds the float64 kernels: one warp divides and shares the
-// quotient (power-law LP, 64 iterations 6.54 -> 6.38 ms, with max0 above), and
-// float weights are divided in float (transportation LP, 64 Halpern iterations
-// 4.92 -> 4.89 ms).  Ends with a block barrier in float64.
+// quotient (power-law LP, 64 iterations 6.54 -> 6.38 ms, with max0 above).  Float
+// weights are divided in float (no difference measured).  Ends with a block barrier in float64.
 template <typename T>
 struct StepScalars {
   T step, w;

@@ -89,9 +89,9 @@ struct ResCg {
 
 // Bound by the float64 pipe with an SM per LP or more LPs than SMs, else by the
 // latency of a pass over a slice, two exchanges of a vector and two sums per
-// step.  64 LPs of 2000 x 5000: 8.7 us per step (719 steps of the adjoint in 6.3
+// step.  64 LPs of 2000 x 5000: 8.8 us per step (676 steps of the adjoint in 5.9
 // ms) against 57 us of four launches on the tile kernels; 5 LPs of 333 x 832:
-// 5.5 us against 31.  With every warp taking the sums and quotients itself the
+// 6.0 us against 31.  With every warp taking the sums and quotients itself the
 // same steps took 12.5 and 9 us.
 template <int C>
 __global__ void __launch_bounds__(kResThreads) k_res_cg(ResCg A) {
